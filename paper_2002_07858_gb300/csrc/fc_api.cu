@@ -1033,12 +1033,22 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 // at the true point is loose there; later scans probe at the previous minimum), then the top-k
                 // pass.  Later rounds are seeded by the best binary64 value (round 1: top-k, round 2: list).
                 const bool min_pass = (!seeded && first_heavy);
+                ScreenSplit ss;
+                ss.parts = screen_parts(n_tiles, g->G_pad, c->n_sm, &ss.len);
+                if (ss.parts > 1) {
+                    // a split that has no room for its storage runs unsplit
+                    const size_t rows = (size_t)n_tiles * kBM, cand = listing ? 0 : rows * ss.parts * rtopk;
+                    if ((min_pass && scratch(c, "split_key", rows, &ss.key) != FC_OK) ||
+                        (cand && (scratch(c, "split_val", cand, &ss.val) != FC_OK ||
+                                  scratch(c, "split_idx", cand, &ss.idx) != FC_OK)))
+                        ss.parts = 1;
+                }
                 for (int pass = min_pass ? 0 : 1; pass < 2; ++pass) {
                     const int mode = pass == 0 ? kScreenMin : (listing ? kScreenList : kScreenTopK);
                     if (!launch_screen(g->K, rtopk, mode, g->tune.screen_stages, g->tune.screen_ybuf, Yt, g->Bt, g->Qb3,
                                        tslot, tau0, tj0, n_tiles, g->G, g->G_pad, cval, cidx, ccount, c->status_dev,
                                        g->Qc, g->Qb, g->gnorm, alpha, g->spec(), g->nfit, ListArgs{tuniv, loff, lnum},
-                                       c->wait_test, c->n_sm, c->stream))
+                                       c->wait_test, ss, c->n_sm, c->stream))
                         return fail(FC_ERR_ARG, "no tensor-core screen instance for K = " + std::to_string(g->K));
                     S->screen_launches += 1;
                     S->screen_tiles += n_tiles;

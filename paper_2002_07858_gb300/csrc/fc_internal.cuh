@@ -211,6 +211,17 @@ struct WaitTest {
     uint64_t wait_ns;
     int64_t stop_after;
 };
+// Split of a launch over the grid (few universe tiles, many grid tiles): parts
+// ranges of len grid tiles, and the storage the ranges meet in: val / idx
+// [parts][rows][topk] of a top-k launch, key [rows] of a min pass.  parts = 1:
+// unsplit, no storage.
+struct ScreenSplit {
+    int parts = 1, len = 0;
+    float* val = nullptr;
+    int32_t* idx = nullptr;
+    unsigned long long* key = nullptr;
+};
+int screen_parts(int64_t n_tiles, int64_t G_pad, int n_sm, int* len);
 // stages / ybuf: pipeline depth and A-image buffers, 0 = built-in choice.
 bool screen_config_ok(int K, int stages, int ybuf);
 bool launch_screen(int K, int topk, int mode, int stages, int ybuf, const uint16_t* Ytiles, const uint16_t* Btiles,
@@ -218,7 +229,7 @@ bool launch_screen(int K, int topk, int mode, int stages, int ybuf, const uint16
                    const int32_t* quad_slot, float* tau0, const int32_t* tile_j0, int64_t n_tiles, int64_t G,
                    int64_t G_pad, float* cand_val, int32_t* cand_idx, int32_t* cand_count, int* status,
                    const float* Qc, const float* Qb, const float4* gnorm, const float4* alpha, const GridSpec& gs,
-                   int nfit, const ListArgs& la, const WaitTest& wt, int n_sm, cudaStream_t st);
+                   int nfit, const ListArgs& la, const WaitTest& wt, const ScreenSplit& ss, int n_sm, cudaStream_t st);
 // Resolution of one mixed-path scan per screen tile (see k_resolve).
 struct ResolveArgs {
     const int32_t* quad_slot;  // [n_tiles * kQuads] covariance slot of each 32-row quadrant

@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 #include <float.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "fc_internal.cuh"
@@ -161,6 +162,38 @@ __device__ __forceinline__ void list_chunk(int32_t& n, int32_t cap, float* __res
     }
 }
 
+// The same into a half row that several CTAs append to (a split launch): the
+// entries' positions come from one atomic per chunk that holds any.  The order
+// of a list does not matter: a complete list's first minimum is taken by
+// (value, index).
+__device__ __forceinline__ void list_chunk_shared(int32_t* __restrict__ count, int32_t cap, float* __restrict__ lval,
+                                                  int32_t* __restrict__ lidx, float seed, const uint32_t (&r)[32],
+                                                  float m, int64_t g0, int64_t G) {
+    if (m <= seed) {
+        uint32_t mask = below_mask(r, seed);
+        const int64_t lim = G - g0;
+        if (lim < 32) mask &= (lim <= 0) ? 0u : ((1u << lim) - 1u);
+        if (!mask) return;
+        int32_t n = atomicAdd(count, __popc(mask));
+        while (mask) {
+            const int i = __ffs(mask) - 1;
+            mask &= mask - 1;
+            if (n < cap) {
+                lidx[n] = (int32_t)(g0 + i);
+                lval[n] = m;
+            }
+            ++n;
+        }
+    }
+}
+
+// (value, index) as one unsigned key with the order of the pair
+__device__ __forceinline__ unsigned long long min_key(float v, int32_t g) {
+    const uint32_t b = __float_as_uint(v);
+    const uint32_t o = (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+    return ((unsigned long long)o << 32) | (uint32_t)g;
+}
+
 // First pass: running minimum of a row.  The index is recovered only when the
 // chunk improves the minimum (rare after the first tiles).
 __device__ __forceinline__ void min_chunk(float& bv, int32_t& bi, const uint32_t (&r)[32], float m, int64_t g0,
@@ -206,15 +239,16 @@ __device__ float probe_upper_bound(const uint16_t* __restrict__ Yt, int64_t item
 }
 
 // After a min-only pass: tau0 <- min(tau0, certified upper bound at the row's
-// minimum index bidx), one thread per row (bidx = INT32_MAX: no minimum).
+// minimum index bidx), one thread per row (bidx = INT32_MAX: no minimum); a
+// split launch leaves the index in the low word of bkey instead.
 __global__ void k_min_seed(const uint16_t* __restrict__ Yt, const int32_t* __restrict__ quad_slot,
-                           const int32_t* __restrict__ bidx, float* __restrict__ tau0, int64_t n_rows, int64_t G,
+                           const int32_t* __restrict__ bidx, const unsigned long long* __restrict__ bkey, float* __restrict__ tau0, int64_t n_rows, int64_t G,
                            int64_t G_pad, ProbeArgs pa, const int* __restrict__ status) {
     const int64_t orow = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (orow >= n_rows) return;
     // an aborted min pass leaves rows it never reached unwritten: use nothing of it
     if (*status & kDevTimeout) return;
-    const int32_t bi = bidx[orow];
+    const int32_t bi = bkey ? (int32_t)(uint32_t)bkey[orow] : bidx[orow];
     const float seed = tau0[orow];
     if (bi < 0 || bi >= G || !(seed > -FLT_MAX)) return;
     const int64_t item = orow / kBM;
@@ -269,13 +303,32 @@ inline ScreenLayout screen_layout(int K, int stages, int ybuf, int kchunk) {
     return l;
 }
 
+// Split launches.  A launch with few universe tiles on a large grid would
+// leave most SMs idle (one CTA per tile), so the grid tiles are cut into
+// `parts` ranges of `len` and a work item is (universe tile, range): items are
+// numbered range-major, so the CTAs that run side by side read the same range
+// of the B image and share it through L2.  A range's results meet outside the
+// CTA: top-k lists go to [part][row][TOPK] and are merged by k_topk_merge, the
+// min pass takes an atomic minimum of (value, index) keys, list entries are
+// appended with an atomic.  All three give the very sets an unsplit launch
+// gives (a top-k list is the k smallest (value, index) pairs at or below the
+// seed, whatever the order they come in).  Measured: a screen of 1 to 11 tiles
+// over 16.7 million points took 86 to 99 ms on as many CTAs; the job of 4
+// points x 16 universes there went from 1 227 to 90 ms (64 x 141x141 data
+// sets: 1.31 to 1.15 ms; 4 points of 27^3, N = 200: 64.6 to 61.3 ms).
+struct SplitArgs {
+    int parts;                 // 1: unsplit
+    int len;                   // grid tiles per range
+    unsigned long long* key;   // [rows] min pass of a split launch
+};
+
 template <int TOPK, int MODE, bool KCHUNK>
 __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
     k_screen(const uint16_t* __restrict__ Yt, const uint16_t* __restrict__ Bt, const uint16_t* __restrict__ Qb3,
              const int32_t* __restrict__ quad_slot, float* __restrict__ tau0, const int32_t* __restrict__ tile_j0,
              int64_t n_tiles, int64_t G, int64_t G_pad, float* __restrict__ cand_val, int32_t* __restrict__ cand_idx,
              int32_t* __restrict__ cand_count, int* __restrict__ status, ProbeArgs pa, ScreenLayout lay,
-             ListArgs la, WaitTest wt) {
+             ListArgs la, WaitTest wt, SplitArgs sp) {
     static_assert(2 * TOPK * 32 * 4 <= 4096, "top-k hand-over exceeds the warp scratch");
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + (kSmemAlign - 1)) & ~(uintptr_t)(kSmemAlign - 1));
@@ -341,6 +394,18 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
     tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
     const int n_gt = (int)(G_pad / kBN);
+    const bool split = sp.parts > 1;
+    const int64_t n_items = n_tiles * sp.parts;
+    // work item w: universe tile, and the grid-tile range [lo, hi) with the tile it starts from (the
+    // one holding row 0's covariance index when the range has it: its values are the smallest)
+    auto item_of = [&](int64_t w, int64_t& item, int& lo, int& hi, int& j) {
+        const int part = split ? (int)(w / n_tiles) : 0;
+        item = w - (int64_t)part * n_tiles;
+        lo = part * sp.len;
+        hi = lo + sp.len < n_gt ? lo + sp.len : n_gt;
+        const int j0 = ((tile_j0[item] % n_gt) + n_gt) % n_gt;
+        j = (j0 >= lo && j0 < hi) ? j0 : lo;
+    };
     // limit of the pipeline waits (the drain and completion waits keep the built-in limit)
     const uint64_t wlim = wt.wait_ns ? wt.wait_ns : kWaitNs;
 
@@ -354,7 +419,10 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
         // ring positions and phases advance by counting (no division in the issue loop)
         int yb = 0, s = 0;
         uint32_t yph = 0, ph = 0;
-        for (int64_t item = blockIdx.x; ok && !stopped && item < n_tiles; item += gridDim.x) {
+        for (int64_t w = blockIdx.x; ok && !stopped && w < n_items; w += gridDim.x) {
+            int64_t item;
+            int lo, hi, j;
+            item_of(w, item, lo, hi, j);
             if (!mbar_wait(bar(Y_EMPTY + yb), yph ^ 1, abort_flag, wlim)) { ok = false; break; }
             mbar_expect_tx(bar(Y_FULL + yb), lay.y_bytes);
             bulk_g2s(sbase + yb * lay.y_bytes, Yt + item * (int64_t)(lay.y_bytes / 2), lay.y_bytes,
@@ -364,8 +432,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
             const int32_t* qs = quad_slot + item * kQuads;
             const bool mixed = qs[1] != qs[0] || qs[2] != qs[0] || qs[3] != qs[0];
             const uint16_t* qrow = Qb3 + (int64_t)qs[0] * G_pad * 8;
-            int j = ((tile_j0[item] % n_gt) + n_gt) % n_gt;
-            for (int jj = 0; ok && !stopped && jj < n_gt; ++jj) {
+            for (int jj = lo; ok && !stopped && jj < hi; ++jj) {
                 const uint16_t* btile = Bt + (int64_t)j * tile_elems;
                 if (mixed) {
                     // an extra stage: the q-step slabs of the four quadrants' slots, side by side
@@ -402,7 +469,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                     b_par[s] = (int)ph;
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (++j == n_gt) j = 0;
+                if (++j == hi) j = lo;
             }
         }
         if (!ok) {
@@ -426,13 +493,16 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
         const uint64_t a_s23 = smem_desc(sbase + lay.off_sel + 2 * kAChunk, kAChunk, 128);
         int yb = 0, s = 0, ab = 0;
         uint32_t yph = 0, ph = 0, aph = 0;
-        for (int64_t item = blockIdx.x; ok && item < n_tiles; item += gridDim.x) {
+        for (int64_t w = blockIdx.x; ok && w < n_items; w += gridDim.x) {
+            int64_t item;
+            int lo, hi, j;
+            item_of(w, item, lo, hi, j);
             if (!mbar_wait(bar(Y_FULL + yb), yph, abort_flag, wlim)) { ok = false; break; }
             tc_fence_after();
             const uint32_t a0 = sbase + yb * lay.y_bytes;
             const int32_t* qs = quad_slot + item * kQuads;
             const bool mixed = qs[1] != qs[0] || qs[2] != qs[0] || qs[3] != qs[0];
-            for (int jj = 0; ok && jj < n_gt; ++jj) {
+            for (int jj = lo; ok && jj < hi; ++jj) {
                 if (!mbar_wait(bar(T_EMPTY + ab), aph ^ 1, abort_flag, wlim)) { ok = false; break; }
                 const uint32_t d = tmem_base + (uint32_t)(ab * kBN);
                 if (mixed) {
@@ -503,8 +573,12 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
         float* mval = (float*)(smem + lay.off_scratch + (half ? warp - 2 : warp + 2) * 4096);
         int32_t* midx = (int32_t*)(mval + TOPK * 32);
         bool ok = true;
-        int it = 0;
-        for (int64_t item = blockIdx.x; item < n_tiles; item += gridDim.x, ++it) {
+        int ab = 0;
+        uint32_t aph = 0;
+        for (int64_t w = blockIdx.x; w < n_items; w += gridDim.x) {
+            int64_t item;
+            int lo, hi, j;
+            item_of(w, item, lo, hi, j);
             // seeded with the row's certified upper bound: larger values can never be the minimum
             const float seed = tau0[item * kBM + row];
             float vals[TOPK];
@@ -527,11 +601,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                 lbase = (u >= 0) ? la.off[u] + (half ? nn.x : 0) : 0;
                 lcap = half ? nn.y : nn.x;
             }
-            int j = ((tile_j0[item] % n_gt) + n_gt) % n_gt;
-            for (int jj = 0; ok && jj < n_gt; ++jj, j = (j + 1 == n_gt) ? 0 : j + 1) {
-                const int64_t seq = (int64_t)it * n_gt + jj;
-                const int ab = (int)(seq & 1);
-                const uint32_t aph = (uint32_t)((seq >> 1) & 1);
+            for (int jj = lo; ok && jj < hi; ++jj, j = (j + 1 == hi) ? lo : j + 1) {
                 bool w_ok = mbar_wait(bar(T_FULL + ab), aph, abort_flag, wlim);
                 if (!__all_sync(0xffffffffu, w_ok)) {
                     ok = false;
@@ -545,6 +615,9 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                 auto chunk = [&](const uint32_t(&r)[32], float m, int64_t gc) {
                     if (MODE == kModeMin)
                         min_chunk(bv, bi, r, m, gc, G);
+                    else if (MODE == kModeList && split)
+                        list_chunk_shared(cand_count + (item * kBM + row) * 2 + half, lcap, cand_val + lbase,
+                                          cand_idx + lbase, seed, r, m, gc, G);
                     else if (MODE == kModeList)
                         list_chunk(nlist, lcap, cand_val + lbase, cand_idx + lbase, seed, r, m, gc, G);
                     else
@@ -563,6 +636,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(T_EMPTY + ab));
+                if (++ab == 2) { ab = 0; aph ^= 1u; }
                 // the four chunk minima first (independent trees), then the rare slow paths
                 const float m0 = min32(r0), m1 = min32(r1), m2 = min32(r2), m3 = min32(r3);
                 // top-k: a chunk acts only at or below the row's k-th value, so a warp none of whose
@@ -580,7 +654,10 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                 __syncwarp();
             }
             if (MODE == kModeList) {
-                cand_count[(item * kBM + row) * 2 + half] = ok ? nlist : -1;
+                if (!split)
+                    cand_count[(item * kBM + row) * 2 + half] = ok ? nlist : -1;
+                else if (!ok)  // negative whatever is still added
+                    atomicMin(cand_count + (item * kBM + row) * 2 + half, INT32_MIN);
                 if (!ok) break;
                 continue;
             }
@@ -603,7 +680,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
             named_bar(1 + quad, 64);
             const bool pair_done = pair_ok[quad * 2] && pair_ok[quad * 2 + 1];
             if (half == 0) {
-                const int64_t orow = item * kBM + row;
+                const int64_t orow = (MODE == kModeTopK ? w : item) * kBM + row;  // [part][row] when split
                 if (MODE == kModeMin) {
                     const float x = mval[lane];
                     const int32_t xi = midx[lane];
@@ -613,7 +690,10 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
                     }
                     // the row's minimum index; k_min_seed turns it into the certified seed after the
                     // launch, so the epilogue never stalls the MMAs on the probe's scattered loads
-                    cand_idx[orow] = (pair_done && seed > -FLT_MAX) ? bi : INT32_MAX;
+                    if (!split)
+                        cand_idx[orow] = (pair_done && seed > -FLT_MAX) ? bi : INT32_MAX;
+                    else if (pair_done && seed > -FLT_MAX)
+                        atomicMin(sp.key + orow, min_key(bv, bi));
                 } else {
 #pragma unroll 1
                     for (int t = 0; t < TOPK; ++t) {
@@ -646,23 +726,98 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
     }
 }
 
+// Merge of a split launch's top-k lists, one warp per row: the k smallest
+// (value, index) pairs of the parts' sorted lists.  Each lane folds the lists
+// of every 32nd part into one in registers; then k pops of the warp's smallest
+// head.
+template <int TOPK>
+__global__ void __launch_bounds__(128) k_topk_merge(const float* __restrict__ pv, const int32_t* __restrict__ pi,
+                                                    int parts, int64_t rows, float* __restrict__ cand_val,
+                                                    int32_t* __restrict__ cand_idx) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (row >= rows) return;
+    float vals[TOPK];
+    int32_t idx[TOPK];
+#pragma unroll
+    for (int t = 0; t < TOPK; ++t) {
+        vals[t] = FLT_MAX;
+        idx[t] = INT32_MAX;
+    }
+    for (int p = lane; p < parts; p += 32) {
+        const int64_t o = ((int64_t)p * rows + row) * TOPK;
+        for (int t = 0; t < TOPK; ++t) {
+            const float x = pv[o + t];
+            const int32_t g = pi[o + t];
+            const int32_t gi = g < 0 ? INT32_MAX : g;  // an empty entry holds the seed
+            if (!(x < vals[TOPK - 1] || (x == vals[TOPK - 1] && gi < idx[TOPK - 1]))) break;
+            topk_insert<TOPK>(vals, idx, x, gi);
+        }
+    }
+    for (int t = 0; t < TOPK; ++t) {
+        float v = vals[0];
+        int32_t g = idx[0];
+        int who = lane;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+            const int32_t og = __shfl_xor_sync(0xffffffffu, g, o);
+            const int ow = __shfl_xor_sync(0xffffffffu, who, o);
+            if (ov < v || (ov == v && (og < g || (og == g && ow < who)))) {
+                v = ov;
+                g = og;
+                who = ow;
+            }
+        }
+        if (who == lane) {
+#pragma unroll
+            for (int k = 0; k + 1 < TOPK; ++k) {
+                vals[k] = vals[k + 1];
+                idx[k] = idx[k + 1];
+            }
+            vals[TOPK - 1] = FLT_MAX;
+            idx[TOPK - 1] = INT32_MAX;
+        }
+        if (lane == 0) {
+            cand_val[row * TOPK + t] = v;
+            cand_idx[row * TOPK + t] = (g == INT32_MAX) ? -1 : g;
+        }
+    }
+}
+
 template <int TOPK, int MODE, bool KCHUNK>
 void run_screen(const ScreenLayout& lay, const uint16_t* Yt, const uint16_t* Bt, const uint16_t* Qb3,
                 const int32_t* quad_slot, float* tau0, const int32_t* tile_j0, int64_t n_tiles, int64_t G,
                 int64_t G_pad, float* cv, int32_t* ci, int32_t* cc, int* status, const ProbeArgs& pa,
-                const ListArgs& la, const WaitTest& wt, int n_sm, cudaStream_t st) {
+                const ListArgs& la, const WaitTest& wt, const ScreenSplit& ss, int n_sm, cudaStream_t st) {
     auto kern = k_screen<TOPK, MODE, KCHUNK>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes);
-    int64_t grid = n_tiles < n_sm ? n_tiles : n_sm;
+    const int n_gt = (int)(G_pad / kBN);
+    const bool split = ss.parts > 1;
+    const int64_t rows = n_tiles * kBM;
+    const SplitArgs sp{split ? ss.parts : 1, split ? ss.len : n_gt, ss.key};
+    const int64_t items = n_tiles * sp.parts;
+    int64_t grid = items < n_sm ? items : n_sm;
     if (grid < 1) grid = 1;
+    float* ov = cv;
+    int32_t* oi = ci;
+    if (split && MODE == kModeTopK) {
+        ov = ss.val;
+        oi = ss.idx;
+    }
+    if (split && MODE == kModeMin) cudaMemsetAsync(ss.key, 0xff, (size_t)rows * 8, st);
+    if (split && MODE == kModeList) cudaMemsetAsync(cc, 0, (size_t)rows * 2 * sizeof(int32_t), st);
     count_launch();
     kern<<<(unsigned)grid, 64 + 32 * kEpiWarps, lay.bytes, st>>>(Yt, Bt, Qb3, quad_slot, tau0, tile_j0, n_tiles, G,
-                                                                   G_pad, cv, ci, cc, status, pa, lay, la, wt);
+                                                                   G_pad, ov, oi, cc, status, pa, lay, la, wt, sp);
     if (MODE == kModeMin) {
-        const int64_t rows = n_tiles * kBM;
         count_launch();
-        k_min_seed<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Yt, quad_slot, ci, tau0, rows, G, G_pad, pa,
-                                                                   status);
+        k_min_seed<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(Yt, quad_slot, ci, split ? ss.key : nullptr, tau0,
+                                                                   rows, G, G_pad, pa, status);
+    }
+    if (split && MODE == kModeTopK) {
+        count_launch();
+        k_topk_merge<TOPK><<<(unsigned)((rows + 3) / 4), 128, 0, st>>>(ss.val, ss.idx, ss.parts, rows, cv, ci);
     }
 }
 
@@ -686,6 +841,35 @@ ScreenLayout choose_layout(int K, int stages, int ybuf) {
 
 }  // namespace
 
+// Ranges a screen launch of n_tiles universe tiles cuts the grid into.  The
+// launch takes ceil(items / SMs) rounds of one range each plus, per item, a
+// start-up of about kItemTiles grid tiles (A image, pipeline fill, hand-over
+// of the lists); the cheapest number of ranges wins.  A split adds a merge
+// launch (about kMergeTiles grid tiles of time), so it has to save that and a
+// tenth, and a range holds at least kMinRange grid tiles.  Launches with many
+// tiles per SM have nothing to gain and stay unsplit.
+int screen_parts(int64_t n_tiles, int64_t G_pad, int n_sm, int* len) {
+    constexpr int kItemTiles = 3, kMergeTiles = 4, kMinRange = 4;
+    const int64_t n_gt = G_pad / kBN;
+    *len = (int)n_gt;
+    if (n_tiles <= 0 || n_tiles >= 8 * (int64_t)n_sm) return 1;
+    auto cost = [&](int64_t parts) {
+        const int64_t l = (n_gt + parts - 1) / parts;
+        return ((n_tiles * parts + n_sm - 1) / n_sm) * (l + kItemTiles);
+    };
+    const int64_t unsplit = cost(1);
+    int64_t best = 1, best_cost = unsplit - std::max<int64_t>(unsplit / 10, kMergeTiles);
+    const int64_t most = std::min<int64_t>(n_gt / kMinRange, std::max<int64_t>(2, 4 * (int64_t)n_sm / n_tiles));
+    for (int64_t p = 2; p <= most; ++p)
+        if (cost(p) < best_cost) {
+            best = p;
+            best_cost = cost(p);
+        }
+    if (best == 1) return 1;
+    *len = (int)((n_gt + best - 1) / best);
+    return (int)((n_gt + *len - 1) / *len);  // no empty range
+}
+
 bool screen_config_ok(int K, int stages, int ybuf) {
     if (K < 16 || K % 16 != 0 || K > kMaxScreenK) return false;
     if (stages != 0 && (stages < 2 || stages > 8)) return false;
@@ -699,14 +883,14 @@ bool launch_screen(int K, int topk, int mode, int stages, int ybuf, const uint16
                    const uint16_t* Qb3, const int32_t* quad_slot, float* tau0, const int32_t* tile_j0,
                    int64_t n_tiles, int64_t G, int64_t G_pad, float* cv, int32_t* ci, int32_t* cc, int* status,
                    const float* Qc, const float* Qb, const float4* gnorm, const float4* alpha, const GridSpec& gs,
-                   int nfit, const ListArgs& la, const WaitTest& wt, int n_sm, cudaStream_t st) {
+                   int nfit, const ListArgs& la, const WaitTest& wt, const ScreenSplit& ss, int n_sm, cudaStream_t st) {
     if (n_tiles <= 0) return true;
     if (!screen_config_ok(K, stages, ybuf) || (topk != 4 && topk != 8 && topk != 16)) return false;
     const ScreenLayout lay = choose_layout(K, stages, ybuf);
     const ProbeArgs pa{Qc, Qb, gnorm, alpha, gs, nfit};
 #define FC_SCREEN_RUN(TT, MM, CC) \
     run_screen<TT, MM, CC>(lay, Yt, Bt, Qb3, quad_slot, tau0, tile_j0, n_tiles, G, G_pad, cv, ci, cc, status, pa, la, \
-                           wt, n_sm, st)
+                           wt, ss, n_sm, st)
 #define FC_SCREEN_MODES(TT, CC)                 \
     do {                                        \
         if (mode == kModeMin)                   \
