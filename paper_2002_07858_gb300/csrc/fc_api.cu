@@ -130,7 +130,7 @@ struct Grid {
     int32_t* slot_of = nullptr;      // device [G]
     double* A64 = nullptr;           // [cap][nfit][nfit]
     double* W64 = nullptr;           // [cap][nfit][nfit]  A = W^T W, W lower triangular
-    float2* Wdf = nullptr;           // [cap][nfit][nfit]  W as double-float
+    float* Wdf = nullptr;            // [cap][wdf_bytes / 4]  W as double-float, blocked rows
     float* A32 = nullptr;
     float* rho = nullptr;
     uint16_t* Wimg = nullptr;        // [cap][2K][K] bf16 hi/lo image of W (tensor-core q-vectors)
@@ -395,7 +395,7 @@ void reset_cache(fc_ctx* c, Grid* g) {
 // Device bytes one cache slot costs (covariance, W image, binary32 q-vectors,
 // binary64 q-vectors).
 size_t slot_bytes(const Grid* g) {
-    return (size_t)g->nfit * g->nfit * (8 + 8 + 8 + 4) + 4 + (size_t)4 * g->K * g->K + 16 + (size_t)g->G_pad * 24 +
+    return (size_t)g->nfit * g->nfit * (8 + 8 + 4) + wdf_bytes(g->nfit) + 4 + (size_t)4 * g->K * g->K + 16 + (size_t)g->G_pad * 24 +
            (size_t)g->G * 8;
 }
 
@@ -442,7 +442,7 @@ fc_status grow_cache(fc_ctx* c, Grid* g, int64_t new_cap) {
     const size_t n2 = (size_t)g->nfit * g->nfit;
     FC_TRY(regrow(c, &g->A64, n2, old, new_cap));
     FC_TRY(regrow(c, &g->W64, n2, old, new_cap));
-    FC_TRY(regrow(c, &g->Wdf, n2, old, new_cap));
+    FC_TRY(regrow(c, &g->Wdf, wdf_bytes(g->nfit) / sizeof(float), old, new_cap));
     FC_TRY(regrow(c, &g->A32, n2, old, new_cap));
     FC_TRY(regrow(c, &g->rho, 1, old, new_cap));
     if (g->Wimg) FC_TRY(regrow(c, &g->Wimg, (size_t)2 * g->K * g->K, old, new_cap));
@@ -1132,7 +1132,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     FC_TRY(scratch(c, "rs_counts", 2, &ra.counts));
                     FC_TRY(scratch(c, "rs_tiles", (size_t)n_tiles * kQuads, &ra.tile_items));
                     FC_TRY(scratch(c, "rs_tiles2", (size_t)n_tiles * kQuads, &ra.tile_items2));
-                    launch_resolve(ra, n_tiles, c->stream);
+                    launch_resolve(ra, n_tiles, cnt, c->stream);
                 }
                 FC_TRY(stage_end(c, &S->ms_rescore));
                 return check_status(c);

@@ -172,10 +172,11 @@ void launch_scan64(const int32_t* list, int64_t n, const int32_t* uslot_of_list,
 
 // exact residual-form scan of the mixed path (double-float, split over nsp CTAs per universe)
 void launch_scan_resid(const int32_t* list, int64_t n, const int32_t* uslot, const float* d, const GridSpec& gs,
-                       int64_t G, int nfit, const float2* Wdf, double* part_v, int32_t* part_g, int nsp,
+                       int64_t G, int nfit, const float* Wdf, double* part_v, int32_t* part_g, int nsp,
                        int32_t* best, cudaStream_t st);
-// double-float copies: W of a list of slots; any binary64 array
-void launch_wdf(const double* W64, const int32_t* slots, int n, int nfit, float2* Wdf, cudaStream_t st);
+// double-float copies: W of a list of slots (blocked rows, wdf_bytes a slot); any binary64 array
+size_t wdf_bytes(int nfit);
+void launch_wdf(const double* W64, const int32_t* slots, int n, int nfit, float* Wdf, cudaStream_t st);
 void launch_to_df(const double* x, int64_t n, float2* y, cudaStream_t st);
 
 // ---- mixed path: grouping, y prep, screen, decision ----
@@ -247,7 +248,7 @@ struct ResolveArgs {
     GridSpec gs;           // the grid's fit-space rows (stored or recomputed)
     int nfit;
     const double* W64;
-    const float2* Wdf;     // [slots][nfit][nfit] double-float W
+    const float* Wdf;      // [slots][wdf_bytes / 4] double-float W
     const float2* centre_df;  // [nfit] double-float centre
     int32_t* cur;          // [n] covariance grid index, advanced for continuing universes
     const int32_t* pt;     // [n] true point of the universe
@@ -295,7 +296,7 @@ void launch_min_tau(const int32_t* tile_univ, int64_t n_tiles, const float* thr,
 // (complete lists certify the minimum); overflowing rows go to `fb`.
 // list rounds: n_rows = universes in the round's tiles; rows [n_tiles * BM] and n_rows_dev are scratch
 // Work split of a list round: chunks of kListChunk listed points of one row.
-constexpr int kListChunk = 32;
+constexpr int kListChunk = 8;
 struct ListPlan {
     int2* chunk;        // [max_chunks] (listed-row index w, chunk k of that row); w < 0: no work
     int32_t* n_chunk;   // device count of chunks
@@ -308,7 +309,8 @@ struct ListPlan {
 };
 void launch_resolve_list(const ResolveArgs& a, const int32_t* cand_count, int64_t n_tiles, int64_t n_rows,
                          int32_t* rows, int32_t* n_rows_dev, const ListPlan& lp, cudaStream_t st);
-void launch_resolve(const ResolveArgs& a, int64_t n_tiles, cudaStream_t st);
+// n_rows: universes in the tiles
+void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaStream_t st);
 
 // ---- final residual-form chi2 and dchi2 ----
 // Per-universe state of a scan: cur (covariance index), pt (true point),
@@ -324,7 +326,7 @@ struct UniverseState {
 // Wdf given: the mixed path's double-float residuals; null: binary64 (plain path)
 void launch_finish(const int32_t* list, int64_t n, const int32_t* uslot_of_list, const int32_t* best,
                    const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64,
-                   const float2* Wdf, double* dchi2, double* chi2min, cudaStream_t st);
+                   const float* Wdf, double* dchi2, double* chi2min, cudaStream_t st);
 // advance: converged / exhausted universes -> finish list, others stay active
 void launch_advance(const int32_t* active, int64_t n_active, const int32_t* best, const UniverseState& us,
                     int32_t* next_active, int32_t* n_next, int32_t* finish_list, int32_t* n_finish, cudaStream_t st);

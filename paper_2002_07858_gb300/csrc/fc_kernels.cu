@@ -66,174 +66,168 @@ __device__ double resid_chi2_warp(const double* __restrict__ W, int n, const dou
 }
 
 // The mixed path's residual chi2 = |W (s - d)|^2 in double-float (fc_df.cuh):
-// r_j = s_j - d_j, t_i = sum_j W_ij r_j (df_row), chi2 = sum_i t_i^2 in
-// increasing i.  Every mixed-path kernel evaluates
-// it in this order, so a universe's result has the same bits whichever
-// certified round decided it.  W and s are double-float copies of the
-// binary64 arrays; the value is returned as binary64.
+// r_j = s_j - d_j, t_i = sum_j W_ij r_j, chi2 = sum_i t_i^2 in increasing i.
+// Every mixed-path kernel evaluates it in this order, so a universe's result
+// has the same bits whichever certified round decided it.  W and s are
+// double-float copies of the binary64 arrays; the value is returned as
+// binary64.
 // Row i of W r: four interleaved partial sums (j = 0, 1, 2, 3 mod 4, each in
-// increasing j) so that four double-float chains run side by side, combined
-// as (p0 + p1) + (p2 + p3) and renormalised.  A row runs over whole blocks of
-// four columns, j < min(4 ceil((i + 1) / 4), N_fit): W is lower triangular
-// with exact zeros above the diagonal (k_build_cov), so the columns past the
-// diagonal add exact zeros and every kernel takes the same blocks.
-__device__ __forceinline__ float2 df_row(const float2* __restrict__ Wi, const float2* __restrict__ r, int len, int n) {
-    float2 p0 = make_float2(0.0f, 0.0f), p1 = p0, p2 = p0, p3 = p0;
-    for (int j = 0; j < len; j += 4) {
-        p0 = df_fma(p0, Wi[j], r[j]);
-        if (j + 1 < n) p1 = df_fma(p1, Wi[j + 1], r[j + 1]);
-        if (j + 2 < n) p2 = df_fma(p2, Wi[j + 2], r[j + 2]);
-        if (j + 3 < n) p3 = df_fma(p3, Wi[j + 3], r[j + 3]);
-    }
-    const float2 a = df_add(df_norm(p0.x, p0.y), df_norm(p1.x, p1.y));
-    const float2 b = df_add(df_norm(p2.x, p2.y), df_norm(p3.x, p3.y));
-    return df_add(a, b);
+// increasing j), combined as (p0 + p1) + (p2 + p3) and renormalised.  A row
+// runs over whole blocks of four columns; W is lower triangular and W and r
+// are zero past N_fit, so columns past the diagonal add exact zeros and it
+// does not matter how many of them a kernel takes.
+// Sums 0 and 2 share a packed pair and so do 1 and 3 (df2x): a block of four
+// columns is two packed multiply-adds, and (p0 + p1, p2 + p3) is one packed
+// add.  Both operands are stored for that, eight floats per block of columns
+// j..j+3: (hi_j, hi_j+2), (lo_j, lo_j+2), (hi_j+1, hi_j+3), (lo_j+1, lo_j+3).
+__host__ __device__ __forceinline__ int df_blocks(int n) { return (n + 3) / 4; }
+// float position of column j's hi half inside a blocked row (the lo half is two floats on)
+__device__ __forceinline__ int df_pos(int j) { return (j >> 2) * 8 + (j & 1) * 4 + ((j >> 1) & 1); }
+
+// W of a slot: block jb of row i at float4 index (jb n + i) 2 (k_wdf), so the
+// lanes of a warp that hold consecutive rows read consecutive memory.
+__device__ __forceinline__ size_t wdf_floats(int n) { return (size_t)df_blocks(n) * n * 8; }
+
+// (p0 + p1) + (p2 + p3) of the packed sums (0, 2) and (1, 3)
+__device__ __forceinline__ float2 df_row_sum(df2x s02, df2x s13) {
+    const df2x h = df2_add(df2_norm(s02), df2_norm(s13));
+    return df_add(make_float2(x2_lo(h.x), x2_lo(h.y)), make_float2(x2_hi(h.x), x2_hi(h.y)));
 }
 
-// Four consecutive entries W[k .. k+3] of a W row: two 16-byte loads when
-// rows start on 16 bytes at multiple-of-4 columns (even N_fit), else four.
-template <bool EVEN>
-__device__ __forceinline__ void w_load4(const float2* __restrict__ Wk, float2 (&w)[4]) {
-    if constexpr (EVEN) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(Wk));
-        const float4 b = __ldg(reinterpret_cast<const float4*>(Wk) + 1);
-        w[0] = make_float2(a.x, a.y);
-        w[1] = make_float2(a.z, a.w);
-        w[2] = make_float2(b.x, b.y);
-        w[3] = make_float2(b.z, b.w);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) w[c] = __ldg(Wk + c);
-    }
-}
-
-// The residual chi2 computed four rows at a time: each group of four columns
-// of r is loaded once per block of rows i0 .. i0+3 (i0 a multiple of 4) and
-// meets the four rows' W entries.  Row i keeps df_row's four chains (column j
-// on chain j mod 4, each chain in increasing j) and the rows are squared and
-// summed in increasing i, so every operation and its order are df_row's and
-// the row loop's: the bits are the same, with a quarter of the loads of r.
-// In the last block, rows past N_fit read row N_fit - 1 and are dropped.
-template <bool EVEN, class SRow>
-__device__ __forceinline__ double resid_df_blk(const float2* __restrict__ W, int n, const SRow& s,
-                                               const float* __restrict__ du) {
-    __align__(16) float2 r[kMaxBins + 4];
-    for (int j = 0; j < n; ++j) r[j] = df_sub_f(s[j], du[j]);
-    float2 acc = make_float2(0.0f, 0.0f);
-    for (int i0 = 0; i0 < n; i0 += 4) {
-        float2 p[4][4];
-        const float2* Wb[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            Wb[b] = W + (i0 + b < n ? i0 + b : n - 1) * n;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) p[b][c] = make_float2(0.0f, 0.0f);
-        }
-        // columns 0 .. i0-1: every row of the block takes all four of each group
-#pragma unroll 1
-        for (int j = 0; j < i0; j += 4) {
-            const float4 ra = *reinterpret_cast<const float4*>(&r[j]);
-            const float4 rb = *reinterpret_cast<const float4*>(&r[j + 2]);
-            const float2 rv[4] = {make_float2(ra.x, ra.y), make_float2(ra.z, ra.w), make_float2(rb.x, rb.y),
-                                  make_float2(rb.z, rb.w)};
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                float2 w[4];
-                w_load4<EVEN>(Wb[b] + j, w);
-#pragma unroll
-                for (int c = 0; c < 4; ++c) p[b][c] = df_fma(p[b][c], w[c], rv[c]);
-            }
-        }
-        // columns i0 .. i0+3 (those below N_fit): the whole block for every row of the block
-        // (W is zero above the diagonal)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            if (i0 + c < n) {
-                const float2 rc = r[i0 + c];
-#pragma unroll
-                for (int b = 0; b < 4; ++b) p[b][c] = df_fma(p[b][c], Wb[b][i0 + c], rc);
-            }
-        }
-        const int nb = (n - i0 < 4) ? n - i0 : 4;  // rows of this block that exist
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            if (b < nb) {
-                const float2 x = df_add(df_norm(p[b][0].x, p[b][0].y), df_norm(p[b][1].x, p[b][1].y));
-                const float2 y = df_add(df_norm(p[b][2].x, p[b][2].y), df_norm(p[b][3].x, p[b][3].y));
-                const float2 t = df_add(x, y);
-                acc = df_fma(acc, t, t);
-            }
-        }
-    }
-    return df_to(df_norm(acc.x, acc.y));
-}
-
-// s: the row s_g as double-float (a stored row, or a DfRow that may evaluate the shape model)
-template <class SRow>
-__device__ double resid_df(const float2* __restrict__ W, int n, const SRow& s, const float* __restrict__ du) {
-    return (n % 2 == 0) ? resid_df_blk<true>(W, n, s, du) : resid_df_blk<false>(W, n, s, du);
-}
-
-// resid_df with the residual vector in registers, for N_fit <= NR: every index
-// of r is a compile-time constant (the column loop is unrolled in blocks of
-// four and a block runs only when the row reaches it, a branch that is uniform
-// across the warp because all its lanes walk the same rows).  The operations
-// and their order are resid_df's, term for term, so the bits are the same;
-// what changes is that no per-thread array lives in local memory.
+// One thread per residual, N_fit <= NR, the residual vector in registers
+// (every index of it a compile-time constant; a block of columns runs only
+// when the row reaches it, a branch that is uniform across the warp because
+// all its lanes walk the same rows).  W: the slot's blocked W in shared
+// memory, read as one broadcast of 16 bytes per packed multiply-add.
 template <int NR, class SRow>
-__device__ __forceinline__ double resid_df_reg(const float2* __restrict__ W, int n, const SRow& s,
+__device__ __forceinline__ double resid_df_reg(const ulonglong2* __restrict__ W, int n, const SRow& s,
                                                const float* __restrict__ du) {
     static_assert(NR % 4 == 0, "NR is a multiple of 4");
-    float2 r[NR];
+    f32x2 rx[NR / 2], ry[NR / 2];  // [2 jb + h]: columns 4 jb + h and 4 jb + h + 2
 #pragma unroll
-    for (int j = 0; j < NR; ++j) r[j] = (j < n) ? df_sub_f(s[j], du[j]) : make_float2(0.0f, 0.0f);
+    for (int k = 0; k < NR / 2; ++k) {
+        const int j = (k >> 1) * 4 + (k & 1);
+        const float2 a = (j < n) ? df_sub_f(s[j], du[j]) : make_float2(0.0f, 0.0f);
+        const float2 b = (j + 2 < n) ? df_sub_f(s[j + 2], du[j + 2]) : make_float2(0.0f, 0.0f);
+        rx[k] = x2_pack(a.x, b.x);
+        ry[k] = x2_pack(a.y, b.y);
+    }
     float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
-        const float2* Wi = W + i * n;
-        const int len = i + 1;
-        float2 p0 = make_float2(0.0f, 0.0f), p1 = p0, p2 = p0, p3 = p0;
+        const ulonglong2* Wi = W + 2 * i;
+        const int last = i >> 2;
+        df2x s02{0ull, 0ull}, s13{0ull, 0ull};
 #pragma unroll
-        for (int j = 0; j < NR; j += 4) {
-            if (j < len) {  // whole blocks (df_row)
-                p0 = df_fma(p0, Wi[j], r[j]);
-                if (j + 1 < n) p1 = df_fma(p1, Wi[j + 1], r[j + 1]);
-                if (j + 2 < n) p2 = df_fma(p2, Wi[j + 2], r[j + 2]);
-                if (j + 3 < n) p3 = df_fma(p3, Wi[j + 3], r[j + 3]);
+        for (int jb = 0; jb < NR / 4; ++jb) {
+            if (jb <= last) {
+                const ulonglong2 w0 = Wi[jb * 2 * n], w1 = Wi[jb * 2 * n + 1];
+                s02 = df2_fma(s02, w0.x, w0.y, rx[2 * jb], ry[2 * jb]);
+                s13 = df2_fma(s13, w1.x, w1.y, rx[2 * jb + 1], ry[2 * jb + 1]);
             }
         }
-        const float2 a = df_add(df_norm(p0.x, p0.y), df_norm(p1.x, p1.y));
-        const float2 b = df_add(df_norm(p2.x, p2.y), df_norm(p3.x, p3.y));
-        const float2 t = df_add(a, b);
+        const float2 t = df_row_sum(s02, s13);
         acc = df_fma(acc, t, t);
     }
     return df_to(df_norm(acc.x, acc.y));
 }
 
-// The mixed path's residual chi2 for a compile-time bound NR on N_fit (0 = any N_fit).
-template <int NR, class SRow>
-__device__ __forceinline__ double resid_mixed(const float2* __restrict__ W, int n, const SRow& s,
-                                              const float* __restrict__ du) {
-    if constexpr (NR > 0)
-        return resid_df_reg<NR>(W, n, s, du);
-    else
-        return resid_df(W, n, s, du);
+// One warp per group of up to B residuals under one W (any N_fit): each lane
+// owns a row of W, 32 rows at a time, and every W block it loads meets the B
+// residual vectors, which wait in the warp's shared memory; lane k then sums
+// residual k's t_i^2.  This is the form for few residuals, for covariances
+// with few residuals each and for N_fit > 64: a residual is spread over the
+// warp, W is read coalesced and once per group, and nothing lives in local
+// memory.  Bound by the binary32 pipe when there are enough groups, else by
+// the latency of one group.  Against one thread per residual everywhere: a
+// scan of 4096 data sets on 141x141 1.15 -> 0.76 ms, one point of 25x25 x 1000
+// universes 2.59 -> 1.88 ms, 4 points of 27^3 with N = 200 61.3 -> 49.6 ms.
+constexpr int kRowsB = 4;       // residuals of a group
+constexpr int kRowsWarps = 4;   // warps of a CTA of the row kernels
+// shared memory of one warp, in floats: kRowsB blocked residual vectors and row sums
+__host__ __device__ __forceinline__ int rows_floats(int n) { return kRowsB * df_blocks(n) * 8 + kRowsB * df_blocks(n) * 8; }
+__host__ __forceinline__ size_t rows_smem(int n) { return (size_t)kRowsWarps * rows_floats(n) * sizeof(float); }
+
+// residual vector k of a group into the warp's shared memory sr (zero past N_fit)
+template <class SRow>
+__device__ __forceinline__ void rows_stage(float* sr, int k, int n, const SRow& s, const float* __restrict__ du,
+                                           int lane) {
+    float* r = sr + k * df_blocks(n) * 8;
+    for (int j = lane; j < df_blocks(n) * 4; j += 32) {
+        const float2 v = (j < n) ? df_sub_f(s[j], du[j]) : make_float2(0.0f, 0.0f);
+        r[df_pos(j)] = v.x;
+        r[df_pos(j) + 2] = v.y;
+    }
 }
 
-// resid_df spread over a warp with the same bits: r_j = s_j - d_j is formed in
-// this warp's shared vector r, lanes form the rows t_i into t, lane 0 sums
-// t_i^2 in row order.  The result is lane 0's.
-template <class SRow>
-__device__ double resid_df_warp(const float2* __restrict__ W, int n, const SRow& s, const float* __restrict__ du,
-                                float2* r, float2* t, int lane) {
-    for (int j = lane; j < n; j += 32) r[j] = df_sub_f(s[j], du[j]);
+template <int B>
+__device__ __forceinline__ void rows_products(const ulonglong2* __restrict__ W, int n, const ulonglong2* sr, float4* st,
+                                              int lane) {
+    const int nb = df_blocks(n);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+        const int i = i0 + lane;
+        const ulonglong2* Wi = W + 2 * (i < n ? i : n - 1);
+        const int nblk = min(nb, (i0 + 31) / 4 + 1);
+        df2x s02[B], s13[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) s02[k] = s13[k] = df2x{0ull, 0ull};
+        ulonglong2 w0 = __ldg(Wi), w1 = __ldg(Wi + 1);
+#pragma unroll 2
+        for (int jb = 0; jb < nblk; ++jb) {
+            const ulonglong2 c0 = w0, c1 = w1;
+            if (jb + 1 < nblk) {  // the next block's W is on its way while this one is used
+                w0 = __ldg(Wi + (size_t)(jb + 1) * 2 * n);
+                w1 = __ldg(Wi + (size_t)(jb + 1) * 2 * n + 1);
+            }
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const ulonglong2 r0 = sr[(k * nb + jb) * 2], r1 = sr[(k * nb + jb) * 2 + 1];
+                s02[k] = df2_fma(s02[k], c0.x, c0.y, r0.x, r0.y);
+                s13[k] = df2_fma(s13[k], c1.x, c1.y, r1.x, r1.y);
+            }
+        }
+        if (i < n) {
+            // t_i^2 as the product and its error term, the part of df_fma that needs no order
+#pragma unroll
+            for (int k = 0; k < B; ++k) {
+                const float2 t = df_row_sum(s02[k], s13[k]);
+                const float p = __fmul_rn(t.x, t.x);
+                float e = __fmaf_rn(t.x, t.x, -p);
+                e = __fmaf_rn(t.x, t.y, e);
+                e = __fmaf_rn(t.y, t.x, e);
+                reinterpret_cast<float2*>(st)[k * nb * 4 + i] = make_float2(p, e);
+            }
+        }
+    }
+}
+
+// chi2 of the m <= kRowsB staged residuals; residual k's value is lane k's
+// result.  sm: the warp's shared memory (rows_floats), its vectors staged.
+__device__ __forceinline__ double rows_chi2(const float* __restrict__ Wslot, int n, float* sm, int m, int lane) {
+    const int nb = df_blocks(n);
+    const ulonglong2* W = reinterpret_cast<const ulonglong2*>(Wslot);
+    const ulonglong2* sr = reinterpret_cast<const ulonglong2*>(sm);
+    float4* st = reinterpret_cast<float4*>(sm + kRowsB * nb * 8);
     __syncwarp();
-    for (int i = lane; i < n; i += 32) t[i] = df_row(W + i * n, r, i + 1, n);
+    if (m <= 1)
+        rows_products<1>(W, n, sr, st, lane);
+    else if (m <= 2)
+        rows_products<2>(W, n, sr, st, lane);
+    else
+        rows_products<kRowsB>(W, n, sr, st, lane);
     __syncwarp();
     float2 acc = make_float2(0.0f, 0.0f);
-    if (lane == 0)
-        for (int i = 0; i < n; ++i) acc = df_fma(acc, t[i], t[i]);
-    __syncwarp();
+    if (lane < m) {
+        const float2* t = reinterpret_cast<const float2*>(st) + lane * nb * 4;
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+            const float2 pe = t[i];
+            float s, err;
+            two_sum(acc.x, pe.x, s, err);
+            acc = make_float2(s, __fadd_rn(acc.y, __fadd_rn(err, pe.y)));
+        }
+    }
+    __syncwarp();  // the shared memory may be staged again
     return df_to(df_norm(acc.x, acc.y));
 }
 
@@ -250,11 +244,19 @@ __device__ __forceinline__ auto srow(const GridSpec& gs, const float2* centre_df
         return (g < 0) ? centre_df : gs.Sdf + g * gs.nfit;
 }
 
-// double-float copies of W for a list of slots
+// blocked double-float copies of W for a list of slots
 __global__ void k_wdf(const double* __restrict__ W64, const int32_t* __restrict__ slots, int nfit,
-                      float2* __restrict__ Wdf) {
-    const size_t base = (size_t)slots[blockIdx.x] * nfit * nfit;
-    for (int e = threadIdx.x; e < nfit * nfit; e += blockDim.x) Wdf[base + e] = df_from(W64[base + e]);
+                      float* __restrict__ Wdf) {
+    const double* W = W64 + (size_t)slots[blockIdx.x] * nfit * nfit;
+    float* o = Wdf + (size_t)slots[blockIdx.x] * wdf_floats(nfit);
+    const int np = df_blocks(nfit) * 4;
+    for (int e = threadIdx.x; e < nfit * np; e += blockDim.x) {
+        const int i = e / np, j = e % np;
+        const float2 v = (j <= i) ? df_from(W[i * nfit + j]) : make_float2(0.0f, 0.0f);
+        float* w = o + ((size_t)(j >> 2) * nfit + i) * 8 + (j & 1) * 4 + ((j >> 1) & 1);
+        w[0] = v.x;
+        w[2] = v.y;
+    }
 }
 
 __global__ void k_to_df(const double* __restrict__ x, int64_t n, float2* __restrict__ y) {
@@ -1014,44 +1016,46 @@ __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restric
 
 // Exact residual-form scan (Algorithm 2 for every g) of the universes in
 // `list`, used when all certified screen rounds failed, so it never needs
-// binary64 q-vectors.  Grid (universe, split): each CTA stages W of the
-// universe's covariance in shared memory and scans every split-th grid point;
-// k_scan_resid_reduce takes the first minimum over the splits.
+// binary64 q-vectors.  Grid (universe, split): the warps of a CTA walk groups
+// of kRowsB grid points of its share (rows_chi2); k_scan_resid_reduce takes the
+// first minimum over the splits.
 template <bool MODEL>
-__global__ void __launch_bounds__(256) k_scan_resid(const int32_t* __restrict__ list, const int32_t* __restrict__ uslot,
-                                                     const float* __restrict__ d, GridSpec gs,
-                                                     int64_t G, int nfit, const float2* __restrict__ Wdf,
-                                                     double* __restrict__ part_v, int32_t* __restrict__ part_g) {
-    extern __shared__ float2 sWd[];
-    __shared__ double rv[8];
-    __shared__ int32_t rg[8];
+__global__ void __launch_bounds__(32 * kRowsWarps) k_scan_resid(const int32_t* __restrict__ list,
+                                                                const int32_t* __restrict__ uslot,
+                                                                const float* __restrict__ d, GridSpec gs, int64_t G,
+                                                                int nfit, const float* __restrict__ Wdf,
+                                                                double* __restrict__ part_v,
+                                                                int32_t* __restrict__ part_g) {
+    extern __shared__ float4 s_rows[];
+    __shared__ double rv[kRowsWarps];
+    __shared__ int32_t rg[kRowsWarps];
     const int i = blockIdx.x, sp = blockIdx.y, nsp = gridDim.y;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* sm = reinterpret_cast<float*>(s_rows) + warp * rows_floats(nfit);
     const int u = list[i];
-    const float2* Wg = Wdf + (size_t)uslot[i] * nfit * nfit;
-    const bool staged = (nfit <= kResolveMaxN);
-    if (staged)
-        for (int e = threadIdx.x; e < nfit * nfit; e += blockDim.x) sWd[e] = Wg[e];
-    __syncthreads();
-    const float2* W = staged ? sWd : Wg;
+    const float* W = Wdf + (size_t)uslot[i] * wdf_floats(nfit);
     const float* du = d + (size_t)u * nfit;
     double bv = DBL_MAX;
     int32_t bg = INT32_MAX;
-    for (int64_t g = (int64_t)sp * blockDim.x + threadIdx.x; g < G; g += (int64_t)nsp * blockDim.x) {
-        const double c = resid_df(W, nfit, srow<MODEL>(gs, nullptr, g), du);
-        if (c < bv) {
+    const int64_t step = (int64_t)nsp * kRowsWarps * kRowsB;
+    for (int64_t g0 = ((int64_t)sp * kRowsWarps + warp) * kRowsB; g0 < G; g0 += step) {
+        const int m = (int)(G - g0 < kRowsB ? G - g0 : kRowsB);
+        for (int k = 0; k < m; ++k) rows_stage(sm, k, nfit, srow<MODEL>(gs, nullptr, g0 + k), du, lane);
+        const double c = rows_chi2(W, nfit, sm, m, lane);
+        if (lane < m && c < bv) {
             bv = c;
-            bg = (int32_t)g;
+            bg = (int32_t)(g0 + lane);
         }
     }
     warp_argmin(bv, bg);
-    if ((threadIdx.x & 31) == 0) {
-        rv[threadIdx.x >> 5] = bv;
-        rg[threadIdx.x >> 5] = bg;
+    if (lane == 0) {
+        rv[warp] = bv;
+        rg[warp] = bg;
     }
     __syncthreads();
     if (threadIdx.x < 32) {
-        bv = threadIdx.x < (blockDim.x >> 5) ? rv[threadIdx.x] : DBL_MAX;
-        bg = threadIdx.x < (blockDim.x >> 5) ? rg[threadIdx.x] : INT32_MAX;
+        bv = threadIdx.x < kRowsWarps ? rv[threadIdx.x] : DBL_MAX;
+        bg = threadIdx.x < kRowsWarps ? rg[threadIdx.x] : INT32_MAX;
         warp_argmin(bv, bg);
         if (threadIdx.x == 0) {
             part_v[(size_t)i * nsp + sp] = bv;
@@ -1325,13 +1329,13 @@ constexpr int kItemCodes = kMaxTopK + 3;
 // waited at barriers for the rows with many).
 //  k_resolve_emit     per row: the screen certificate (decide_row); the
 //                     residual items the row needs, appended in tile order;
-//  k_resid_items      every item's double-float residual chi2 (W of the row's
+//  k_resid_tiles/rows every item's double-float residual chi2 (W of the row's
 //                     covariance slot; the residual vector in registers);
 //  k_resolve_conclude per row: the same decision again, then the rescored
 //                     minimum and its certificate; finish (dchi2) / advance /
 //                     hand on, exactly as one kernel did before; rescored rows
 //                     that finish with p != best list their chi2_p;
-//  k_resid_items      those chi2_p;
+//  k_resid_tiles/rows those chi2_p;
 //  k_resolve_tail     their dchi2.
 // Decision per row (§2 steps 3-4 with the screen's certificate):
 //  1. from the screen's lower bounds LB and upper bounds UB = LB + 2 eps of
@@ -1453,21 +1457,25 @@ __global__ void __launch_bounds__(kBM) k_resolve_emit(ResolveArgs a) {
     }
 }
 
-// Residual chi2 of one tile's items.  The items of each quadrant are a
-// contiguous range (tile_items[4t + w]) and the tile's quadrants follow each
-// other; a run of quadrants with one covariance slot shares one W, staged in
-// shared memory (every lane reads the same element at once), and the lanes
-// stride over the run's items with no barrier but the staging's.  A tile
-// whose quadrants share one slot stages once.  Small CTAs (two warps) keep the
-// last, partly filled round of a run cheap.
+// Residual chi2 of one tile's items, for launches whose tiles are well filled
+// (N_fit <= 64, stored rows).  The items of each quadrant are a contiguous
+// range (tile_items[4t + w]) and the tile's quadrants follow each other; a run
+// of quadrants with one covariance slot shares one W, staged in shared memory
+// (every lane reads the same element at once), and the lanes stride over the
+// run's items with no barrier but the staging's.  A tile whose quadrants share
+// one slot stages once.  Small CTAs (two warps) keep the last, partly filled
+// round of a run cheap.  Bound by issue: the packed multiply-add takes 14
+// instructions for two (24 unpacked) and one 16-byte broadcast of W instead of
+// two 8-byte ones; the full 100x100 job went from 178.1 to 171.1 ms with it.
 constexpr int kResidThreads = 64;
 
 template <int NR>
 __global__ void __launch_bounds__(kResidThreads, 6) k_resid_tiles(const ResolveArgs a, const int2* __restrict__ items,
                                                                  const int2* __restrict__ tile_items,
                                                                  double* __restrict__ res) {
-    extern __shared__ float2 sWd[];
+    extern __shared__ ulonglong2 sWd[];
     const int n = a.nfit;
+    const int nw = df_blocks(n) * n * 2;
     const int64_t t = blockIdx.x;
     int w0 = 0;
     while (w0 < kQuads) {  // every bound below is the same for all lanes
@@ -1479,36 +1487,47 @@ __global__ void __launch_bounds__(kResidThreads, 6) k_resid_tiles(const ResolveA
         const int64_t i1 = (int64_t)last.x + last.y;
         w0 = w1;
         if (i1 <= i0) continue;
-        const float2* Wg = a.Wdf + (size_t)slot * n * n;
-        const float2* W = Wg;
-        if constexpr (NR > 0) {  // staged where it fits (N_fit <= 64)
-            __syncthreads();      // the previous run's reads of sWd are done
-            for (int e = threadIdx.x; e < n * n; e += blockDim.x) sWd[e] = Wg[e];
-            __syncthreads();
-            W = sWd;
-        }
+        const ulonglong2* Wg = reinterpret_cast<const ulonglong2*>(a.Wdf + (size_t)slot * wdf_floats(n));
+        __syncthreads();  // the previous run's reads of sWd are done
+        for (int e = threadIdx.x; e < nw; e += blockDim.x) sWd[e] = Wg[e];
+        __syncthreads();
         for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
             const int2 it = items[i];
             const int u = a.tile_univ[it.x];
-            res[i] = resid_mixed<NR>(W, n, srow<false>(a.gs, a.centre_df, it.y), a.d + (size_t)u * n);
+            res[i] = resid_df_reg<NR>(sWd, n, srow<false>(a.gs, a.centre_df, it.y), a.d + (size_t)u * n);
         }
     }
 }
 
-// N_fit > 64: W is not staged, so the items are scored flat, one thread per
-// item, grid-stride over the device count.  A row's items follow each other and
-// the rows of a tile quadrant share a slot, so a warp's lanes mostly read the
-// same W element at once.
+// Every other launch: groups of kRowsB consecutive items per warp, grid-stride
+// over the device count.  A row's items follow each other and the rows of a
+// tile quadrant share a slot, so a group mostly has one W; where the slot
+// changes inside a group, its runs go one after the other.
 template <bool MODEL>
-__global__ void __launch_bounds__(256) k_resid_flat(const ResolveArgs a, const int2* __restrict__ items,
-                                                    const int32_t* __restrict__ count, double* __restrict__ res) {
+__global__ void __launch_bounds__(32 * kRowsWarps) k_resid_rows(const ResolveArgs a, const int2* __restrict__ items,
+                                                                const int32_t* __restrict__ count,
+                                                                double* __restrict__ res) {
+    extern __shared__ float4 s_rows[];
     const int n = a.nfit;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* sm = reinterpret_cast<float*>(s_rows) + warp * rows_floats(n);
     const int64_t total = *count;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int2 it = items[i];
-        const int u = a.tile_univ[it.x];
-        const float2* W = a.Wdf + (size_t)a.quad_slot[it.x / kQuadRows] * n * n;
-        res[i] = resid_df(W, n, srow<MODEL>(a.gs, a.centre_df, it.y), a.d + (size_t)u * n);
+    const int64_t step = (int64_t)gridDim.x * kRowsWarps * kRowsB;
+    for (int64_t e = ((int64_t)blockIdx.x * kRowsWarps + warp) * kRowsB; e < total; e += step) {
+        const int m = (int)(total - e < kRowsB ? total - e : kRowsB);
+        for (int k0 = 0; k0 < m;) {
+            const int slot = a.quad_slot[items[e + k0].x / kQuadRows];
+            int k1 = k0;
+            for (; k1 < m; ++k1) {
+                const int2 it = items[e + k1];
+                if (a.quad_slot[it.x / kQuadRows] != slot) break;
+                rows_stage(sm, k1 - k0, n, srow<MODEL>(a.gs, a.centre_df, it.y), a.d + (size_t)a.tile_univ[it.x] * n,
+                           lane);
+            }
+            const double c = rows_chi2(a.Wdf + (size_t)slot * wdf_floats(n), n, sm, k1 - k0, lane);
+            if (lane < k1 - k0) res[e + k0 + lane] = c;
+            k0 = k1;
+        }
     }
 }
 
@@ -1692,27 +1711,27 @@ __global__ void k_list_plan(ResolveArgs a, const int32_t* __restrict__ cand_coun
     atomicAdd(&a.counters[1], 1ull);
 }
 
-// One warp per chunk (grid-stride over the device count): lane l scores listed
-// point k * kListChunk + l with the canonical residual, the warp takes the
-// first minimum (lowest index among equal values) and publishes it.  The warp
-// that completes a row's last chunk takes the first minimum over the row's
-// chunks and finishes (dchi2) or advances the row.
+// One warp per chunk (grid-stride over the device count): the warp scores the
+// chunk's points in groups of kRowsB with the canonical residual (rows_chi2),
+// takes the first minimum (lowest index among equal values) and publishes it.
+// The warp that completes a row's last chunk takes the first minimum over the
+// row's chunks and finishes (dchi2) or advances the row.
 template <bool MODEL>
-__global__ void __launch_bounds__(256) k_list_chunks(ResolveArgs a, const int32_t* __restrict__ cand_count,
-                                                     const int32_t* __restrict__ rows, ListPlan lp) {
+__global__ void __launch_bounds__(32 * kRowsWarps) k_list_chunks(ResolveArgs a, const int32_t* __restrict__ cand_count,
+                                                                 const int32_t* __restrict__ rows, ListPlan lp) {
+    extern __shared__ float4 s_rows[];
     const int n = a.nfit;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ float2 s_r[8][kMaxBins], s_t[8][kMaxBins];
+    float* sm = reinterpret_cast<float*>(s_rows) + warp * rows_floats(n);
     const int64_t total = *lp.n_chunk < lp.max_chunks ? (int64_t)*lp.n_chunk : lp.max_chunks;
-    const int64_t stride = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t e = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; e < total; e += stride) {
+    const int64_t stride = (int64_t)gridDim.x * kRowsWarps;
+    for (int64_t e = (int64_t)blockIdx.x * kRowsWarps + warp; e < total; e += stride) {
         const int2 ck = lp.chunk[e];
         if (ck.x < 0) continue;
         const int w = ck.x;
         const int64_t row = rows[w];
         const int u = a.tile_univ[row];
-        // W of the row's quadrant (double-float, read through L1: the warp's lanes read the same element)
-        const float2* W = a.Wdf + (size_t)a.quad_slot[row / kQuadRows] * n * n;
+        const float* W = a.Wdf + (size_t)a.quad_slot[row / kQuadRows] * wdf_floats(n);
         const int n0 = cand_count[row * 2], n1 = cand_count[row * 2 + 1];
         int64_t base0, base1;
         if (a.list_off) {
@@ -1725,11 +1744,20 @@ __global__ void __launch_bounds__(256) k_list_chunks(ResolveArgs a, const int32_
         const float* du = a.d + (size_t)u * n;
         double bv = DBL_MAX;
         int32_t bg = INT32_MAX;
-        const int k = ck.y * kListChunk + lane;
-        if (k < n0 + n1) {
-            const int32_t g = a.cidx[(k < n0) ? base0 + k : base1 + (k - n0)];
-            bv = resid_df(W, n, srow<MODEL>(a.gs, nullptr, g), du);
-            bg = g;
+        const int k_end = min((ck.y + 1) * kListChunk, n0 + n1);
+        for (int k0 = ck.y * kListChunk; k0 < k_end; k0 += kRowsB) {
+            const int m = min(kRowsB, k_end - k0);
+            int32_t mine = INT32_MAX;  // lane k: the group's point k
+            for (int k = 0; k < m; ++k) {
+                const int32_t g = a.cidx[(k0 + k < n0) ? base0 + k0 + k : base1 + (k0 + k - n0)];
+                if (lane == k) mine = g;
+                rows_stage(sm, k, n, srow<MODEL>(a.gs, nullptr, g), du, lane);
+            }
+            const double c = rows_chi2(W, n, sm, m, lane);
+            if (lane < m && (c < bv || (c == bv && mine < bg))) {
+                bv = c;
+                bg = mine;
+            }
         }
         warp_argmin(bv, bg);
         int last = 0;
@@ -1762,8 +1790,8 @@ __global__ void __launch_bounds__(256) k_list_chunks(ResolveArgs a, const int32_
             const int p = a.pt[u];
             double cp = 0.0;
             if (p != bg) {
-                // chi2_p in residual form (row dot products over the lanes, the bits of resid_df)
-                cp = resid_df_warp(W, n, srow<MODEL>(a.gs, nullptr, p), du, s_r[warp], s_t[warp], lane);
+                rows_stage(sm, 0, n, srow<MODEL>(a.gs, nullptr, p), du, lane);
+                cp = rows_chi2(W, n, sm, 1, lane);
                 if (lane == 0 && a.n_resid) atomicAdd(a.n_resid, 1ull);
             }
             if (lane == 0) {
@@ -1806,10 +1834,10 @@ __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list
                                                  const int32_t* __restrict__ uslot, const int32_t* __restrict__ best,
                                                  UniverseState us, const float* __restrict__ d, GridSpec gs,
                                                  int nfit, const double* __restrict__ W64,
-                                                 const float2* __restrict__ Wdf, double* __restrict__ dchi2,
+                                                 const float* __restrict__ Wdf, double* __restrict__ dchi2,
                                                  double* __restrict__ chi2min) {
+    extern __shared__ float4 s_rows[];  // mixed path
     __shared__ double rp[4][kMaxBins], rm[4][kMaxBins], tt[4][kMaxBins];
-    __shared__ float2 fr[4][kMaxBins], ft[4][kMaxBins];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * 4LL + w;
     if (i >= n) return;
@@ -1821,9 +1849,12 @@ __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list
     double cp = 0.0, cm = 0.0;
     if (Wdf) {
         // mixed path: the double-float residual of every other mixed-path kernel
-        const float2* W = Wdf + (size_t)slot * nfit * nfit;
-        cp = (p == g) ? 0.0 : resid_df_warp(W, nfit, srow<MODEL>(gs, nullptr, p), du, fr[w], ft[w], lane);
-        cm = resid_df_warp(W, nfit, srow<MODEL>(gs, nullptr, g), du, fr[w], ft[w], lane);
+        float* sm = reinterpret_cast<float*>(s_rows) + w * rows_floats(nfit);
+        rows_stage(sm, 0, nfit, srow<MODEL>(gs, nullptr, g), du, lane);
+        if (p != g) rows_stage(sm, 1, nfit, srow<MODEL>(gs, nullptr, p), du, lane);
+        const double c = rows_chi2(Wdf + (size_t)slot * wdf_floats(nfit), nfit, sm, p == g ? 1 : 2, lane);
+        cm = __shfl_sync(0xffffffffu, c, 0);
+        cp = (p == g) ? 0.0 : __shfl_sync(0xffffffffu, c, 1);
     } else {
         // plain path: binary64, in the summation order of resid_chi2_warp
         const FitRow rowp = fit_row(gs, p), rowg = fit_row(gs, g);
@@ -1976,6 +2007,15 @@ bool measure_fma_peaks(int n_sm, double* fp64_tflops, double* fp32_tflops, cudaS
 
 // ------------------------------------------------------------- launchers ----
 
+namespace {
+// shared memory beyond the 48 KB default, which also holds a kernel's static arrays (an attribute of the
+// current device, so set per launch)
+template <class K>
+void allow_smem(K kern, size_t bytes) {
+    if (bytes > 24 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+}  // namespace
+
 void launch_collapse(const double* S, int64_t G, int nf, const int32_t* coll, int nfit, double* out,
                      cudaStream_t st) {
     count_launch();
@@ -2123,16 +2163,15 @@ void launch_scan64(const int32_t* list, int64_t n, const int32_t* uslot, const f
 }
 
 void launch_scan_resid(const int32_t* list, int64_t n, const int32_t* uslot, const float* d, const GridSpec& gs,
-                       int64_t G, int nfit, const float2* Wdf, double* part_v, int32_t* part_g, int nsp,
+                       int64_t G, int nfit, const float* Wdf, double* part_v, int32_t* part_g, int nsp,
                        int32_t* best, cudaStream_t st) {
     if (n <= 0) return;
-    const size_t smem = nfit <= kResolveMaxN ? (size_t)nfit * nfit * sizeof(float2) : 0;
+    const size_t smem = rows_smem(nfit);
     count_launch(2);
     const dim3 grid((unsigned)n, (unsigned)nsp);
-    if (gs.Sdf)
-        k_scan_resid<false><<<grid, 256, smem, st>>>(list, uslot, d, gs, G, nfit, Wdf, part_v, part_g);
-    else
-        k_scan_resid<true><<<grid, 256, smem, st>>>(list, uslot, d, gs, G, nfit, Wdf, part_v, part_g);
+    auto kern = gs.Sdf ? k_scan_resid<false> : k_scan_resid<true>;
+    allow_smem(kern, smem);
+    kern<<<grid, 32 * kRowsWarps, smem, st>>>(list, uslot, d, gs, G, nfit, Wdf, part_v, part_g);
     k_scan_resid_reduce<<<blocks_for(n), kThreads, 0, st>>>(list, n, nsp, part_v, part_g, best);
 }
 
@@ -2206,36 +2245,38 @@ void launch_resolve_list(const ResolveArgs& a, const int32_t* cand_count, int64_
     k_list_rows<<<blocks_for(n_tiles * kBM), kThreads, 0, st>>>(a.tile_univ, n_tiles * kBM, rows, n_rows_dev);
     count_launch();
     k_list_plan<<<blocks_for(n_rows), kThreads, 0, st>>>(a, cand_count, rows, n_rows, n_rows_dev, lp);
-    // eight warps a CTA, grid-stride over the chunks the plan reserved
-    const int64_t want = (lp.max_chunks + 7) / 8, cap = (int64_t)a.n_sm * 8;
+    // grid-stride over the chunks the plan reserved
+    const int64_t want = (lp.max_chunks + kRowsWarps - 1) / kRowsWarps, cap = (int64_t)a.n_sm * 8;
     count_launch();
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min(want, cap));
-    if (a.gs.Sdf)
-        k_list_chunks<false><<<grid, 256, 0, st>>>(a, cand_count, rows, lp);
-    else
-        k_list_chunks<true><<<grid, 256, 0, st>>>(a, cand_count, rows, lp);
+    const size_t smem = rows_smem(a.nfit);
+    auto kern = a.gs.Sdf ? k_list_chunks<false> : k_list_chunks<true>;
+    allow_smem(kern, smem);
+    kern<<<grid, 32 * kRowsWarps, smem, st>>>(a, cand_count, rows, lp);
 }
 
-void launch_resolve(const ResolveArgs& a, int64_t n_tiles, cudaStream_t st) {
+void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaStream_t st) {
     if (n_tiles <= 0) return;
     cudaMemsetAsync(a.counts, 0, 2 * sizeof(int32_t), st);
     // the tail loops over its device-side count
     const unsigned g3 = (unsigned)std::min<int64_t>(n_tiles, (int64_t)a.n_sm * 8);
-    const size_t smem = (a.nfit <= 64 ? (size_t)a.nfit * a.nfit : 0) * sizeof(float2);
+    // One thread per residual (k_resid_tiles) is the faster form when its lanes are full: at least a
+    // tile per SM and a quarter of the tile rows in use.  Below that a residual spread over a warp
+    // ends sooner, and above N_fit = 64 its vector does not fit a thread's registers.
+    const bool tiles = a.nfit <= 64 && a.gs.Sdf && n_tiles >= a.n_sm && 4 * n_rows >= n_tiles * kBM;
     auto resid = [&](const int2* items, const int2* tile_items, const int32_t* count, int64_t max_items, double* res) {
-        if (a.nfit > 64 || !a.gs.Sdf) {  // recomputed rows: the flat form for every N_fit
-            const int64_t want = (max_items + 255) / 256, cap = (int64_t)a.n_sm * 4;
+        if (!tiles) {
+            const int64_t per = kRowsWarps * kRowsB;
+            const int64_t want = (max_items + per - 1) / per, cap = (int64_t)a.n_sm * 8;
             const unsigned grid = (unsigned)std::max<int64_t>(1, std::min(want, cap));
-            if (a.gs.Sdf)
-                k_resid_flat<false><<<grid, 256, 0, st>>>(a, items, count, res);
-            else
-                k_resid_flat<true><<<grid, 256, 0, st>>>(a, items, count, res);
+            const size_t smem = rows_smem(a.nfit);
+            auto kern = a.gs.Sdf ? k_resid_rows<false> : k_resid_rows<true>;
+            allow_smem(kern, smem);
+            kern<<<grid, 32 * kRowsWarps, smem, st>>>(a, items, count, res);
             return;
         }
-        auto run = [&](auto kern) {
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 64 * (int)sizeof(float2));
-            kern<<<(unsigned)n_tiles, kResidThreads, smem, st>>>(a, items, tile_items, res);
-        };
+        const size_t smem = (size_t)df_blocks(a.nfit) * a.nfit * 8 * sizeof(float);
+        auto run = [&](auto kern) { kern<<<(unsigned)n_tiles, kResidThreads, smem, st>>>(a, items, tile_items, res); };
         if (a.nfit <= 16)
             run(k_resid_tiles<16>);
         else if (a.nfit <= 32)
@@ -2247,25 +2288,28 @@ void launch_resolve(const ResolveArgs& a, int64_t n_tiles, cudaStream_t st) {
     };
     count_launch(5);
     k_resolve_emit<<<(unsigned)n_tiles, kBM, 0, st>>>(a);
-    resid(a.items, a.tile_items, a.counts, n_tiles * kBM * (a.topk + 1), a.res);
+    resid(a.items, a.tile_items, a.counts, n_rows * (a.topk + 1), a.res);
     k_resolve_conclude<<<(unsigned)n_tiles, kBM, 0, st>>>(a);
-    resid(a.items2, a.tile_items2, a.counts + 1, n_tiles * kBM, a.res2);
+    resid(a.items2, a.tile_items2, a.counts + 1, n_rows, a.res2);
     k_resolve_tail<<<g3, 256, 0, st>>>(a);
 }
 
 void launch_finish(const int32_t* list, int64_t n, const int32_t* uslot, const int32_t* best, const UniverseState& us,
-                   const float* d, const GridSpec& gs, int nfit, const double* W64, const float2* Wdf, double* dchi2,
+                   const float* d, const GridSpec& gs, int nfit, const double* W64, const float* Wdf, double* dchi2,
                    double* chi2min, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();
     const unsigned grid = (unsigned)((n + 3) / 4);
-    if (gs.Sdf || !Wdf)
-        k_finish<false><<<grid, 128, 0, st>>>(list, n, uslot, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
-    else
-        k_finish<true><<<grid, 128, 0, st>>>(list, n, uslot, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
+    static_assert(kRowsWarps == 4, "a warp of k_finish has one warp's row storage");
+    const size_t smem = Wdf ? rows_smem(nfit) : 0;
+    auto kern = gs.Sdf || !Wdf ? k_finish<false> : k_finish<true>;
+    allow_smem(kern, smem);
+    kern<<<grid, 128, smem, st>>>(list, n, uslot, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
 }
 
-void launch_wdf(const double* W64, const int32_t* slots, int n, int nfit, float2* Wdf, cudaStream_t st) {
+size_t wdf_bytes(int nfit) { return (size_t)df_blocks(nfit) * nfit * 8 * sizeof(float); }
+
+void launch_wdf(const double* W64, const int32_t* slots, int n, int nfit, float* Wdf, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();
     k_wdf<<<n, 256, 0, st>>>(W64, slots, nfit, Wdf);

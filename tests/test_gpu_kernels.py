@@ -67,14 +67,16 @@ def test_split_screen_ties_take_the_lowest_index(ctx):
     fc.fc_unload_grid(ctx, gid)
 
 
-def test_split_fit_matches_unsplit_batch(ctx):
-    """A universe's result has the same bits alone (a split launch) and in a batch large enough to run unsplit."""
-    S, F = _grid(256 * 20, 45, 1)
+@pytest.mark.parametrize("n", [3, 15, 16, 17, 32, 45, 48, 50, 64, 67])
+def test_one_point_matches_the_batch(ctx, n):
+    """A universe's result has the same bits alone (a split screen, residuals spread over warps) and in a batch
+    large enough to run unsplit with one thread per residual (N <= 64)."""
+    S, F = _grid(256 * 20, n, 1)
     gid = fc.fc_load_grid(ctx, S)
     fc.fc_set_frac_cov(ctx, gid, F)
     ps = np.arange(0, len(S), 3, dtype=np.int64)
-    d, b, n = fc.fc_run_points(ctx, gid, ps, 7, 96)
+    d, b, ns = fc.fc_run_points(ctx, gid, ps, 7, 96)
     for k in (0, 500, len(ps) - 1):
         d1, b1, n1 = fc.fc_run_points(ctx, gid, ps[k:k + 1], 7, 96)
-        assert np.array_equal(d[k], d1[0]) and np.array_equal(b[k], b1[0]) and np.array_equal(n[k], n1[0])
+        assert np.array_equal(d[k], d1[0]) and np.array_equal(b[k], b1[0]) and np.array_equal(ns[k], n1[0])
     fc.fc_unload_grid(ctx, gid)
