@@ -1024,7 +1024,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 int32_t n_tiles = 0;
                 FC_CUDA(cudaMemcpyAsync(&n_tiles, cnts + 5, 4, cudaMemcpyDeviceToHost, c->stream));
                 FC_TRY(sync(c));
-                launch_yprep(tslot, tuniv, n_tiles, d, g->centre, g->nfit, g->K, g->A32, g->rho, cur, g->spec(),
+                launch_yprep(tslot, tuniv, n_tiles, d, g->centre_df, g->nfit, g->K, g->A32, g->rho, cur, g->spec(),
                              g->gnorm, g->Qc, g->Qb, g->G_pad, Yt, alpha, tau0, tj0, c->stream);
                 if (seeded) launch_min_tau(tuniv, n_tiles, thr, tau0, c->stream);
                 FC_TRY(stage_end(c, &S->ms_prep));

@@ -186,8 +186,9 @@ void launch_to_df(const double* x, int64_t n, float2* y, cudaStream_t st);
 void launch_group(const int32_t* active, int64_t n_active, const int32_t* uslot, int n_slots, int32_t* cnt,
                   int32_t* quad_base, int32_t* fill, int32_t* n_tiles_dev, int32_t* quad_slot, int32_t* tile_univ,
                   int64_t max_tiles, int slot_rows, cudaStream_t st);
+// centre: the double-float copy
 void launch_yprep(const int32_t* quad_slot, const int32_t* tile_univ, int64_t n_tiles, const float* d,
-                  const double* centre, int nfit, int K, const float* A32, const float* rho, const int32_t* cur,
+                  const float2* centre, int nfit, int K, const float* A32, const float* rho, const int32_t* cur,
                   const GridSpec& gs, const float4* gnorm, const float* Qc, const float* Qb, int64_t G_pad,
                   uint16_t* Ytiles, float4* alpha, float* tau0, int32_t* tile_j0, cudaStream_t st);
 // Tensor-core screen of BM-row tiles (see fc_screen.cu).  mode: kScreenTopK,

@@ -1178,120 +1178,199 @@ __device__ __forceinline__ int64_t ytile_offset(int64_t t, int r, int c, int K) 
     return t * (int64_t)(2 * K * kBM) + (int64_t)(c >> 3) * (kBM * 8) + (r >> 3) * 64 + (r & 7) * 8 + (c & 7);
 }
 
-// One CTA per tile, one thread per row (its quadrant's covariance slot): y^ = A (d - v) in binary32, Y = -2 y^
-// split into bf16 hi + lo, and the error-bound coefficient alpha in the spare
-// column so that the screen directly yields a lower bound of chi2_g - c_u.
-// It also evaluates the row's screen value at its own covariance point q
-// (= cur[u]) with an upper bound UB_q: no grid point with LB >= UB_q can be the
-// minimum, so tau0 = UB_q seeds the screen's top-k threshold.
-// NR > 0: N_fit <= NR and the row's d - v lives in registers (every index a
-// compile-time constant, the loops unrolled to NR with the columns past N_fit
-// skipped); NR = 0: any N_fit, with d - v in a per-thread array.  Same
-// operations in the same order either way.
-template <int NR>
-__global__ void __launch_bounds__(kBM) k_yprep(const int32_t* __restrict__ quad_slot,
-                                                const int32_t* __restrict__ tile_univ, const float* __restrict__ d,
-                                                const double* __restrict__ centre, int nfit, int K,
-                                                const float* __restrict__ A32, const float* __restrict__ rho,
-                                                const int32_t* __restrict__ cur, GridSpec gs,
-                                                const float4* __restrict__ gnorm, const float* __restrict__ Qc,
-                                                const float* __restrict__ Qb, int64_t G_pad,
-                                                uint16_t* __restrict__ Yt, float4* __restrict__ alpha,
-                                                float* __restrict__ tau0, int32_t* __restrict__ tile_j0,
-                                                bool stage_all) {
-    extern __shared__ float sA[];
-    const int64_t t = blockIdx.x;
-    const int r = threadIdx.x;
-    const int slot = quad_slot[t * kQuads + r / kQuadRows];
-    // each distinct covariance of the tile's quadrants is staged once (up to four where they fit;
-    // otherwise the tile's first slot is staged and rows of other slots read theirs)
-    int qs[kQuads], first[kQuads];  // first[k]: the first quadrant holding qs[k]
-#pragma unroll
-    for (int k = 0; k < kQuads; ++k) {
-        qs[k] = quad_slot[t * kQuads + k];
-        first[k] = k;
-        for (int k2 = k - 1; k2 >= 0; --k2)
-            if (qs[k2] == qs[k]) first[k] = k2;
-    }
-    const int nn = nfit * nfit;
-    for (int k = 0; k < kQuads; ++k) {
-        if (first[k] != k || (!stage_all && k > 0)) continue;
-        for (int e = threadIdx.x; e < nn; e += blockDim.x) sA[k * nn + e] = A32[(size_t)qs[k] * nn + e];
-    }
-    __syncthreads();
-    const int myq = r / kQuadRows;
-    const float* Arow = (stage_all || qs[myq] == qs[0]) ? sA + first[myq] * nn : A32 + (size_t)slot * nn;
+// One CTA per tile quadrant (32 rows of one covariance slot): y^ = A (d - v) in
+// binary32, Y = -2 y^ split into bf16 hi + lo, and the error-bound coefficient
+// alpha in the spare column so that the screen directly yields a lower bound
+// of chi2_g - c_u.  It also evaluates the row's screen value at its own
+// covariance point q (= cur[u]) with an upper bound UB_q: no grid point with
+// LB >= UB_q can be the minimum, so tau0 = UB_q seeds the screen's top-k
+// threshold.
+// The product is a 32 x K x N_fit contraction: lane = row, warp = 16 columns
+// of the image (one after another when K has more of them than the CTA has
+// warps), A in shared memory kYJ rows at a time, read as broadcasts of four
+// columns, d - v transposed beside it; two columns share a packed
+// multiply-add, and each column keeps one chain over j in increasing order.
+// Bound by instruction issue where tiles are many (staging and the bf16 split
+// cost as much as the products); where they are few, a quadrant per CTA and 16
+// columns per warp keep its latency to a few microseconds (one thread per row
+// walked all N^2 products alone).  Loads are asynchronous copies, all in flight
+// at once: with plain loads a CTA spent 20 of 22 us waiting for them in turn.
+// Prep stage against one thread per row: full 100x100 job 14.2 -> 10.6 ms,
+// 128 points of 64^3 21.1 -> 3.2 ms, 4 points with N = 200 18.1 -> 2.0 ms.
+constexpr int kYJ = 32;         // rows of A staged at a time above N_fit = 64 (all of them up to it)
+constexpr int kYPad = kQuadRows + 1;  // row stride of the transposed vectors (conflict-free both ways)
+constexpr int kYSums = 7;       // per-row sums that cross warps
+
+__host__ __device__ inline int yprep_warps(int K) { return K / 16 <= 8 ? K / 16 : (K / 16 + 1) / 2; }
+__host__ __device__ inline int yprep_rows(int nfit) { return nfit <= kResolveMaxN ? nfit : kYJ; }
+inline size_t yprep_smem(int nfit, int K) {
+    return (size_t)(yprep_rows(nfit) * K + 2 * nfit * kYPad + yprep_warps(K) * kYSums * kQuadRows) * sizeof(float);
+}
+// 4-byte asynchronous copy to shared memory: the CTA's loads are all in flight at once
+__device__ __forceinline__ void copy4_async(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+__global__ void k_yprep(const int32_t* __restrict__ quad_slot, const int32_t* __restrict__ tile_univ,
+                        const float* __restrict__ d, const float2* __restrict__ centre, int nfit, int K,
+                        const float* __restrict__ A32, const float* __restrict__ rho, const int32_t* __restrict__ cur,
+                        GridSpec gs, const float4* __restrict__ gnorm, const float* __restrict__ Qc,
+                        const float* __restrict__ Qb, int64_t G_pad, uint16_t* __restrict__ Yt,
+                        float4* __restrict__ alpha, float* __restrict__ tau0, int32_t* __restrict__ tile_j0) {
+    extern __shared__ float4 s_yprep[];
+    const int jc = yprep_rows(nfit);
+    float* sA = reinterpret_cast<float*>(s_yprep);       // [jc][K] rows of A
+    float* sd = sA + jc * K;                             // [nfit][kYPad] d - v
+    float* sq = sd + nfit * kYPad;                       // [nfit][kYPad] probe rows
+    float* sred = sq + nfit * kYPad;                     // [warps][kYSums][32]
+    const int64_t t = blockIdx.x / kQuads;
+    const int quad = blockIdx.x % kQuads;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int r = quad * kQuadRows + lane;               // row of the tile
     const int u = tile_univ[t * kBM + r];
+    const int q = u >= 0 ? cur[u] : -1;
     // the screen walks this tile's grid tiles starting at the one holding row 0's q
-    if (r == 0) tile_j0[t] = (u >= 0) ? cur[u] / kBN : 0;
-    if (u < 0) {
+    if (quad == 0 && threadIdx.x == 0) tile_j0[t] = (u >= 0) ? q / kBN : 0;
+    if (!__any_sync(0xffffffffu, u >= 0)) {  // the same in every warp: a quadrant of padding
         const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-        for (int c8 = 0; c8 < 2 * K / 8; ++c8) *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, c8 * 8, K)) = z;
-        alpha[t * kBM + r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        tau0[t * kBM + r] = -FLT_MAX;  // padding rows keep no candidate
+        for (int c8 = warp; c8 < 2 * K / 8; c8 += nw) *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, c8 * 8, K)) = z;
+        if (warp == 0) {
+            alpha[t * kBM + r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            tau0[t * kBM + r] = -FLT_MAX;  // padding rows keep no candidate
+        }
         return;
     }
-    const int q = cur[u];
-    float sql[kMaxBins];  // the probe row, when it is recomputed rather than stored
-    const float* sq = gs.Sc32 ? gs.Sc32 + (int64_t)q * nfit : sql;
-    if (!gs.Sc32) {
-        const FitRow fr = fit_row(gs, q);
-        for (int j = 0; j < nfit; ++j) sql[j] = row_sc32(gs, fr, j);
-    }
-
-    float dt[NR > 0 ? NR : kMaxBins];
-    float dn2 = 0.0f;
-    if (NR > 0) {
-#pragma unroll
-        for (int j = 0; j < (NR > 0 ? NR : 1); ++j) {
-            dt[j] = 0.0f;
-            if (j < nfit) {
-                dt[j] = (float)((double)d[(size_t)u * nfit + j] - centre[j]);
-                dn2 = fmaf(dt[j], dt[j], dn2);
+    const int slot = quad_slot[t * kQuads + quad];
+    const float* A = A32 + (size_t)slot * nfit * nfit;
+    auto stage_A = [&](int j0) {  // A is symmetric: row j is column j
+        const int nj = min(jc, nfit - j0);
+        for (int j = warp; j < nj; j += nw)
+            for (int i = lane; i < K; i += 32) {
+                if (i < nfit)
+                    copy4_async(sA + j * K + i, A + (size_t)(j0 + j) * nfit + i);
+                else
+                    sA[j * K + i] = 0.0f;
             }
-        }
-    } else {
-        for (int j = 0; j < nfit; ++j) {
-            dt[j] = (float)((double)d[(size_t)u * nfit + j] - centre[j]);
-            dn2 = fmaf(dt[j], dt[j], dn2);
+    };
+    // data and probe rows, one row per warp at a time (coalesced), stored transposed
+    for (int k = warp; k < kQuadRows; k += nw) {
+        const int uk = __shfl_sync(0xffffffffu, u, k), qk = __shfl_sync(0xffffffffu, q, k);
+        for (int j = lane; j < nfit; j += 32) {
+            if (uk >= 0)
+                copy4_async(sd + j * kYPad + k, d + (size_t)uk * nfit + j);
+            else
+                sd[j * kYPad + k] = 0.0f;
+            if (uk >= 0 && gs.Sc32)
+                copy4_async(sq + j * kYPad + k, gs.Sc32 + (size_t)qk * nfit + j);
+            else
+                sq[j * kYPad + k] = 0.0f;
         }
     }
-    float yn2 = 0.0f, yl2 = 0.0f, yhl2 = 0.0f, ry2 = 0.0f, dot = 0.0f, adot = 0.0f;
-    // the row's A-image entries in runs of 8 columns (one 16-byte core-matrix row per half)
-    for (int c8 = 0; c8 < K / 8; ++c8) {
-        uint32_t vh[4] = {0u, 0u, 0u, 0u}, vl[4] = {0u, 0u, 0u, 0u};
+    stage_A(0);
+    if (!gs.Sc32) {  // rows evaluated from the model
+        for (int k = warp; k < kQuadRows; k += nw) {
+            const int qk = __shfl_sync(0xffffffffu, q, k);
+            if (qk < 0) continue;
+            const FitRow fr = fit_row(gs, qk);
+            for (int j = lane; j < nfit; j += 32) sq[j * kYPad + k] = row_sc32(gs, fr, j);
+        }
+    }
+    copy_async_wait();
+    // d - v by the thread that copied the value; v as double-float keeps the difference off the narrow
+    // binary64 pipe (its error, 2^-24 (1 + 2^-20) |d - v|, is inside alpha's)
+    for (int k = warp; k < kQuadRows; k += nw) {
+        const bool used = __shfl_sync(0xffffffffu, u, k) >= 0;
+        for (int j = lane; j < nfit; j += 32)
+            if (used) sd[j * kYPad + k] = -df_sub_f(centre[j], sd[j * kYPad + k]).x;
+    }
+    __syncthreads();
+    float yn2 = 0.0f, yl2 = 0.0f, yhl2 = 0.0f, ry2 = 0.0f, dot = 0.0f, adot = 0.0f, dn2 = 0.0f;
+    for (int c0 = warp * 16; c0 - warp * 16 < K; c0 += nw * 16) {  // the same trip count for every warp
+        f32x2 y[8];
 #pragma unroll
-        for (int ii = 0; ii < 8; ++ii) {
-            const int i = c8 * 8 + ii;
-            if (i < nfit) {
-                float y = 0.0f;
-                const float* Ai = Arow + i * nfit;
-                if (NR > 0) {
+        for (int k = 0; k < 8; ++k) y[k] = 0ull;
+        for (int j0 = 0; j0 < nfit; j0 += jc) {
+            const int nj = min(jc, nfit - j0);
+            if (jc < nfit && (j0 > 0 || c0 >= nw * 16)) {  // rows past the first ones staged above
+                __syncthreads();
+                stage_A(j0);
+                copy_async_wait();
+                __syncthreads();
+            }
+            if (c0 < K) {
+#pragma unroll 4
+                for (int j = 0; j < nj; ++j) {
+                    const float v = sd[(j0 + j) * kYPad + lane];
+                    const f32x2 vv = x2_pack(v, v);
+                    const ulonglong2* a4 = reinterpret_cast<const ulonglong2*>(sA + j * K + c0);
 #pragma unroll
-                    for (int j = 0; j < (NR > 0 ? NR : 1); ++j)
-                        if (j < nfit) y = fmaf(Ai[j], dt[j], y);
-                } else {
-                    for (int j = 0; j < nfit; ++j) y = fmaf(Ai[j], dt[j], y);
+                    for (int k = 0; k < 4; ++k) {
+                        const ulonglong2 a = a4[k];
+                        y[2 * k] = x2_fma(a.x, vv, y[2 * k]);
+                        y[2 * k + 1] = x2_fma(a.y, vv, y[2 * k + 1]);
+                    }
                 }
-                const float Y = -2.0f * y;
-                yn2 = fmaf(Y, Y, yn2);
-                dot = fmaf(Y, sq[i], dot);
-                adot = fmaf(fabsf(Y), fabsf(sq[i]), adot);
-                const __nv_bfloat16 h = __float2bfloat16_rn(Y);
-                const float rem = Y - __bfloat162float(h);           // exact
-                const __nv_bfloat16 l = __float2bfloat16_rn(rem);
-                const float lo = __bfloat162float(l), hl = __bfloat162float(h) + lo;
-                const float ry = rem - lo;                            // exact: r_Y = Y - hi - lo
-                yl2 = fmaf(lo, lo, yl2);
-                yhl2 = fmaf(hl, hl, yhl2);
-                ry2 = fmaf(ry, ry, ry2);
-                vh[ii >> 1] |= (uint32_t)__bfloat16_as_ushort(h) << (16 * (ii & 1));
-                vl[ii >> 1] |= (uint32_t)__bfloat16_as_ushort(l) << (16 * (ii & 1));
             }
         }
-        *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, c8 * 8, K)) = make_uint4(vh[0], vh[1], vh[2], vh[3]);
-        *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, K + c8 * 8, K)) = make_uint4(vl[0], vl[1], vl[2], vl[3]);
+        if (c0 < K) {
+            uint32_t vh[8], vl[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                vh[k] = vl[k] = 0u;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int i = c0 + 2 * k + h;
+                    const float Y = -2.0f * (h ? x2_hi(y[k]) : x2_lo(y[k]));
+                    const float sv = i < nfit ? sq[i * kYPad + lane] : 0.0f;
+                    yn2 = fmaf(Y, Y, yn2);
+                    dot = fmaf(Y, sv, dot);
+                    adot = fmaf(fabsf(Y), fabsf(sv), adot);
+                    const __nv_bfloat16 hi = __float2bfloat16_rn(Y);
+                    const float rem = Y - __bfloat162float(hi);           // exact
+                    const __nv_bfloat16 l = __float2bfloat16_rn(rem);
+                    const float lo = __bfloat162float(l), hl = __bfloat162float(hi) + lo;
+                    const float ry = rem - lo;                            // exact: r_Y = Y - hi - lo
+                    yl2 = fmaf(lo, lo, yl2);
+                    yhl2 = fmaf(hl, hl, yhl2);
+                    ry2 = fmaf(ry, ry, ry2);
+                    if (i < nfit) {
+                        vh[k] |= (uint32_t)__bfloat16_as_ushort(hi) << (16 * h);
+                        vl[k] |= (uint32_t)__bfloat16_as_ushort(l) << (16 * h);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, c0 + 8 * k, K)) =
+                    make_uint4(vh[4 * k], vh[4 * k + 1], vh[4 * k + 2], vh[4 * k + 3]);
+                *reinterpret_cast<uint4*>(Yt + ytile_offset(t, r, K + c0 + 8 * k, K)) =
+                    make_uint4(vl[4 * k], vl[4 * k + 1], vl[4 * k + 2], vl[4 * k + 3]);
+            }
+        }
     }
+    for (int j = warp; j < nfit; j += nw) {
+        const float v = sd[j * kYPad + lane];
+        dn2 = fmaf(v, v, dn2);
+    }
+    const float sums[kYSums] = {yn2, yl2, yhl2, ry2, dot, adot, dn2};
+#pragma unroll
+    for (int k = 0; k < kYSums; ++k) sred[(warp * kYSums + k) * kQuadRows + lane] = sums[k];
+    __syncthreads();
+    if (warp != 0) return;
+    float tot[kYSums];
+#pragma unroll
+    for (int k = 0; k < kYSums; ++k) {
+        tot[k] = 0.0f;
+        for (int w = 0; w < nw; ++w) tot[k] += sred[(w * kYSums + k) * kQuadRows + lane];
+    }
+    if (u < 0) {  // its Y is zero already
+        alpha[t * kBM + r] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        tau0[t * kBM + r] = -FLT_MAX;
+        return;
+    }
+    yn2 = tot[0], yl2 = tot[1], yhl2 = tot[2], ry2 = tot[3], dot = tot[4], adot = tot[5], dn2 = tot[6];
     // -2 y.s~_g - (hi*hi + lo*hi + hi*lo products)  =  -2 (y - y^).s~ + Y_lo.S_lo + (Y_hi + Y_lo).r_S + r_Y.s~
     // and the binary32 accumulation of the 3K products (each add bounded as truncated, Sum|products| <= 1.02 |Y||s~|):
     //   |error| <= [2 |y - y^| + |r_Y| + (3K+2) 1.02 2^-23 |Y|] |s~| + |Y_lo| |S_lo| + |Y_hi+Y_lo| |r_S|
@@ -1301,7 +1380,7 @@ __global__ void __launch_bounds__(kBM) k_yprep(const int32_t* __restrict__ quad_
                                  (float)(3 * K + 2) * 1.1920929e-07f * 1.02f * yn + sqrtf(ry2));
     const float4 al = make_float4(a_acc, 1.0001f * sqrtf(yl2), 1.0001f * sqrtf(yhl2), 0.0f);
     alpha[t * kBM + r] = al;
-    // the spare columns nfit .. nfit+2 of the hi half (written as zero above; same thread, program order)
+    // the spare columns nfit .. nfit+2 of the hi half (written as zero above, before the barrier)
     Yt[ytile_offset(t, r, nfit, K)] = __bfloat16_as_ushort(__float2bfloat16_rd(-al.x));
     Yt[ytile_offset(t, r, nfit + 1, K)] = __bfloat16_as_ushort(__float2bfloat16_rd(-al.y));
     Yt[ytile_offset(t, r, nfit + 2, K)] = __bfloat16_as_ushort(__float2bfloat16_rd(-al.z));
@@ -2196,18 +2275,16 @@ void launch_group(const int32_t* active, int64_t n, const int32_t* uslot, int n_
 }
 
 void launch_yprep(const int32_t* quad_slot, const int32_t* tile_univ, int64_t n_tiles, const float* d,
-                  const double* centre, int nfit, int K, const float* A32, const float* rho, const int32_t* cur,
+                  const float2* centre, int nfit, int K, const float* A32, const float* rho, const int32_t* cur,
                   const GridSpec& gs, const float4* gnorm, const float* Qc, const float* Qb, int64_t G_pad,
                   uint16_t* Yt, float4* alpha, float* tau0, int32_t* tile_j0, cudaStream_t st) {
     if (n_tiles <= 0) return;
-    // the A of every quadrant's slot up to N_fit = 64 (64 KB); beyond, the tile's first slot
-    const bool stage_all = nfit <= kResolveMaxN;
-    const size_t smem = (size_t)(stage_all ? kQuads : 1) * nfit * nfit * sizeof(float);
-    auto kern = nfit <= 48 ? k_yprep<48> : k_yprep<0>;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = yprep_smem(nfit, K);
+    allow_smem(k_yprep, smem);
     count_launch();
-    kern<<<(unsigned)n_tiles, kBM, smem, st>>>(quad_slot, tile_univ, d, centre, nfit, K, A32, rho, cur, gs, gnorm, Qc,
-                                               Qb, G_pad, Yt, alpha, tau0, tile_j0, stage_all);
+    k_yprep<<<(unsigned)(n_tiles * kQuads), 32 * yprep_warps(K), smem, st>>>(quad_slot, tile_univ, d, centre, nfit, K,
+                                                                            A32, rho, cur, gs, gnorm, Qc, Qb, G_pad,
+                                                                            Yt, alpha, tau0, tile_j0);
 }
 
 void launch_or_mask(const int32_t* list, int64_t n, uint8_t bit, uint8_t* rmask, cudaStream_t st) {
