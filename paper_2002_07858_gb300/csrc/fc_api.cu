@@ -296,6 +296,18 @@ fc_status scratch(fc_ctx* c, const char* name, size_t count, T** out) {
     return FC_OK;
 }
 
+// The caller's array where a kernel can read it in place: memory of this context's device, aligned for
+// its elements (a misaligned or foreign array is copied instead).
+template <class T>
+bool readable_in_place(fc_ctx* c, const T* p) {
+    cudaPointerAttributes a;
+    if (((uintptr_t)p % alignof(T)) != 0 || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+
 fc_status copy_in(fc_ctx* c, void* dst, const void* src, size_t bytes) {
     const cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     FC_CUDA(cudaMemcpyAsync(dst, src, bytes, k, c->stream));
@@ -347,6 +359,19 @@ fc_status stage_end(fc_ctx* c, double* acc_ms) {
     float ms = 0.0f;
     FC_CUDA(cudaEventElapsedTime(&ms, c->ev_a, c->ev_b));
     *acc_ms += ms;
+    return FC_OK;
+}
+
+// x where launch_quantiles can read it: in place, or copied to scratch
+fc_status quantile_input(fc_ctx* c, const double* x, size_t count, const double** out) {
+    if (readable_in_place(c, x)) {
+        *out = x;
+        return FC_OK;
+    }
+    double* dx = nullptr;
+    FC_TRY(scratch(c, "qx", count, &dx));
+    FC_TRY(copy_in(c, dx, x, count * 8));
+    *out = dx;
     return FC_OK;
 }
 
@@ -2172,11 +2197,11 @@ fc_status fc_fc_region(fc_ctx* c, const double* dchi2_univ, int32_t P, int32_t U
     if (P == 0) return FC_OK;
     std::lock_guard<std::mutex> lk(c->api_mu);
     cudaSetDevice(c->device);
-    double *dx = nullptr, *dp = nullptr, *dout = nullptr;
-    FC_TRY(scratch(c, "qx", (size_t)P * U, &dx));
+    double *dp = nullptr, *dout = nullptr;
+    const double* dx = nullptr;
     FC_TRY(scratch(c, "qp", 1, &dp));
     FC_TRY(scratch(c, "qout", (size_t)P, &dout));
-    FC_TRY(copy_in(c, dx, dchi2_univ, (size_t)P * U * 8));
+    FC_TRY(quantile_input(c, dchi2_univ, (size_t)P * U, &dx));
     FC_CUDA(cudaMemcpyAsync(dp, &cl, 8, cudaMemcpyHostToDevice, c->stream));
     launch_quantiles(dx, P, U, dp, 1, dout, c->stream);
     std::vector<double> hc(P), hd(P);
@@ -2293,11 +2318,11 @@ fc_status fc_quantiles(fc_ctx* c, const double* x, int32_t rows, int32_t n, cons
     if (rows == 0) return FC_OK;
     std::lock_guard<std::mutex> lk(c->api_mu);
     cudaSetDevice(c->device);
-    double *dx = nullptr, *dp = nullptr, *dout = nullptr;
-    FC_TRY(scratch(c, "qx", (size_t)rows * n, &dx));
+    double *dp = nullptr, *dout = nullptr;
+    const double* dx = nullptr;
     FC_TRY(scratch(c, "qp", (size_t)nq, &dp));
     FC_TRY(scratch(c, "qout", (size_t)rows * nq, &dout));
-    FC_TRY(copy_in(c, dx, x, (size_t)rows * n * 8));
+    FC_TRY(quantile_input(c, x, (size_t)rows * n, &dx));
     FC_CUDA(cudaMemcpyAsync(dp, hp.data(), (size_t)nq * 8, cudaMemcpyHostToDevice, c->stream));
     launch_quantiles(dx, rows, n, dp, nq, dout, c->stream);
     FC_TRY(copy_out(c, out, dout, (size_t)rows * nq * 8));

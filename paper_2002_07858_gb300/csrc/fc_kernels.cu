@@ -1991,12 +1991,31 @@ __global__ void k_count_below(const double* __restrict__ x, int n, const double*
 }
 
 
-// One CTA per row: bitonic sort in shared memory, then numpy's "linear" rule.
-__global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, const double* __restrict__ probs,
-                            int nq, double* __restrict__ out) {
-    extern __shared__ double sx[];
-    const int row = blockIdx.x;
-    for (int i = threadIdx.x; i < npow2; i += blockDim.x) sx[i] = (i < n) ? x[(size_t)row * n + i] : DBL_MAX;
+// Order of binary64 values as unsigned integers (comparing integers keeps the
+// narrow binary64 pipe out of a sort); NaN sorts by its bits, -0 before +0.
+// It takes the bits, loaded as an integer: of a value that was a binary64
+// before, the compiler may set the sign by negating it, which a NaN ignores.
+__device__ __forceinline__ unsigned long long f64_key(unsigned long long b) {
+    return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double f64_of_key(unsigned long long k) {
+    return __longlong_as_double((long long)((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k));
+}
+
+// numpy's "linear" rule between two order statistics
+__device__ __forceinline__ void quantile_ranks(int n, double prob, int& lo, int& hi, double& f) {
+    const double h = (double)(n - 1) * prob;
+    lo = (int)floor(h);
+    if (lo < 0) lo = 0;
+    if (lo > n - 1) lo = n - 1;
+    hi = lo + 1 < n ? lo + 1 : n - 1;
+    f = h - lo;
+}
+
+// Whole row by a bitonic sort of its keys in shared memory (npow2 of them).
+__device__ void quantiles_by_sort(unsigned long long* key, int n, int npow2, const double* __restrict__ probs, int nq,
+                                  double* __restrict__ out) {
+    for (int i = n + threadIdx.x; i < npow2; i += blockDim.x) key[i] = ~0ull;
     __syncthreads();
     for (int k = 2; k <= npow2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
@@ -2004,10 +2023,10 @@ __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, cons
                 const int ixj = i ^ j;
                 if (ixj > i) {
                     const bool up = ((i & k) == 0);
-                    const double a = sx[i], b = sx[ixj];
+                    const unsigned long long a = key[i], b = key[ixj];
                     if ((a > b) == up) {
-                        sx[i] = b;
-                        sx[ixj] = a;
+                        key[i] = b;
+                        key[ixj] = a;
                     }
                 }
             }
@@ -2015,13 +2034,150 @@ __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, cons
         }
     }
     for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-        const double h = (double)(n - 1) * probs[q];
-        int lo = (int)floor(h);
-        if (lo < 0) lo = 0;
-        if (lo > n - 1) lo = n - 1;
-        const int hi = lo + 1 < n ? lo + 1 : n - 1;
-        const double f = h - lo;
-        out[(size_t)row * nq + q] = sx[lo] + f * (sx[hi] - sx[lo]);
+        int lo, hi;
+        double f;
+        quantile_ranks(n, probs[q], lo, hi, f);
+        const double a = f64_of_key(key[lo]), b = f64_of_key(key[hi]);
+        out[q] = a + f * (b - a);
+    }
+}
+
+// One CTA per row.  A few quantiles need a few order statistics, not a sorted
+// row: the values are counted into BINS buckets by a monotone function
+// (their binary32 rounding, linear between the row's extremes), the running
+// count finds the buckets that hold each quantile's two ranks, the values of
+// those buckets go to a short list, and their ranks in it are counted.  Rows
+// that this does not suit (a crowded bucket, infinities, NaN) and calls with
+// many quantiles sort the row.  Bound by shared memory (three passes over the
+// row and its counting atomics).  10000 rows of 1000 values, three quantiles:
+// 1.04 -> 0.13 ms a call (the sort compared on the binary64 pipe and its rows
+// were copied first).
+constexpr int kQuantSelect = 8;   // quantiles of a call that selects
+constexpr int kQuantList = 128;   // values of a quantile's list
+
+template <int BINS>
+__global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, const double* __restrict__ probs,
+                            int nq, double* __restrict__ out) {
+    extern __shared__ unsigned long long s_key[];  // [npow2], then the lists [min(nq, kQuantSelect)][kQuantList]
+    __shared__ int s_bin[BINS];
+    __shared__ int s_warp[16];
+    __shared__ float s_lo[16], s_hi[16];
+    __shared__ int s_b0[kQuantSelect], s_b1[kQuantSelect], s_before[kQuantSelect], s_n[kQuantSelect];
+    __shared__ double s_v[kQuantSelect][2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const unsigned long long* xr = reinterpret_cast<const unsigned long long*>(x) + (size_t)blockIdx.x * n;
+    double* o = out + (size_t)blockIdx.x * nq;
+    const bool select = nq <= kQuantSelect;
+    float lo = FLT_MAX, hi = -FLT_MAX;
+    bool odd = false;  // a value whose binary32 rounding is not an ordinary number
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const unsigned long long v = xr[i];
+        s_key[i] = f64_key(v);
+        const float f = (float)__longlong_as_double((long long)v);
+        odd = odd || !(fabsf(f) < 1.0e38f);
+        lo = fminf(lo, f);
+        hi = fmaxf(hi, f);
+    }
+    if (!select || __syncthreads_or(odd)) {
+        quantiles_by_sort(s_key, n, npow2, probs, nq, o);
+        return;
+    }
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, k));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, k));
+    }
+    if (lane == 0) {
+        s_lo[warp] = lo;
+        s_hi[warp] = hi;
+    }
+    for (int b = threadIdx.x; b < BINS; b += blockDim.x) s_bin[b] = 0;
+    if (threadIdx.x < kQuantSelect) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    for (int w = 0; w < nw; ++w) {
+        lo = fminf(lo, s_lo[w]);
+        hi = fmaxf(hi, s_hi[w]);
+    }
+    const float scale = hi > lo ? (float)BINS / (hi - lo) : 0.0f;
+    // monotone in the value, whatever the roundings
+    auto bin = [&](unsigned long long k) {
+        const float v = ((float)f64_of_key(k) - lo) * scale;
+        return v < (float)(BINS - 1) ? (int)v : BINS - 1;
+    };
+    for (int i = threadIdx.x; i < n; i += blockDim.x) atomicAdd(&s_bin[bin(s_key[i])], 1);
+    __syncthreads();
+    // running count up to and including each bucket
+    const int per = BINS / blockDim.x;
+    int sum = 0;
+    for (int k = 0; k < per; ++k) sum += s_bin[threadIdx.x * per + k];
+    int run = sum;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, run, k);
+        if (lane >= k) run += y;
+    }
+    if (lane == 31) s_warp[warp] = run;
+    __syncthreads();
+    run -= sum;
+    for (int w = 0; w < warp; ++w) run += s_warp[w];
+    for (int k = 0; k < per; ++k) {
+        run += s_bin[threadIdx.x * per + k];
+        s_bin[threadIdx.x * per + k] = run;
+    }
+    __syncthreads();
+    if (threadIdx.x < nq) {  // the buckets of ranks r0 and r1
+        int r0, r1;
+        double f;
+        quantile_ranks(n, probs[threadIdx.x], r0, r1, f);
+        auto find = [&](int r) {  // first bucket whose running count exceeds r
+            int a = 0, b = BINS - 1;
+            while (a < b) {
+                const int m = (a + b) >> 1;
+                if (s_bin[m] > r) b = m; else a = m + 1;
+            }
+            return a;
+        };
+        const int b0 = find(r0), b1 = find(r1);
+        s_b0[threadIdx.x] = b0;
+        s_b1[threadIdx.x] = b1;
+        s_before[threadIdx.x] = b0 ? s_bin[b0 - 1] : 0;
+    }
+    __syncthreads();
+    // the values of those buckets (the buckets between them are empty)
+    unsigned long long* list = s_key + npow2;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const unsigned long long k = s_key[i];
+        const int b = bin(k);
+        for (int q = 0; q < nq; ++q)
+            if (b >= s_b0[q] && b <= s_b1[q]) {
+                const int at = atomicAdd(&s_n[q], 1);
+                if (at < kQuantList) list[q * kQuantList + at] = k;
+            }
+    }
+    __syncthreads();
+    bool crowded = false;
+    for (int q = 0; q < nq; ++q) crowded = crowded || s_n[q] > kQuantList;
+    if (crowded) {  // the same for every thread
+        quantiles_by_sort(s_key, n, npow2, probs, nq, o);
+        return;
+    }
+    for (int q = warp; q < nq; q += nw) {
+        int r0, r1;
+        double f;
+        quantile_ranks(n, probs[q], r0, r1, f);
+        r0 -= s_before[q];
+        r1 -= s_before[q];
+        const int m = s_n[q];
+        const unsigned long long* l = list + q * kQuantList;
+        for (int e = lane; e < m; e += 32) {
+            const unsigned long long k = l[e];
+            int rank = 0;  // equal values take their places in list order
+            for (int j = 0; j < m; ++j) rank += (l[j] < k || (l[j] == k && j < e)) ? 1 : 0;
+            if (rank == r0) s_v[q][0] = f64_of_key(k);
+            if (rank == r1) s_v[q][1] = f64_of_key(k);
+        }
+        __syncwarp();
+        if (lane == 0) o[q] = s_v[q][0] + f * (s_v[q][1] - s_v[q][0]);
     }
 }
 
@@ -2425,13 +2581,17 @@ void launch_osc_spectra(const SpecModel& m, int64_t G, double* S, int* bad, cuda
     k_osc_spectra<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m, G, S, bad);
 }
 
-void launch_quantiles(double* x, int rows, int n, const double* probs, int nq, double* out, cudaStream_t st) {
+void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, cudaStream_t st) {
     int p2 = 1;
     while (p2 < n) p2 <<= 1;
-    const size_t smem = (size_t)p2 * sizeof(double);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_quantiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = ((size_t)p2 + (nq <= kQuantSelect ? nq * kQuantList : 0)) * sizeof(unsigned long long);
     count_launch();
-    k_quantiles<<<rows, 512, smem, st>>>(x, n, p2, probs, nq, out);
+    // short rows: small CTAs, many rows in flight; long rows (and a sort of many quantiles) a wide CTA,
+    // with as many buckets as keep a bucket of a smooth distribution below the list's length
+    const bool small = n <= 2048 && nq <= kQuantSelect;
+    auto kern = small ? k_quantiles<1024> : k_quantiles<4096>;
+    allow_smem(kern, smem);
+    kern<<<rows, small ? 128 : 512, smem, st>>>(x, n, p2, probs, nq, out);
 }
 
 }  // namespace fcdev

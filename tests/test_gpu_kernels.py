@@ -80,3 +80,56 @@ def test_one_point_matches_the_batch(ctx, n):
         d1, b1, n1 = fc.fc_run_points(ctx, gid, ps[k:k + 1], 7, 96)
         assert np.array_equal(d[k], d1[0]) and np.array_equal(b[k], b1[0]) and np.array_equal(ns[k], n1[0])
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- quantiles: selection, and the sort behind it --------------------------------------------
+
+def _quantile_rows(kind, rows, n, rng):
+    if kind == "chi2":
+        x = rng.chisquare(2, (rows, n))
+        return np.where(x < 0.2, 0.0, x)
+    if kind == "normal":
+        return rng.standard_normal((rows, n))
+    if kind == "ties":  # few distinct values: crowded buckets
+        return rng.integers(0, 3, (rows, n)).astype(np.float64)
+    if kind == "equal":
+        return np.full((rows, n), 1.25)
+    if kind == "outlier":  # everything but one value in one bucket
+        x = rng.random((rows, n))
+        x[:, n // 2] = 1e30
+        return x
+    if kind == "huge":  # beyond binary32
+        return rng.standard_normal((rows, n)) * 1e300
+    x = rng.chisquare(2, (rows, n))
+    x[:, ::7] = np.inf
+    x[0, 0] = -np.inf
+    return x
+
+
+@pytest.mark.parametrize("kind", ["chi2", "normal", "ties", "equal", "outlier", "huge", "inf"])
+@pytest.mark.parametrize("n", [1, 2, 31, 129, 1000, 2048, 2049, 16384])
+@pytest.mark.parametrize("nq", [1, 3, 8, 9])
+def test_quantiles(ctx, kind, n, nq):
+    import torch
+
+    x = _quantile_rows(kind, 3, n, np.random.default_rng(n * 10 + nq))
+    probs = np.linspace(0.0, 1.0, nq) if nq > 1 else np.array([0.9])
+    with np.errstate(invalid="ignore"):
+        s = np.sort(x, axis=1)
+        h = (n - 1) * probs
+        lo = np.floor(h).astype(int)
+        a, b = s[:, lo], s[:, np.minimum(lo + 1, n - 1)]
+        want = a + (h - lo) * (b - a)  # the rule itself: numpy's own function rounds its blend differently
+    # a blend of two values: a few roundings of the larger one
+    np.testing.assert_allclose(fc.fc_quantiles(ctx, x, probs), want, rtol=0, atol=4e-16 * np.max(np.abs(
+        np.where(np.isfinite(x), x, 0.0))))
+    dev = torch.from_numpy(x).cuda()
+    torch.cuda.synchronize()
+    assert np.array_equal(fc.fc_quantiles(ctx, dev, probs), fc.fc_quantiles(ctx, x, probs), equal_nan=True)
+
+
+def test_quantiles_with_nan_sorts_it_last(ctx):
+    x = np.random.default_rng(0).random((2, 100))
+    x[1, 5] = np.nan
+    q = fc.fc_quantiles(ctx, x, np.array([0.0, 0.5, 1.0]))
+    assert np.isfinite(q[0]).all() and np.isfinite(q[1, :2]).all() and np.isnan(q[1, 2])
