@@ -47,6 +47,9 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 
 // Default limit of a bounded wait (a context can shorten the screen's for tests).
 constexpr uint64_t kWaitNs = 2000000000ull;
+// Limit of a producer's wait for one of its own copies in flight before the CTA gives up (they land
+// within microseconds; a slot that another producer has filled since shows another phase).
+constexpr uint64_t kDrainNs = 100000000ull;
 
 // Bounded wait on a phase parity; false on timeout or when another role aborted.
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const volatile int* abort_flag,
@@ -67,6 +70,36 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const v
                                           uint64_t limit_ns = kWaitNs) {
     if (mbar_test(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, abort_flag, limit_ns);
+}
+
+// ---- roles that issue asynchronous work run as whole warps ----
+// tcgen05.mma, its commit and the bulk copies take their operands from uniform
+// registers.  Issued from a branch on one lane, their operands are moved there
+// one by one (about 110 cycles an MMA, 55 ns a bulk copy, more than a small MMA
+// takes); with the whole warp in the role and only the instruction under an
+// elected lane, descriptors and addresses are computed in uniform registers.
+
+// One lane of the converged warp, the same at every call from the same place.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t x;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.b32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(x));
+    return x != 0;
+}
+
+// x of lane 0: tells the compiler that a value is the same in every lane
+template <class T>
+__device__ __forceinline__ T uniform(T x) {
+    return __shfl_sync(0xffffffffu, x, 0);
+}
+
+// mbar_wait by every lane of the warp, one outcome for all
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const volatile int* abort_flag,
+                                          uint64_t limit_ns = kWaitNs) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit_ns));
 }
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {

@@ -133,3 +133,23 @@ def test_quantiles_with_nan_sorts_it_last(ctx):
     x[1, 5] = np.nan
     q = fc.fc_quantiles(ctx, x, np.array([0.0, 0.5, 1.0]))
     assert np.isfinite(q[0]).all() and np.isfinite(q[1, :2]).all() and np.isnan(q[1, 2])
+
+
+# ---- tensor-core q-vectors: triangular steps, slots interleaved in 16-row blocks -------------
+
+@pytest.mark.parametrize("n", [5, 13, 14, 29, 45, 61, 77, 93, 109, 125, 141, 157, 173, 189, 200])
+@pytest.mark.parametrize("n_pts", [1, 2, 7])
+def test_qvec_groups(ctx, n, n_pts):
+    """Every K, with whole and partial slot groups: the scan equals the plain one, and needs no fallback."""
+    S, F = _grid(700, n, 2)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    pts = np.linspace(3, 690, n_pts).astype(np.int64)
+    d, q = _data(S, pts, 12, n)
+    _same_scan(ctx, gid, d, q, 8)
+    tc = fc.fc_run_points(ctx, gid, pts, 3, 20)
+    assert fc.fc_get_stats(ctx)["fallback"] == 0
+    fc.fc_set_tuning(ctx, gid, qvec=fc.FC_QVEC_SIMT)
+    simt = fc.fc_run_points(ctx, gid, pts, 3, 20)
+    assert all(np.array_equal(a, b) for a, b in zip(tc, simt))
+    fc.fc_unload_grid(ctx, gid)
