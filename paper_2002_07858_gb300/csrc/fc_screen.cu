@@ -19,7 +19,8 @@
 // the strict "<" of Algorithm 1.  The U x G score matrix never leaves the SM.
 //
 // Roles (one CTA per SM, persistent over universe tiles):
-//   warp 0      bulk-async (TMA) copies: Y tile, then S~ tile + qb rows per stage
+//   warps 0, 10, 11  bulk-async (TMA) copies: Y tile (warp 0), then S~ tile + qb
+//               rows per stage, the three taking the stages in turn
 //   warp 1      TMEM allocation; one lane issues tcgen05.mma and commits
 //   warps 2..9  epilogue: two warps per TMEM lane quadrant, each owning half of
 //               the BN columns; tcgen05.ld double-buffered in registers, running
@@ -258,6 +259,15 @@ __global__ void k_min_seed(const uint16_t* __restrict__ Yt, const int32_t* __res
 
 constexpr int kTmemCols = 2 * kBN;  // two accumulator buffers
 constexpr int kEpiWarps = 8;
+// Copy producers, taking the stages in turn: a 16-column stage of two 8 KB
+// copies keeps one of them busy for 330 ns, its MMAs take 200 ns (67 ns in a
+// min pass).  With three the CTA has three warps on each scheduler, so the
+// registers a thread may use stay as they were with one.  Three producers and
+// whole-warp issue: screens of 128 points of 64^3 (K = 128) 144.6 -> 129.1 ms,
+// of the full 100x100 job (K = 48) 70.2 -> 67.2 ms, of 4 points of 16^6 (K = 80)
+// 26.5 -> 23.0 ms.
+constexpr int kProducers = 3;
+constexpr int kScreenThreads = 32 * (1 + kEpiWarps + kProducers);
 constexpr int kHalfCols = kBN / 2;
 constexpr uint32_t kAChunk = kBM * 16u;  // one 8-column slab of the A image
 constexpr uint32_t kBChunk = kBN * 16u;  // one 8-column slab of the B image
@@ -323,7 +333,7 @@ struct SplitArgs {
 };
 
 template <int TOPK, int MODE, bool KCHUNK>
-__global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
+__global__ void __launch_bounds__(kScreenThreads, 1)
     k_screen(const uint16_t* __restrict__ Yt, const uint16_t* __restrict__ Bt, const uint16_t* __restrict__ Qb3,
              const int32_t* __restrict__ quad_slot, float* __restrict__ tau0, const int32_t* __restrict__ tile_j0,
              int64_t n_tiles, int64_t G, int64_t G_pad, float* __restrict__ cand_val, int32_t* __restrict__ cand_idx,
@@ -348,7 +358,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
     constexpr bool kLo = (MODE != kModeMin);
     const uint32_t tile_elems = 2u * K * kBN;  // bf16 elements of one B tile
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     // constant q-step operand slabs (generic-proxy writes, fenced for the tensor core below)
     {
         uint32_t* ones = (uint32_t*)(smem + lay.off_ones);
@@ -392,7 +402,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = uniform(*tmem_holder);
     const int n_gt = (int)(G_pad / kBN);
     const bool split = sp.parts > 1;
     const int64_t n_items = n_tiles * sp.parts;
@@ -403,19 +413,25 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
         item = w - (int64_t)part * n_tiles;
         lo = part * sp.len;
         hi = lo + sp.len < n_gt ? lo + sp.len : n_gt;
-        const int j0 = ((tile_j0[item] % n_gt) + n_gt) % n_gt;
+        const int j0 = uniform(((tile_j0[item] % n_gt) + n_gt) % n_gt);
         j = (j0 >= lo && j0 < hi) ? j0 : lo;
     };
     // limit of the pipeline waits (the drain and completion waits keep the built-in limit)
     const uint64_t wlim = wt.wait_ns ? wt.wait_ns : kWaitNs;
 
-    if (warp == 0 && lane == 0) {
-        // ---------------------------------------------------------- producer
-        int y_par[2] = {-1, -1};
-        int b_par[16];
-        for (int s = 0; s < STAGES; ++s) b_par[s] = -1;
+    // warp 0 and the warps after the epilogue's are producers 0, 1, ...
+    // At most as many as there are stages: a producer that has filled stage n knows stage n - STAGES
+    // consumed, and its next wait, for stage n + producers, tells phases apart by their parity only if
+    // the use before the slot's last one is consumed too.
+    const int n_prod = min(kProducers, STAGES);
+    const int prod = warp == 0 ? 0 : warp - (1 + kEpiWarps);
+    if ((warp == 0 || warp >= 2 + kEpiWarps) && prod < n_prod) {
+        // --------------------------------------------------------- producers
+        const bool leader = elect_one();
+        int turn = 0;  // whose stage the next one is
+        uint32_t y_used = 0, y_phase = 0, used = 0, phase = 0;  // slots filled, and the phase of the last fill
         bool ok = true, stopped = false;
-        int64_t issued = 0;  // pipeline stages issued (for the test hook wt.stop_after)
+        int64_t issued = 0;  // pipeline stages so far, every producer's (for the test hook wt.stop_after)
         // ring positions and phases advance by counting (no division in the issue loop)
         int yb = 0, s = 0;
         uint32_t yph = 0, ph = 0;
@@ -423,146 +439,182 @@ __global__ void __launch_bounds__(64 + 32 * kEpiWarps, 1)
             int64_t item;
             int lo, hi, j;
             item_of(w, item, lo, hi, j);
-            if (!mbar_wait(bar(Y_EMPTY + yb), yph ^ 1, abort_flag, wlim)) { ok = false; break; }
-            mbar_expect_tx(bar(Y_FULL + yb), lay.y_bytes);
-            bulk_g2s(sbase + yb * lay.y_bytes, Yt + item * (int64_t)(lay.y_bytes / 2), lay.y_bytes,
-                     bar(Y_FULL + yb));
-            y_par[yb] = (int)yph;
-            if (++yb == YBUF) { yb = 0; yph ^= 1u; }
-            const int32_t* qs = quad_slot + item * kQuads;
-            const bool mixed = qs[1] != qs[0] || qs[2] != qs[0] || qs[3] != qs[0];
-            const uint16_t* qrow = Qb3 + (int64_t)qs[0] * G_pad * 8;
+            if (prod == 0) {
+                if (!warp_wait(bar(Y_EMPTY + yb), yph ^ 1, abort_flag, wlim)) { ok = false; break; }
+                if (leader) {
+                    mbar_expect_tx(bar(Y_FULL + yb), lay.y_bytes);
+                    bulk_g2s(sbase + yb * lay.y_bytes, Yt + item * (int64_t)(lay.y_bytes / 2), lay.y_bytes,
+                             bar(Y_FULL + yb));
+                }
+                __syncwarp();
+                y_used |= 1u << yb;
+                y_phase = (y_phase & ~(1u << yb)) | (yph << yb);
+                if (++yb == YBUF) { yb = 0; yph ^= 1u; }
+            }
+            const int32_t* qsp = quad_slot + item * kQuads;
+            const int q0 = uniform(qsp[0]), q1 = uniform(qsp[1]), q2 = uniform(qsp[2]), q3 = uniform(qsp[3]);
+            const bool mixed = q1 != q0 || q2 != q0 || q3 != q0;
+            const int64_t qld = G_pad * 8;  // q-step elements of a slot
             for (int jj = lo; ok && !stopped && jj < hi; ++jj) {
                 const uint16_t* btile = Bt + (int64_t)j * tile_elems;
+                const uint16_t* qtile = Qb3 + (int64_t)j * kBN * 8;
                 if (mixed) {
                     // an extra stage: the q-step slabs of the four quadrants' slots, side by side
                     if (wt.stop_after >= 0 && issued >= wt.stop_after) { stopped = true; break; }
                     ++issued;
-                    if (!mbar_wait(bar(B_EMPTY + s), ph ^ 1, abort_flag, wlim)) { ok = false; break; }
-                    const uint32_t st0 = sbase + lay.off_b + s * lay.stage_bytes;
-                    mbar_expect_tx(bar(B_FULL + s), kQuads * kQBytes);
-                    for (int k = 0; k < kQuads; ++k)
-                        bulk_g2s(st0 + k * kQBytes, Qb3 + ((int64_t)qs[k] * G_pad + (int64_t)j * kBN) * 8, kQBytes,
-                                 bar(B_FULL + s));
-                    b_par[s] = (int)ph;
+                    const bool mine = turn == prod;
+                    if (++turn == n_prod) turn = 0;
+                    if (mine) {
+                        if (!warp_wait(bar(B_EMPTY + s), ph ^ 1, abort_flag, wlim)) { ok = false; break; }
+                        if (leader) {
+                            const uint32_t st0 = sbase + lay.off_b + s * lay.stage_bytes, full = bar(B_FULL + s);
+                            mbar_expect_tx(full, kQuads * kQBytes);
+                            bulk_g2s(st0, qtile + q0 * qld, kQBytes, full);
+                            bulk_g2s(st0 + kQBytes, qtile + q1 * qld, kQBytes, full);
+                            bulk_g2s(st0 + 2 * kQBytes, qtile + q2 * qld, kQBytes, full);
+                            bulk_g2s(st0 + 3 * kQBytes, qtile + q3 * qld, kQBytes, full);
+                        }
+                        __syncwarp();
+                        used |= 1u << s;
+                        phase = (phase & ~(1u << s)) | (ph << s);
+                    }
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
                 for (int c = 0; c < NC; ++c) {
                     if (wt.stop_after >= 0 && issued >= wt.stop_after) { stopped = true; break; }
                     ++issued;
-                    if (!mbar_wait(bar(B_EMPTY + s), ph ^ 1, abort_flag, wlim)) { ok = false; break; }
-                    const uint32_t st0 = sbase + lay.off_b + s * lay.stage_bytes;
-                    const uint32_t hi_bytes = KCHUNK ? 2u * kBChunk : lay.bpart_bytes / 2u;
-                    const uint32_t bytes = (kLo ? 2u * hi_bytes : hi_bytes) + (c == 0 && !mixed ? kQBytes : 0u);
-                    mbar_expect_tx(bar(B_FULL + s), bytes);
-                    if (KCHUNK) {
-                        // hi slabs 2c, 2c+1 and lo slabs K/8 + 2c, K/8 + 2c + 1 of the tile
-                        bulk_g2s(st0, btile + (int64_t)(2 * c) * (kBChunk / 2), hi_bytes, bar(B_FULL + s));
-                        if (kLo)
-                            bulk_g2s(st0 + hi_bytes, btile + (int64_t)(K / 8 + 2 * c) * (kBChunk / 2), hi_bytes,
-                                     bar(B_FULL + s));
-                    } else {
-                        bulk_g2s(st0, btile, kLo ? lay.bpart_bytes : hi_bytes, bar(B_FULL + s));
+                    const bool mine = turn == prod;
+                    if (++turn == n_prod) turn = 0;
+                    if (mine) {
+                        if (!warp_wait(bar(B_EMPTY + s), ph ^ 1, abort_flag, wlim)) { ok = false; break; }
+                        if (leader) {
+                            const uint32_t st0 = sbase + lay.off_b + s * lay.stage_bytes, full = bar(B_FULL + s);
+                            const uint32_t hi_bytes = KCHUNK ? 2u * kBChunk : lay.bpart_bytes / 2u;
+                            mbar_expect_tx(full, (kLo ? 2u * hi_bytes : hi_bytes) + (c == 0 && !mixed ? kQBytes : 0u));
+                            if (KCHUNK) {
+                                // hi slabs 2c, 2c+1 and lo slabs K/8 + 2c, K/8 + 2c + 1 of the tile
+                                bulk_g2s(st0, btile + (int64_t)(2 * c) * (kBChunk / 2), hi_bytes, full);
+                                if (kLo)
+                                    bulk_g2s(st0 + hi_bytes, btile + (int64_t)(K / 8 + 2 * c) * (kBChunk / 2),
+                                             hi_bytes, full);
+                            } else {
+                                bulk_g2s(st0, btile, kLo ? lay.bpart_bytes : hi_bytes, full);
+                            }
+                            if (c == 0 && !mixed) bulk_g2s(st0 + lay.bpart_bytes, qtile + q0 * qld, kQBytes, full);
+                        }
+                        __syncwarp();
+                        used |= 1u << s;
+                        phase = (phase & ~(1u << s)) | (ph << s);
                     }
-                    if (c == 0 && !mixed)
-                        bulk_g2s(st0 + lay.bpart_bytes, qrow + (int64_t)j * kBN * 8, kQBytes, bar(B_FULL + s));
-                    b_par[s] = (int)ph;
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
                 if (++j == hi) j = lo;
             }
         }
-        if (!ok) {
+        if (!ok && lane == 0) {
             *abort_flag = 1;
             atomicOr(status, kDevTimeout);
         }
         if (!ok || stopped) {
-            // let every copy this thread issued land before the CTA can exit (the consumers of a
+            // let every copy this warp issued land before the CTA can exit (the consumers of a
             // stopped producer time out on the stages that never come)
             for (int i = 0; i < YBUF; ++i)
-                if (y_par[i] >= 0) mbar_wait(bar(Y_FULL + i), (uint32_t)y_par[i], nullptr);
+                if ((y_used >> i) & 1u) mbar_wait(bar(Y_FULL + i), (y_phase >> i) & 1u, nullptr);
             for (int s = 0; s < STAGES; ++s)
-                if (b_par[s] >= 0) mbar_wait(bar(B_FULL + s), (uint32_t)b_par[s], nullptr);
+                if ((used >> s) & 1u) mbar_wait(bar(B_FULL + s), (phase >> s) & 1u, nullptr, kDrainNs);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // --------------------------------------------------------------- MMA
+        const bool leader = elect_one();
         bool ok = true;
         const uint64_t a_q = smem_desc(sbase + lay.off_ones, lay.off_zero - lay.off_ones, 128);
         // selector pairs of a mixed tile: quadrants 0 and 1 in K columns 0-7 and 8-15, then 2 and 3
         const uint64_t a_s01 = smem_desc(sbase + lay.off_sel, kAChunk, 128);
         const uint64_t a_s23 = smem_desc(sbase + lay.off_sel + 2 * kAChunk, kAChunk, 128);
+        // low words of the image descriptors (the high word, row-group stride and version, is common): the
+        // first K step's, advanced by two slabs a step
+        const uint64_t dhi = smem_desc(0, 0, 128) & 0xffffffff00000000ull;
+        constexpr uint32_t kALbo = (kAChunk >> 4) << 16, kBLbo = (kBChunk >> 4) << 16;
+        constexpr uint32_t kAStep = (2 * kAChunk) >> 4, kBStep = (2 * kBChunk) >> 4;
+        const uint32_t a_lo_off = ((K / 8) * kAChunk) >> 4,
+                       b_lo_off = (KCHUNK ? 2 * kBChunk : (K / 8) * kBChunk) >> 4;
+        const uint32_t b_first = ((sbase + lay.off_b) >> 4) | kBLbo, b_stage = lay.stage_bytes >> 4;
         int yb = 0, s = 0, ab = 0;
         uint32_t yph = 0, ph = 0, aph = 0;
         for (int64_t w = blockIdx.x; ok && w < n_items; w += gridDim.x) {
             int64_t item;
             int lo, hi, j;
             item_of(w, item, lo, hi, j);
-            if (!mbar_wait(bar(Y_FULL + yb), yph, abort_flag, wlim)) { ok = false; break; }
+            if (!warp_wait(bar(Y_FULL + yb), yph, abort_flag, wlim)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t a0 = sbase + yb * lay.y_bytes;
-            const int32_t* qs = quad_slot + item * kQuads;
-            const bool mixed = qs[1] != qs[0] || qs[2] != qs[0] || qs[3] != qs[0];
+            const uint32_t a_first = ((sbase + yb * lay.y_bytes) >> 4) | kALbo;
+            const int32_t* qsp = quad_slot + item * kQuads;
+            const int q0 = uniform(qsp[0]), q1 = uniform(qsp[1]), q2 = uniform(qsp[2]), q3 = uniform(qsp[3]);
+            const bool mixed = q1 != q0 || q2 != q0 || q3 != q0;
             for (int jj = lo; ok && jj < hi; ++jj) {
-                if (!mbar_wait(bar(T_EMPTY + ab), aph ^ 1, abort_flag, wlim)) { ok = false; break; }
+                if (!warp_wait(bar(T_EMPTY + ab), aph ^ 1, abort_flag, wlim)) { ok = false; break; }
                 const uint32_t d = tmem_base + (uint32_t)(ab * kBN);
                 if (mixed) {
                     // q-step stage: accumulator <- q_g of each row's own covariance (two selector MMAs;
                     // a row takes its quadrant's slab and exact zeros from the other three)
-                    if (!mbar_wait(bar(B_FULL + s), ph, abort_flag, wlim)) { ok = false; break; }
+                    if (!warp_wait(bar(B_FULL + s), ph, abort_flag, wlim)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t q0 = sbase + lay.off_b + s * lay.stage_bytes;
-                    mma_bf16(d, a_s01, smem_desc(q0, kQBytes, 128), kIdesc, 0u);
-                    mma_bf16(d, a_s23, smem_desc(q0 + 2 * kQBytes, kQBytes, 128), kIdesc, 1u);
-                    mma_commit(bar(B_EMPTY + s));
+                    if (leader) {
+                        const uint32_t qa = sbase + lay.off_b + s * lay.stage_bytes;
+                        mma_bf16(d, a_s01, smem_desc(qa, kQBytes, 128), kIdesc, 0u);
+                        mma_bf16(d, a_s23, smem_desc(qa + 2 * kQBytes, kQBytes, 128), kIdesc, 1u);
+                        mma_commit(bar(B_EMPTY + s));
+                    }
+                    __syncwarp();
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
+                uint32_t ak = a_first;
                 for (int c = 0; c < NC; ++c) {
-                    if (!mbar_wait(bar(B_FULL + s), ph, abort_flag, wlim)) { ok = false; break; }
+                    if (!warp_wait(bar(B_FULL + s), ph, abort_flag, wlim)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t b0 = sbase + lay.off_b + s * lay.stage_bytes;
-                    if (c == 0 && !mixed) {
+                    if (leader && c == 0 && !mixed) {
                         // q-step: accumulator <- qb_g
                         const uint32_t qoff = lay.off_b + s * lay.stage_bytes + lay.bpart_bytes;
                         mma_bf16(d, a_q, smem_desc(sbase + qoff, lay.off_zero - qoff, 128), kIdesc, 0u);
                     }
-                    // descriptors of the first K step; a step of 16 columns moves the start address by
-                    // two slabs, i.e. adds (2 slab bytes) >> 4 to the descriptor's address field
-                    const int k_lo = KCHUNK ? c : 0, k_hi = KCHUNK ? c + 1 : K / 16;
-                    uint64_t a_hi = smem_desc(a0 + (2 * k_lo) * kAChunk, kAChunk, 128);
-                    uint64_t a_lo = smem_desc(a0 + (K / 8 + 2 * k_lo) * kAChunk, kAChunk, 128);
-                    uint64_t b_hi = smem_desc(KCHUNK ? b0 : b0 + (2 * k_lo) * kBChunk, kBChunk, 128);
-                    uint64_t b_lo = smem_desc(KCHUNK ? b0 + 2 * kBChunk : b0 + (K / 8 + 2 * k_lo) * kBChunk,
-                                              kBChunk, 128);
-                    constexpr uint64_t kAStep = (2 * kAChunk) >> 4, kBStep = (2 * kBChunk) >> 4;
+                    uint32_t bk = b_first + (uint32_t)s * b_stage;
+                    const int steps = KCHUNK ? 1 : K / 16;
 #pragma unroll 4
-                    for (int kk = k_lo; kk < k_hi; ++kk) {
-                        mma_bf16(d, a_hi, b_hi, kIdesc, 1u);
-                        if (kLo) {
-                            mma_bf16(d, a_lo, b_hi, kIdesc, 1u);
-                            mma_bf16(d, a_hi, b_lo, kIdesc, 1u);
+                    for (int k = 0; k < steps; ++k) {
+                        if (leader) {
+                            mma_bf16(d, dhi | ak, dhi | bk, kIdesc, 1u);
+                            if (kLo) {
+                                mma_bf16(d, dhi | (ak + a_lo_off), dhi | bk, kIdesc, 1u);
+                                mma_bf16(d, dhi | ak, dhi | (bk + b_lo_off), kIdesc, 1u);
+                            }
                         }
-                        a_hi += kAStep;
-                        a_lo += kAStep;
-                        b_hi += kBStep;
-                        b_lo += kBStep;
+                        ak += kAStep;
+                        bk += kBStep;
                     }
-                    mma_commit(bar(B_EMPTY + s));
+                    if (leader) mma_commit(bar(B_EMPTY + s));
+                    __syncwarp();
                     if (++s == STAGES) { s = 0; ph ^= 1u; }
                 }
-                if (ok) mma_commit(bar(T_FULL + ab));
+                if (ok && leader) mma_commit(bar(T_FULL + ab));
+                __syncwarp();
                 if (++ab == 2) { ab = 0; aph ^= 1u; }
             }
-            if (ok) mma_commit(bar(Y_EMPTY + yb));
+            if (ok && leader) mma_commit(bar(Y_EMPTY + yb));
+            __syncwarp();
             if (++yb == YBUF) { yb = 0; yph ^= 1u; }
         }
-        if (!ok) {
+        if (!ok && lane == 0) {
             *abort_flag = 1;
             atomicOr(status, kDevTimeout);
         }
+        __syncwarp();
         // every MMA issued above has completed once DONE flips
-        mma_commit(bar(DONE));
-        mbar_wait(bar(DONE), 0, nullptr);
-    } else if (warp >= 2) {
+        if (leader) {
+            mma_commit(bar(DONE));
+            mbar_wait(bar(DONE), 0, nullptr);
+        }
+        __syncwarp();
+    } else if (warp >= 2 && warp < 2 + kEpiWarps) {
         // ---------------------------------------------------------- epilogue
         const int quad = warp & 3;           // TMEM lane quadrant this warp may access
         const int half = (warp - 2) >> 2;    // which half of the BN columns
@@ -808,7 +860,7 @@ void run_screen(const ScreenLayout& lay, const uint16_t* Yt, const uint16_t* Bt,
     if (split && MODE == kModeMin) cudaMemsetAsync(ss.key, 0xff, (size_t)rows * 8, st);
     if (split && MODE == kModeList) cudaMemsetAsync(cc, 0, (size_t)rows * 2 * sizeof(int32_t), st);
     count_launch();
-    kern<<<(unsigned)grid, 64 + 32 * kEpiWarps, lay.bytes, st>>>(Yt, Bt, Qb3, quad_slot, tau0, tile_j0, n_tiles, G,
+    kern<<<(unsigned)grid, kScreenThreads, lay.bytes, st>>>(Yt, Bt, Qb3, quad_slot, tau0, tile_j0, n_tiles, G,
                                                                    G_pad, ov, oi, cc, status, pa, lay, la, wt, sp);
     if (MODE == kModeMin) {
         count_launch();
