@@ -972,9 +972,16 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
             launch_lookup_slots(list, cnt, cur, g->slot_of, fslot, c->stream);
         }
         if (!mixed) {
+            int nsp = scan64_splits(cnt, g->G, c->n_sm);
+            double *pv = nullptr, *py = nullptr;
+            int32_t* pg = nullptr;
+            if (nsp > 1 && (scratch(c, "fb_y", (size_t)cnt * g->nfit, &py) != FC_OK ||
+                            scratch(c, "fb_pv", (size_t)cnt * nsp, &pv) != FC_OK ||
+                            scratch(c, "fb_pg", (size_t)cnt * nsp, &pg) != FC_OK))
+                nsp = 1;  // no room for the partial minima
             stage_begin(c);
-            launch_scan64(list, cnt, fslot, d, g->spec(), g->G, g->nfit, g->A64, g->Q64, g->G, L->best,
-                          c->stream);
+            launch_scan64(list, cnt, fslot, d, g->spec(), g->G, g->nfit, g->A64, g->Q64, g->G, L->best, nsp, py, pv,
+                          pg, c->stream);
             FC_TRY(stage_end(c, &S->ms_scan64));
         }
         launch_or_mask(list, cnt, mixed ? kDecidedScan : kDecidedPlain, L->rmask, c->stream);

@@ -168,7 +168,10 @@ void launch_set_slots(const int32_t* q_list, const int32_t* slot_list, int n, in
 // ---- plain binary64 scan ----
 void launch_scan64(const int32_t* list, int64_t n, const int32_t* uslot_of_list, const float* d,
                    const GridSpec& gs, int64_t G, int nfit, const double* A64,
-                   const double* Q64, int64_t ldq, int32_t* best, cudaStream_t st);
+                   const double* Q64, int64_t ldq, int32_t* best, int nsp, double* y, double* part_v,
+                   int32_t* part_g, cudaStream_t st);
+// its split over the grid (nsp; 1: none); y [n * nfit] and part_v / part_g [n * nsp] when split
+int scan64_splits(int64_t n, int64_t G, int n_sm);
 
 // exact residual-form scan of the mixed path (double-float, split over nsp CTAs per universe)
 void launch_scan_resid(const int32_t* list, int64_t n, const int32_t* uslot, const float* d, const GridSpec& gs,

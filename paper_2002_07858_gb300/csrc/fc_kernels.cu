@@ -890,21 +890,43 @@ __global__ void k_set_slots(const int32_t* __restrict__ q, const int32_t* __rest
 // grid points are a small dense contraction on the FP64 pipe: y and a tile of
 // s~ (transposed to [j][g]) sit in shared memory and every thread keeps a 4 x 2
 // block of dot products in registers (the binary64 pipe is narrow, so operand
-// loads are never the limit; 16 universes per CTA keep enough CTAs for the
-// later scans, which hold fewer universes).  Every dot product is one fma chain
-// over j in increasing order, as in a per-pair loop, so the minimum found does
-// not depend on the blocking.
+// loads are never the limit).  Every dot product is one fma chain over j in
+// increasing order, as in a per-pair loop, so the minimum found does not depend
+// on the blocking.  Grid (16 universes, split): few universes leave SMs idle,
+// so the grid's tiles are then dealt to gridDim.y CTAs, which read y (k_y64)
+// and write their minima for k_scan_resid_reduce.  One point of 25x25 x 1000
+// universes: 2.00 ms a job unsplit, 1.54 ms split with every CTA forming y.
 constexpr int kS64U = 16;   // universes per CTA
 constexpr int kS64G = 64;   // grid points per staged tile
 constexpr int kS64LdS = kS64G + 2;  // row stride of the staged tile (fewer bank conflicts, 16-byte rows)
 constexpr int kS64Threads = 128;
+
+// y = A (d - v) of each universe in list order, each component one fma chain
+// over j in increasing order (A is symmetric: its columns are read, coalesced)
+__global__ void __launch_bounds__(64) k_y64(const int32_t* __restrict__ list, const int32_t* __restrict__ uslot,
+                                            const float* __restrict__ d, const double* __restrict__ centre, int nfit,
+                                            const double* __restrict__ A64, double* __restrict__ y) {
+    __shared__ double sd[kMaxBins];
+    const int64_t i = blockIdx.x;
+    const float* du = d + (size_t)list[i] * nfit;
+    for (int j = threadIdx.x; j < nfit; j += blockDim.x) sd[j] = (double)du[j] - centre[j];
+    __syncthreads();
+    const double* A = A64 + (size_t)uslot[i] * nfit * nfit;
+    for (int r = threadIdx.x; r < nfit; r += blockDim.x) {
+        double t = 0.0;
+#pragma unroll 4
+        for (int j = 0; j < nfit; ++j) t = fma(A[(size_t)j * nfit + r], sd[j], t);
+        y[i * nfit + r] = t;
+    }
+}
 
 __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restrict__ list, int64_t n,
                                                          const int32_t* __restrict__ uslot,
                                                          const float* __restrict__ d, GridSpec gs, int64_t G,
                                                          int nfit, const double* __restrict__ A64,
                                                          const double* __restrict__ Q64, int64_t ldq,
-                                                         int32_t* __restrict__ best) {
+                                                         int32_t* __restrict__ best, const double* __restrict__ ysrc,
+                                                         double* __restrict__ part_v, int32_t* __restrict__ part_g) {
     extern __shared__ double2 sm64v[];
     double* sy = reinterpret_cast<double*>(sm64v);   // [nfit][kS64U]
     double* ss = sy + (size_t)nfit * kS64U;          // [nfit][kS64LdS]
@@ -916,7 +938,7 @@ __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restric
     const int nu = (int)((n - u0) < kS64U ? (n - u0) : kS64U);
     if (tid < kS64U) s_slot[tid] = (tid < nu) ? uslot[u0 + tid] : 0;
     // d - v of the CTA's universes, [j][u] (in the tile buffer, free until the first tile)
-    for (int e = tid; e < nfit * kS64U; e += kS64Threads) {
+    for (int e = tid; !ysrc && e < nfit * kS64U; e += kS64Threads) {
         const int j = e / kS64U, uu = e - (e / kS64U) * kS64U;
         ss[e] = (uu < nu) ? (double)d[(size_t)list[u0 + uu] * nfit + j] - gs.centre[j] : 0.0;
     }
@@ -925,7 +947,9 @@ __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restric
     for (int e = tid; e < nfit * kS64U; e += kS64Threads) {
         const int r = e / kS64U, uu = e - (e / kS64U) * kS64U;
         double t = 0.0;
-        if (uu < nu) {
+        if (uu < nu && ysrc) {
+            t = ysrc[(u0 + uu) * nfit + r];
+        } else if (uu < nu) {
             const double* A = A64 + (size_t)s_slot[uu] * nfit * nfit + (size_t)r * nfit;
             for (int j = 0; j < nfit; ++j) t = fma(A[j], ss[j * kS64U + uu], t);
         }
@@ -939,7 +963,7 @@ __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restric
         bv[a] = DBL_MAX;
         bg[a] = INT32_MAX;
     }
-    for (int64_t g0 = 0; g0 < G; g0 += kS64G) {
+    for (int64_t g0 = (int64_t)blockIdx.y * kS64G; g0 < G; g0 += (int64_t)gridDim.y * kS64G) {
         __syncthreads();  // y complete / the previous tile's readers done
         if (gs.Sc) {
             for (int e = tid; e < kS64G * nfit; e += kS64Threads) {
@@ -1010,7 +1034,12 @@ __global__ void __launch_bounds__(kS64Threads) k_scan64(const int32_t* __restric
                 g = xg;
             }
         }
-        best[list[u0 + tid]] = g;
+        if (gridDim.y == 1) {
+            best[list[u0 + tid]] = g;
+        } else {
+            part_v[(u0 + tid) * gridDim.y + blockIdx.y] = v;
+            part_g[(u0 + tid) * gridDim.y + blockIdx.y] = g;
+        }
     }
 }
 
@@ -2386,15 +2415,32 @@ void launch_set_slots(const int32_t* q, const int32_t* s, int n, int32_t* slot_o
     k_set_slots<<<blocks_for(n), kThreads, 0, st>>>(q, s, n, slot_of);
 }
 
+// CTAs per group of universes: up to eight for every SM, each with at least
+// one tile of the grid.
+int scan64_splits(int64_t n, int64_t G, int n_sm) {
+    const int64_t groups = (n + kS64U - 1) / kS64U, tiles = (G + kS64G - 1) / kS64G;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(8 * (int64_t)n_sm / groups, tiles));
+}
+
 void launch_scan64(const int32_t* list, int64_t n, const int32_t* uslot, const float* d, const GridSpec& gs,
-                   int64_t G, int nfit, const double* A64, const double* Q64, int64_t ldq, int32_t* best,
-                   cudaStream_t st) {
+                   int64_t G, int nfit, const double* A64, const double* Q64, int64_t ldq, int32_t* best, int nsp,
+                   double* y, double* part_v, int32_t* part_g, cudaStream_t st) {
     if (n <= 0) return;
     const size_t smem = (size_t)nfit * (kS64U + kS64LdS) * sizeof(double);
     cudaFuncSetAttribute(k_scan64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool split = nsp > 1;
+    if (split) {
+        count_launch();
+        k_y64<<<(unsigned)n, 64, 0, st>>>(list, uslot, d, gs.centre, nfit, A64, y);
+    }
     count_launch();
-    k_scan64<<<(unsigned)((n + kS64U - 1) / kS64U), kS64Threads, smem, st>>>(list, n, uslot, d, gs, G, nfit, A64,
-                                                                            Q64, ldq, best);
+    const dim3 grid((unsigned)((n + kS64U - 1) / kS64U), (unsigned)nsp);
+    k_scan64<<<grid, kS64Threads, smem, st>>>(list, n, uslot, d, gs, G, nfit, A64, Q64, ldq, best, split ? y : nullptr,
+                                              part_v, part_g);
+    if (split) {
+        count_launch();
+        k_scan_resid_reduce<<<blocks_for(n), kThreads, 0, st>>>(list, n, nsp, part_v, part_g, best);
+    }
 }
 
 void launch_scan_resid(const int32_t* list, int64_t n, const int32_t* uslot, const float* d, const GridSpec& gs,
