@@ -133,22 +133,23 @@ __device__ __forceinline__ void normal_block(uint32_t j, uint32_t u, uint32_t p,
     }
 }
 
-// A bin's private uniform stream: counter (block, u, p, kTagPoisson | bin).
-struct UniformStream {
-    uint32_t k0, k1, u, p, tag, blk;
-    uint32_t buf[4];
-    int pos;
+// A bin's private uniforms: counter (block, u, p, kTagPoisson | bin), four to
+// a block.  Uniforms 2t and 2t + 1 of the bin, those of its rejection trial t;
+// w holds the last block drawn, number blk (-1: none).
+struct BinUniforms {
+    uint32_t k0, k1, u, p, tag;
+    int blk;
+    Philox4 w;
     __device__ __forceinline__ void init(uint32_t key0, uint32_t key1, uint32_t uu, uint32_t pp, uint32_t bin) {
-        k0 = key0; k1 = key1; u = uu; p = pp; tag = kTagPoisson | bin; blk = 0; pos = 4;
+        k0 = key0; k1 = key1; u = uu; p = pp; tag = kTagPoisson | bin; blk = -1;
     }
-    __device__ __forceinline__ float next() {
-        if (pos == 4) {
-            const Philox4 r = philox4x32_10(blk, u, p, tag, k0, k1);
-            buf[0] = r.x[0]; buf[1] = r.x[1]; buf[2] = r.x[2]; buf[3] = r.x[3];
-            blk += 1;
-            pos = 0;
+    __device__ __forceinline__ void pair(int t, float& a, float& b) {
+        if (blk != (t >> 1)) {
+            blk = t >> 1;
+            w = philox4x32_10((uint32_t)blk, u, p, tag, k0, k1);
         }
-        return unit_uniform(buf[pos++]);
+        a = unit_uniform((t & 1) ? w.x[2] : w.x[0]);
+        b = unit_uniform((t & 1) ? w.x[3] : w.x[1]);
     }
 };
 
@@ -196,44 +197,56 @@ __device__ __forceinline__ float log_pmf(float k, float lam, float loglam) {
     return __fsub_rn(__fsub_rn(-t1, t2), t3);
 }
 
-__device__ __forceinline__ int32_t poisson(float lam, UniformStream& st) {
-    if (!(lam > 0.0f)) return 0;
-    if (lam < 10.0f) {
-        float pk = exp32(-lam);
-        float cdf = pk;
-        int32_t k = 0;
-        const float u = st.next();
-        while (u > cdf && k < 64) {
-            k += 1;
-            pk = __fdiv_rn(__fmul_rn(pk, lam), __int2float_rn(k));
-            cdf = __fadd_rn(cdf, pk);
-        }
-        return k;
+// Poisson(lam) for lam < 10: inversion by sequential search
+__device__ __forceinline__ int32_t poisson_inversion(float lam, float u) {
+    float pk = exp32(-lam);
+    float cdf = pk;
+    int32_t k = 0;
+    while (u > cdf && k < 64) {
+        k += 1;
+        pk = __fdiv_rn(__fmul_rn(pk, lam), __int2float_rn(k));
+        cdf = __fadd_rn(cdf, pk);
     }
-    const float slam = __fsqrt_rn(lam);
-    const float loglam = ln32(lam);
-    const float b = __fmaf_rn(2.53f, slam, 0.931f);
-    const float a = __fmaf_rn(0.02483f, b, -0.059f);
-    const float twoa = __fadd_rn(a, a);
-    const float inv_alpha = __fadd_rn(1.1239f, __fdiv_rn(1.1328f, __fsub_rn(b, 3.4f)));
-    const float v_r = __fsub_rn(0.9277f, __fdiv_rn(3.6224f, __fsub_rn(b, 2.0f)));
-    for (int it = 0; it < 64; ++it) {
-        const float U = __fsub_rn(st.next(), 0.5f);
-        const float V = st.next();
-        const float us = __fsub_rn(0.5f, fabsf(U));
-        float t = __fdiv_rn(twoa, us);
+    return k;
+}
+
+// Poisson(lam) for lam >= 10: trials t = 0, 1, ..., each a proposal from the
+// bin's uniforms 2t and 2t + 1 that is accepted quickly, or by its logarithms,
+// or not at all; the first accepted one is the draw, and after kPtrsTrials of
+// them floor(lam) is.
+constexpr int kPtrsTrials = 64;
+
+struct Ptrs {
+    float lam, b, a, v_r;   // of lam
+    float V, us, kf;        // of the trial
+    __device__ __forceinline__ void init(float l) {
+        lam = l;
+        const float slam = __fsqrt_rn(lam);
+        b = __fmaf_rn(2.53f, slam, 0.931f);
+        a = __fmaf_rn(0.02483f, b, -0.059f);
+        v_r = __fsub_rn(0.9277f, __fdiv_rn(3.6224f, __fsub_rn(b, 2.0f)));
+    }
+    // the proposal of a trial; true when it is accepted quickly
+    __device__ __forceinline__ bool propose(float ua, float ub) {
+        const float U = __fsub_rn(ua, 0.5f);
+        V = ub;
+        us = __fsub_rn(0.5f, fabsf(U));
+        float t = __fdiv_rn(__fadd_rn(a, a), us);
         t = __fadd_rn(t, b);
         t = __fmul_rn(t, U);
         t = __fadd_rn(t, lam);
         t = __fadd_rn(t, 0.43f);
-        const float kf = floorf(t);
-        if (us >= 0.07f && V <= v_r) return (int32_t)kf;
-        if (kf < 0.0f || (us < 0.013f && V > us)) continue;
+        kf = floorf(t);
+        return us >= 0.07f && V <= v_r;
+    }
+    // a proposal that was not accepted quickly, by its logarithms
+    __device__ __forceinline__ bool accept(float loglam) const {
+        if (kf < 0.0f || (us < 0.013f && V > us)) return false;
+        const float inv_alpha = __fadd_rn(1.1239f, __fdiv_rn(1.1328f, __fsub_rn(b, 3.4f)));
         const float den = __fadd_rn(__fdiv_rn(a, __fmul_rn(us, us)), b);
         const float lhs = ln32(__fdiv_rn(__fmul_rn(V, inv_alpha), den));
-        if (lhs <= log_pmf(kf, lam, loglam)) return (int32_t)kf;
+        return lhs <= log_pmf(kf, lam, loglam);
     }
-    return (int32_t)floorf(lam);
-}
+};
 
 }  // namespace fcdev

@@ -153,3 +153,26 @@ def test_qvec_groups(ctx, n, n_pts):
     simt = fc.fc_run_points(ctx, gid, pts, 3, 20)
     assert all(np.array_equal(a, b) for a, b in zip(tc, simt))
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- fake data: blocks of 64 universes, 8 rows of L, queued draws -----------------------------
+
+@pytest.mark.parametrize("nf,collapse", [(1, False), (3, True), (7, False), (8, False), (9, True), (33, True),
+                                         (90, True), (200, False)])
+@pytest.mark.parametrize("U", [1, 63, 64, 65, 130])
+def test_fake_data_blocks(ctx, nf, collapse, U):
+    """Bit for bit against the oracle, with bins from nearly empty (inversion) to crowded (rejection)."""
+    import oracle
+
+    S, F = _grid(12, nf, nf)
+    S = S * np.logspace(-2.5, 0.5, nf)[None, ::-1]
+    coll = workloads.pair_collapse(nf) if collapse else None
+    n_fit = (nf + 1) // 2 if collapse else nf
+    ps = np.array([0, 11, 5], np.int64)
+    gid = fc.fc_load_grid(ctx, S, coll, n_fit)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    for fluct in (fc.FC_FLUCT_POISSON_SYS, fc.FC_FLUCT_GAUSS):
+        got = fc.fc_fake_data(ctx, gid, ps, 17, U, n_fit, fluct)
+        want = oracle.fake_data(S, F, ps, 17, U, coll, n_fit, fluct)
+        assert np.array_equal(got, want)
+    fc.fc_unload_grid(ctx, gid)
