@@ -621,13 +621,11 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
         c->acc->evicted += (int64_t)evicted_q.size();
     }
     if (!new_q.empty()) {
-        double* work = nullptr;
-        FC_TRY(scratch(c, "cov_work", new_q.size() * g->nfit * g->nfit, &work));
         FC_CUDA(cudaMemcpyAsync(dq, new_q.data(), new_q.size() * 4, cudaMemcpyHostToDevice, c->stream));
         FC_CUDA(cudaMemcpyAsync(ds, new_s.data(), new_s.size() * 4, cudaMemcpyHostToDevice, c->stream));
         launch_build_cov(g->full(), g->nf, g->nfit, g->identity_collapse ? nullptr : g->collapse, g->F, dq, ds,
                          (int)new_q.size(), cov_mode == FC_COV_IDENTITY ? 2 : 0, g->A64, g->W64, g->A32, g->rho,
-                         work, c->status_dev, c->stream);
+                         c->status_dev, c->stream);
         launch_wdf(g->W64, ds, (int)new_q.size(), g->nfit, g->Wdf, c->stream);
         if (cov_mode != FC_COV_IDENTITY) launch_set_slots(dq, ds, (int)new_q.size(), g->slot_of, c->stream);
         c->acc->distinct_cov += (int64_t)new_q.size();

@@ -542,30 +542,46 @@ __global__ void k_chol_sys(FullSrc src, int nf, const double* __restrict__ F, co
 }
 
 // One CTA per (slot, q): M(q) = C [diag(s) F diag(s) + diag(s)] C^T, L = chol(M),
-// W = L^-1, A = W^T W.  The binary64 pipe of this GPU is narrow, so every
-// phase spreads its elements over all threads of the CTA (a phase with a few
-// busy lanes would hold the pipe for whole warps) and a column's divisions
-// become one reciprocal and multiplies.  These factors feed the fit, not the
-// fake data, so they need not repeat the oracle's rounding bit for bit.
+// W = L^-1, A = W^T W.  Bound by this GPU's narrow binary64 pipe (two
+// multiply-adds a cycle and SM, whatever the active lanes of a warp), so every
+// phase packs its elements onto full warps and the matrix lives in shared
+// memory as one packed triangle.  Factorisation and inversion are one pass over
+// it: step k scales column k of L and row k of W by the pivot's reciprocal and
+// then takes one rank-1 update of every row below,
+//     T_ij -= L_ik v_j,   v_j = L_jk for j > k, W_kj for j <= k
+// (j > k: L's trailing triangle; j < k: W's rows; j = k: column k of L is done
+// with and becomes -L_ik W_kk), a contiguous range of the packed triangle.  The
+// thread that makes the next pivot takes its root while the others update.
+// Every element sees the operations of the separate right-looking passes, in
+// their order.  These factors feed the fit, not the fake data, so they need not
+// repeat the oracle's rounding bit for bit.  Against separate passes over full
+// squares (in global memory above N_fit = 64): 597 covariances of N = 200 in
+// four launches 18.1 -> 11.3 ms, 10 500 of N = 120 30.1 -> 22.4 ms (their
+// multiply-adds alone take 4.1 and 15.7 ms), 10 000 of N = 45 2.8 -> 1.8 ms.
+__host__ __device__ __forceinline__ int tri(int n) { return n * (n + 1) / 2; }
+inline int build_cov_threads(int nfit) { return nfit > 120 ? 512 : 256; }
+inline size_t build_cov_smem(int nfit) { return (size_t)(tri(nfit) + 2 * nfit) * sizeof(double); }
+
 __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __restrict__ coll,
                             const double* __restrict__ F, const int32_t* __restrict__ q_list,
                             const int32_t* __restrict__ slot_list, int cov_mode, double* __restrict__ A64,
                             double* __restrict__ W64, float* __restrict__ A32, float* __restrict__ rho,
-                            double* __restrict__ work, int* __restrict__ status) {
-    extern __shared__ double sLW[];
+                            int* __restrict__ status) {
+    extern __shared__ double sT[];
     __shared__ int s_moff[kMaxBins + 1], s_mem[kMaxBins], s_cur[kMaxBins];
-    __shared__ double s_inv[kMaxBins];
-    __shared__ int s_bad;
+    __shared__ double s_row[kMaxBins];
+    __shared__ double s_inv;
+    __shared__ int s_bad, s_rho;
     const int e0 = blockIdx.x;
     const int q = q_list[e0];
     const int slot = slot_list[e0];
     const int n = nfit;
-    const bool staged = (n <= kResolveMaxN);
-    double* L = staged ? sLW : work + (size_t)e0 * n * n;
+    double* T = sT;              // packed lower triangle: M, then L / W
+    double* sl = sT + tri(n);    // column k of L below the diagonal
+    double* sv = sl + n;         // v
     double* Wg = W64 + (size_t)slot * n * n;
-    double* W = staged ? sLW + n * n : Wg;
     double* A = A64 + (size_t)slot * n * n;
-    __shared__ double s_row[kMaxBins];
+    float* Af = A32 + (size_t)slot * n * n;
     stage_full_row(src, nf, q, s_row);
     const double* s = s_row;
     if (cov_mode == 2) {  // identity test mode
@@ -573,7 +589,7 @@ __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __rest
             const double v = (e / n == e % n) ? 1.0 : 0.0;
             Wg[e] = v;
             A[e] = v;
-            A32[(size_t)slot * n * n + e] = (float)v;
+            Af[e] = (float)v;
         }
         if (threadIdx.x == 0) rho[slot] = 1.0f;
         return;
@@ -581,6 +597,7 @@ __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __rest
     // full bins of each fit bin, in increasing order (counting sort by one thread)
     if (threadIdx.x == 0) {
         s_bad = 0;
+        s_rho = 0;
         if (coll) {
             for (int j = 0; j <= n; ++j) s_moff[j] = 0;
             for (int i = 0; i < nf; ++i) ++s_moff[coll[i] + 1];
@@ -590,52 +607,59 @@ __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __rest
         }
     }
     __syncthreads();
-    // 1. M in fit space (lower triangle; upper zero): element (j, l) sums (s_a F_ab) s_b (+ s_a when a == b)
-    //    over full bins a -> j, b -> l in increasing (a, b)
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        const int j = e / n, l = e % n;
+    auto pivot = [&](double d) {  // 1 / sqrt(d) for the step to come
+        if (!(d > 0.0)) {
+            s_bad = 1;
+            d = 1.0;
+        }
+        s_inv = 1.0 / __dsqrt_rn(d);
+    };
+    // 1. M in fit space: element (j, l) sums (s_a F_ab) s_b (+ s_a when a == b) over full bins a -> j,
+    //    b -> l in increasing (a, b)
+    for (int e = threadIdx.x; e < tri(n); e += blockDim.x) {
+        int j, l;
+        tri_decode(e, j, l);
         double v = 0.0;
-        if (l <= j) {
-            if (coll == nullptr) {
-                v = (s[j] * F[j * nf + l]) * s[l];
-                if (j == l) v += s[j];
-            } else {
-                for (int ia = s_moff[j]; ia < s_moff[j + 1]; ++ia) {
-                    const int a = s_mem[ia];
-                    for (int ib = s_moff[l]; ib < s_moff[l + 1]; ++ib) {
-                        const int b = s_mem[ib];
-                        double t = (s[a] * F[a * nf + b]) * s[b];
-                        if (a == b) t += s[a];
-                        v += t;
-                    }
+        if (coll == nullptr) {
+            v = (s[j] * F[j * nf + l]) * s[l];
+            if (j == l) v += s[j];
+        } else {
+            for (int ia = s_moff[j]; ia < s_moff[j + 1]; ++ia) {
+                const int a = s_mem[ia];
+                for (int ib = s_moff[l]; ib < s_moff[l + 1]; ++ib) {
+                    const int b = s_mem[ib];
+                    double t = (s[a] * F[a * nf + b]) * s[b];
+                    if (a == b) t += s[a];
+                    v += t;
                 }
             }
         }
-        L[e] = v;
+        T[e] = v;
+        if (e == 0) pivot(v);
     }
     __syncthreads();
-    // 2. Cholesky, right-looking; column k is scaled by the reciprocal of its pivot
+    // 2. L and W
     for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            double d = L[k * n + k];
-            if (!(d > 0.0)) {
-                s_bad = 1;
-                d = 1.0;
+        const double inv = s_inv;
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            if (j > k) {
+                const double l = T[tri(j) + k] * inv;
+                sl[j] = l;
+                sv[j] = l;
+            } else {
+                const double w = j < k ? T[tri(k) + j] * inv : inv;
+                sv[j] = w;
+                T[tri(k) + j] = w;
             }
-            const double sd = __dsqrt_rn(d);
-            L[k * n + k] = sd;
-            s_inv[k] = 1.0 / sd;
         }
         __syncthreads();
-        const double ik = s_inv[k];
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) L[i * n + k] *= ik;
-        __syncthreads();
-        const int m = n - k - 1;
-        for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-            const int a = e / m, b = e % m;
-            if (b > a) continue;
-            const int i = k + 1 + a, jj = k + 1 + b;
-            L[i * n + jj] -= L[i * n + k] * L[jj * n + k];
+        const int next = tri(k + 1) + k + 1;  // the next pivot's element
+        for (int e = tri(k + 1) + threadIdx.x; e < tri(n); e += blockDim.x) {
+            int i, j;
+            tri_decode(e, i, j);
+            const double t = fma(-sl[i], sv[j], j == k ? 0.0 : T[e]);
+            T[e] = t;
+            if (e == next) pivot(t);
         }
         __syncthreads();
     }
@@ -643,45 +667,39 @@ __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __rest
         if (threadIdx.x == 0) atomicOr(status, kDevNotSpd);
         return;
     }
-    // 3. W = L^-1 by elimination on [L | I]: at step k row k of W is scaled by 1/L_kk and
-    //    final; every row i > k then subtracts L_ik times it (columns c <= k)
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) W[e] = (e / n == e % n) ? 1.0 : 0.0;
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        const double ik = s_inv[k];
-        for (int c = threadIdx.x; c <= k; c += blockDim.x) W[k * n + c] *= ik;
-        __syncthreads();
-        const int m = n - k - 1, w = k + 1;
-        for (int e = threadIdx.x; e < m * w; e += blockDim.x) {
-            const int i = k + 1 + e / w, c = e % w;
-            W[i * n + c] -= L[i * n + k] * W[k * n + c];
-        }
-        __syncthreads();
-    }
-    // A = W^T W: A_ij = sum_{k >= max(i,j)} W_ki W_kj
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int i = e / n, j = e % n;
-        if (j > i) continue;
+        Wg[e] = j <= i ? T[tri(i) + j] : 0.0;
+    }
+    // 3. A_ij = sum_{k >= i} W_ki W_kj for j <= i
+    for (int e = threadIdx.x; e < tri(n); e += blockDim.x) {
+        int i, j;
+        tri_decode(e, i, j);
         double acc = 0.0;
-        for (int k = i; k < n; ++k) acc = fma(W[k * n + i], W[k * n + j], acc);
+        const double *wi = T + tri(i) + i, *wj = T + tri(i) + j;
+        for (int k = i; k < n; ++k) {
+            acc = fma(*wi, *wj, acc);
+            wi += k + 1;
+            wj += k + 1;
+        }
         A[i * n + j] = acc;
         A[j * n + i] = acc;
-    }
-    if (staged)
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) Wg[e] = W[e];
-    __syncthreads();
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) A32[(size_t)slot * n * n + e] = (float)A[e];
-    // rho = max_i sum_j |A_ij| (an upper bound of the spectral norm of |A|), rounded up
-    __shared__ double s_rho;
-    if (threadIdx.x == 0) s_rho = 0.0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double r = 0.0;
-        for (int j = 0; j < n; ++j) r += fabs(A[i * n + j]);
-        atomicMax((unsigned long long*)&s_rho, (unsigned long long)__double_as_longlong(r));
+        Af[i * n + j] = (float)acc;
+        Af[j * n + i] = (float)acc;
     }
     __syncthreads();
-    if (threadIdx.x == 0) rho[slot] = __double2float_ru(s_rho * (1.0 + 1e-9));
+    // rho >= max_i sum_j |A_ij| (an upper bound of the spectral norm of |A|): the binary32 sums, raised by
+    // their rounding
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = warp; i < n; i += blockDim.x >> 5) {
+        float r = 0.0f;
+        for (int j = lane; j < n; j += 32) r += fabsf(Af[i * n + j]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        if (lane == 0) atomicMax(&s_rho, __float_as_int(r));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) rho[slot] = __fmul_ru(__int_as_float(s_rho), 1.0f + (float)(n + 4) * 1.1920929e-07f);
 }
 
 // q_g = s~_g^T A s~_g in binary64, one thread per g
@@ -2456,14 +2474,13 @@ void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t*
 
 void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* coll, const double* F, const int32_t* q_list,
                       const int32_t* slot_list, int n, int cov_mode, double* A64, double* W64, float* A32,
-                      float* rho, double* work, int* status, cudaStream_t st) {
+                      float* rho, int* status, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();
-    const size_t smem = nfit <= kResolveMaxN ? 2 * (size_t)nfit * nfit * sizeof(double) : 0;
-    cudaFuncSetAttribute(k_build_cov, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         2 * kResolveMaxN * kResolveMaxN * (int)sizeof(double));
-    k_build_cov<<<n, 256, smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64, A32, rho,
-                                      work, status);
+    const size_t smem = build_cov_smem(nfit);
+    allow_smem(k_build_cov, smem);
+    k_build_cov<<<n, build_cov_threads(nfit), smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64,
+                                                          A32, rho, status);
 }
 
 void launch_qvec64(const GridSpec& gs, int64_t G, int nfit, const double* W64, const int32_t* slots, int n,
