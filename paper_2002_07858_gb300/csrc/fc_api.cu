@@ -14,6 +14,7 @@
 #include <atomic>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
@@ -149,6 +150,16 @@ struct Scratch {
     size_t bytes = 0;
 };
 
+// What the host reads between launches, in one block on the device and one
+// pinned mirror, so that a decision costs one small copy and one wait: the
+// counts of a scan, its counters, and the status word the kernels raise.
+struct Ctrl {
+    int32_t cnts[8];                  // [1] failed rows, [2] continuing, [3] finishing, [4] failed again, [5] tiles, [6] rows
+    unsigned long long counters[16];  // see scan_once
+    int status;                       // kDev* flags, sticky until reported
+};
+constexpr int32_t kListHost = 4096;   // entries of a device list fetched along with its count
+
 // Served job: a copy of the caller's arguments and its completion state.
 struct JobRec {
     fc_job job;
@@ -216,9 +227,16 @@ struct fc_ctx {
     std::map<int32_t, std::unique_ptr<Grid>> grids;
     int32_t next_grid = 1;
     std::map<std::string, Scratch> scratch;
-    int* status_dev = nullptr;
-    unsigned long long* counters_dev = nullptr;
-    cudaEvent_t ev_a = nullptr, ev_b = nullptr;  // stage timers
+    Ctrl* ctrl = nullptr;            // device
+    Ctrl* ctrl_host = nullptr;       // pinned; the device's values as of the last read_ctrl
+    bool ctrl_read = false;          // nothing that changes the counts was launched since then
+    int32_t* list_host = nullptr;    // pinned [kListHost]
+    int* status_dev = nullptr;       // &ctrl->status
+    unsigned long long* counters_dev = nullptr;  // ctrl->counters
+    // stage timers: event pairs around the stages since the last flush_stages, and where each one counts
+    std::vector<std::pair<cudaEvent_t, cudaEvent_t>> stage_ev;
+    std::vector<double*> stage_acc;
+    cudaEvent_t run_ev[3] = {nullptr, nullptr, nullptr};
     fc_stats stats{};              // last synchronous call
     fc_stats serve_stats{};        // everything the serving worker ran
     fc_stats* acc = &stats;        // where the running work counts
@@ -337,10 +355,12 @@ fc_status sync(fc_ctx* c) {
     return FC_OK;
 }
 
-fc_status check_status(fc_ctx* c) {
-    int st = 0;
-    FC_CUDA(cudaMemcpyAsync(&st, c->status_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+// The control block as of now (waits for the stream), and the errors the kernels raised.
+fc_status read_ctrl(fc_ctx* c) {
+    FC_CUDA(cudaMemcpyAsync(c->ctrl_host, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
     FC_TRY(sync(c));
+    c->ctrl_read = true;
+    const int st = c->ctrl_host->status;
     if (st) {
         FC_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), c->stream));
         if (st & kDevTimeout) return fail(FC_ERR_TIMEOUT, "a device-side wait timed out");
@@ -350,15 +370,38 @@ fc_status check_status(fc_ctx* c) {
     return FC_OK;
 }
 
+fc_status check_status(fc_ctx* c) { return read_ctrl(c); }
+
 // Stage timing: an event pair on the context stream around a stage's kernels.
-void stage_begin(fc_ctx* c) { cudaEventRecord(c->ev_a, c->stream); }
+// The pairs are read together once the stream has been waited for anyway.
+fc_status flush_stages(fc_ctx* c, bool waited) {
+    if (!waited) FC_TRY(sync(c));
+    for (size_t i = 0; i < c->stage_acc.size(); ++i) {
+        float ms = 0.0f;
+        FC_CUDA(cudaEventElapsedTime(&ms, c->stage_ev[i].first, c->stage_ev[i].second));
+        *c->stage_acc[i] += ms;
+    }
+    c->stage_acc.clear();
+    return FC_OK;
+}
+
+fc_status stage_begin(fc_ctx* c) {
+    constexpr size_t kMaxStages = 64;
+    if (c->stage_acc.size() >= kMaxStages) FC_TRY(flush_stages(c, false));
+    if (c->stage_acc.size() == c->stage_ev.size()) {
+        cudaEvent_t a = nullptr, b = nullptr;
+        FC_CUDA(cudaEventCreate(&a));
+        c->stage_ev.emplace_back(a, b);
+        FC_CUDA(cudaEventCreate(&b));
+        c->stage_ev.back().second = b;
+    }
+    FC_CUDA(cudaEventRecord(c->stage_ev[c->stage_acc.size()].first, c->stream));
+    return FC_OK;
+}
 
 fc_status stage_end(fc_ctx* c, double* acc_ms) {
-    cudaEventRecord(c->ev_b, c->stream);
-    FC_TRY(sync(c));
-    float ms = 0.0f;
-    FC_CUDA(cudaEventElapsedTime(&ms, c->ev_a, c->ev_b));
-    *acc_ms += ms;
+    FC_CUDA(cudaEventRecord(c->stage_ev[c->stage_acc.size()].second, c->stream));
+    c->stage_acc.push_back(acc_ms);
     return FC_OK;
 }
 
@@ -531,7 +574,9 @@ bool use_qvec_tc(const Grid* g) {
 // Make sure every grid index in `qs` has a covariance slot (build + invert the
 // missing ones) and, for the given path, its q-vector.  The slots of `qs` are
 // all resident when this returns: they are marked as used by this call, so a
-// full cache hands out only slots that this call does not need.
+// full cache hands out only slots that this call does not need.  The kernels
+// are launched, not waited for: a covariance that is not positive definite
+// raises the status word, which the next read_ctrl reports.
 fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int cov_mode, bool need_q32,
                        bool need_q64, std::vector<int32_t>* slots_out) {
     FC_TRY(ensure_cache(c, g));
@@ -617,7 +662,6 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
         FC_CUDA(cudaMemcpyAsync(dq, evicted_q.data(), evicted_q.size() * 4, cudaMemcpyHostToDevice, c->stream));
         FC_CUDA(cudaMemcpyAsync(ds, minus.data(), minus.size() * 4, cudaMemcpyHostToDevice, c->stream));
         launch_set_slots(dq, ds, (int)evicted_q.size(), g->slot_of, c->stream);
-        FC_TRY(sync(c));
         c->acc->evicted += (int64_t)evicted_q.size();
     }
     if (!new_q.empty()) {
@@ -629,7 +673,6 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
         launch_wdf(g->W64, ds, (int)new_q.size(), g->nfit, g->Wdf, c->stream);
         if (cov_mode != FC_COV_IDENTITY) launch_set_slots(dq, ds, (int)new_q.size(), g->slot_of, c->stream);
         c->acc->distinct_cov += (int64_t)new_q.size();
-        FC_TRY(check_status(c));
     }
     if (!q32_list.empty()) {
         FC_TRY(ensure_q32_storage(c, g));
@@ -644,13 +687,11 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
             launch_qvec32(g->spec(), g->gnorm, g->G, g->G_pad, g->nfit, g->A32, g->rho, ds, (int)q32_list.size(),
                           g->Qc, g->Qb, g->Qb3, c->stream);
         }
-        FC_TRY(check_status(c));
     }
     if (!q64_list.empty()) {
         FC_TRY(ensure_q64_storage(c, g));
         FC_CUDA(cudaMemcpyAsync(ds, q64_list.data(), q64_list.size() * 4, cudaMemcpyHostToDevice, c->stream));
         launch_qvec64(g->spec(), g->G, g->nfit, g->W64, ds, (int)q64_list.size(), g->G, g->Q64, c->stream);
-        FC_TRY(sync(c));
     }
     return FC_OK;
 }
@@ -746,20 +787,23 @@ inline unsigned nb(int64_t n, int t = 256) { return (unsigned)std::max<int64_t>(
 fc_status distinct_cur(fc_ctx* c, Grid* g, const int32_t* active, int64_t n_active, const int32_t* cur,
                        std::vector<int32_t>& out) {
     uint8_t* flag = nullptr;
-    int32_t *list = nullptr, *cnt = nullptr;
+    int32_t* list = nullptr;  // [0]: count, then the indices
+    const size_t room = (size_t)std::min<int64_t>(g->G, n_active) + 1;
     FC_TRY(scratch(c, "flag", (size_t)g->G, &flag));
-    FC_TRY(scratch(c, "dlist", (size_t)std::min<int64_t>(g->G, n_active) + 1, &list));
-    FC_TRY(scratch(c, "dcount", 1, &cnt));
+    FC_TRY(scratch(c, "dlist", room, &list));
     FC_CUDA(cudaMemsetAsync(flag, 0, (size_t)g->G, c->stream));
-    FC_CUDA(cudaMemsetAsync(cnt, 0, 4, c->stream));
+    FC_CUDA(cudaMemsetAsync(list, 0, 4, c->stream));
     launch_mark_used(active, n_active, cur, flag, c->stream);
-    launch_compact_flags(flag, g->G, list, cnt, c->stream);
-    int32_t h = 0;
-    FC_CUDA(cudaMemcpyAsync(&h, cnt, 4, cudaMemcpyDeviceToHost, c->stream));
-    FC_TRY(sync(c));
-    out.resize(h);
-    if (h) {
-        FC_CUDA(cudaMemcpyAsync(out.data(), list, (size_t)h * 4, cudaMemcpyDeviceToHost, c->stream));
+    launch_compact_flags(flag, g->G, list + 1, list, c->stream);
+    const size_t first = std::min<size_t>(room, kListHost);
+    FC_CUDA(cudaMemcpyAsync(c->list_host, list, first * 4, cudaMemcpyDeviceToHost, c->stream));
+    FC_TRY(read_ctrl(c));
+    const size_t h = (size_t)c->list_host[0];
+    out.assign(c->list_host + 1, c->list_host + std::min(h + 1, first));
+    if (h + 1 > first) {
+        out.resize(h);
+        FC_CUDA(cudaMemcpyAsync(out.data() + (first - 1), list + first, (h + 1 - first) * 4, cudaMemcpyDeviceToHost,
+                                c->stream));
         FC_TRY(sync(c));
     }
     std::sort(out.begin(), out.end());
@@ -881,7 +925,9 @@ fc_status lane_admit(fc_ctx* c, Lane* L, const std::shared_ptr<LaneJob>& J, cons
         FC_TRY(scratch(c, "s32", (size_t)P * g->nf, &s32));
         launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, nullptr,
                         c->status_dev, c->stream);
-        FC_TRY(check_status(c));
+        // a served job's own factor must not fail the jobs it would join; a synchronous call reports it
+        // with the first count it reads
+        if (J->jr) FC_TRY(check_status(c));
         launch_fake_data(L32, s32, g->nf, g->identity_collapse ? nullptr : g->collapse, g->nfit, ps_dev, P, U, seed,
                          fluct == FC_FLUCT_GAUSS, dst, c->stream);
     }
@@ -920,8 +966,9 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
     const bool skip16 = mixed && g->tune.first_round != FC_ROUND_TOPK;
     int32_t *active = L->active, *next = L->next, *fin = L->fin, *uslot = L->uslot, *cur = L->cur;
     const float* d = L->d;
-    int32_t* cnts = nullptr;
-    FC_TRY(scratch(c, "cnts", 8, &cnts));
+    int32_t* cnts = c->ctrl->cnts;
+    const int32_t* h_cnts = c->ctrl_host->cnts;  // valid after read_ctrl
+    c->stage_acc.clear();                        // of a scan that ended in an error
     UniverseState us;
     us.cur = L->cur;
     us.pt = L->pt;
@@ -929,18 +976,23 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
     us.maxit = L->maxit;
     us.job_of = L->job_of;
     us.job_left = L->job_left;
-    FC_CUDA(cudaMemsetAsync(c->counters_dev, 0, 13 * sizeof(unsigned long long), c->stream));
-    // exact binary64 scan for `list`, then advance / finish them
-    auto exact_scan = [&](const int32_t* list, int64_t cnt) -> fc_status {
-        std::vector<int32_t> fq;
-        int32_t* fslot = nullptr;
-        FC_TRY(scratch(c, "fslot", (size_t)cnt, &fslot));
-        if (mixed) {
-            // the mixed path's last resort: residual form for every g, no binary64 q-vectors
+    // counts ([2], the continuing universes, is the whole scan's) and counters; not the status
+    FC_CUDA(cudaMemsetAsync(c->ctrl, 0, offsetof(Ctrl, status), c->stream));
+    c->ctrl_read = false;
+    // exact scan for `list`, then advance / finish them; lslot: their slots (null: looked up here)
+    auto exact_scan = [&](const int32_t* list, int64_t cnt, const int32_t* lslot) -> fc_status {
+        c->ctrl_read = false;
+        if (!lslot) {
+            int32_t* fslot = nullptr;
+            FC_TRY(scratch(c, "fslot", (size_t)cnt, &fslot));
             if (o.cov == FC_COV_IDENTITY)
                 launch_fill_i32(fslot, cnt, g->ident_slot, c->stream);
             else
                 launch_lookup_slots(list, cnt, cur, g->slot_of, fslot, c->stream);
+            lslot = fslot;
+        }
+        if (mixed) {
+            // the mixed path's last resort: residual form for every g, no binary64 q-vectors.
             // enough CTAs to cover the GPU about four times, each at least 1024 grid points
             int nsp = (int)std::max<int64_t>(1, (4 * (int64_t)c->n_sm + cnt - 1) / cnt);
             nsp = (int)std::min<int64_t>(nsp, std::max<int64_t>(1, g->G / 1024));
@@ -948,28 +1000,12 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
             int32_t* pg = nullptr;
             FC_TRY(scratch(c, "fb_pv", (size_t)cnt * nsp, &pv));
             FC_TRY(scratch(c, "fb_pg", (size_t)cnt * nsp, &pg));
-            stage_begin(c);
-            launch_scan_resid(list, cnt, fslot, d, g->spec(), g->G, g->nfit, g->Wdf, pv, pg, nsp, L->best,
+            FC_TRY(stage_begin(c));
+            launch_scan_resid(list, cnt, lslot, d, g->spec(), g->G, g->nfit, g->Wdf, pv, pg, nsp, L->best,
                               c->stream);
             S->residuals += cnt * g->G;
             FC_TRY(stage_end(c, &S->ms_fallback));
-        } else if (o.cov == FC_COV_IDENTITY) {
-            FC_TRY(ensure_slots(c, g, fq, o.cov, false, true, nullptr));
-            launch_fill_i32(fslot, cnt, g->ident_slot, c->stream);
         } else {
-            int32_t* fcur = nullptr;
-            FC_TRY(scratch(c, "fcur", (size_t)cnt, &fcur));
-            count_launch();
-            k_gather_cur<<<nb(cnt), 256, 0, c->stream>>>(list, (int)cnt, cur, fcur);
-            fq.resize(cnt);
-            FC_CUDA(cudaMemcpyAsync(fq.data(), fcur, (size_t)cnt * 4, cudaMemcpyDeviceToHost, c->stream));
-            FC_TRY(sync(c));
-            std::sort(fq.begin(), fq.end());
-            fq.erase(std::unique(fq.begin(), fq.end()), fq.end());
-            FC_TRY(ensure_slots(c, g, fq, o.cov, false, true, nullptr));
-            launch_lookup_slots(list, cnt, cur, g->slot_of, fslot, c->stream);
-        }
-        if (!mixed) {
             int nsp = scan64_splits(cnt, g->G, c->n_sm);
             double *pv = nullptr, *py = nullptr;
             int32_t* pg = nullptr;
@@ -977,8 +1013,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                             scratch(c, "fb_pv", (size_t)cnt * nsp, &pv) != FC_OK ||
                             scratch(c, "fb_pg", (size_t)cnt * nsp, &pg) != FC_OK))
                 nsp = 1;  // no room for the partial minima
-            stage_begin(c);
-            launch_scan64(list, cnt, fslot, d, g->spec(), g->G, g->nfit, g->A64, g->Q64, g->G, L->best, nsp, py, pv,
+            FC_TRY(stage_begin(c));
+            launch_scan64(list, cnt, lslot, d, g->spec(), g->G, g->nfit, g->A64, g->Q64, g->G, L->best, nsp, py, pv,
                           pg, c->stream);
             FC_TRY(stage_end(c, &S->ms_scan64));
         }
@@ -986,30 +1022,27 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
         // finishing universes keep cur (the covariance of this scan); others move to their minimum
         FC_CUDA(cudaMemsetAsync(cnts + 3, 0, 4, c->stream));
         launch_advance(list, cnt, L->best, us, next, cnts + 2, fin, cnts + 3, c->stream);
-        int32_t n_fin = 0;
-        FC_CUDA(cudaMemcpyAsync(&n_fin, cnts + 3, 4, cudaMemcpyDeviceToHost, c->stream));
-        FC_TRY(sync(c));
-        if (n_fin > 0) {
-            int32_t* finslot = nullptr;
-            FC_TRY(scratch(c, "finslot", (size_t)n_fin, &finslot));
-            if (o.cov == FC_COV_IDENTITY)
-                launch_fill_i32(finslot, n_fin, g->ident_slot, c->stream);
-            else
-                launch_lookup_slots(fin, n_fin, cur, g->slot_of, finslot, c->stream);
-            stage_begin(c);
-            launch_finish(fin, n_fin, finslot, L->best, us, d, g->spec(), g->nfit, g->W64, mixed ? g->Wdf : nullptr,
-                          L->dchi2, L->chi2min, c->stream);
-            if (mixed) S->residuals += 2 * (int64_t)n_fin;
-            FC_TRY(stage_end(c, &S->ms_finish));
+        // as many as finish, a count that stays on the device
+        FC_TRY(stage_begin(c));
+        launch_finish(fin, cnt, cnts + 3, o.cov == FC_COV_IDENTITY ? g->ident_slot : -1, g->slot_of, L->best, us, d,
+                      g->spec(), g->nfit, g->W64, mixed ? g->Wdf : nullptr, L->dchi2, L->chi2min, c->stream);
+        FC_TRY(stage_end(c, &S->ms_finish));
+        if (mixed) {
+            FC_TRY(read_ctrl(c));
+            S->residuals += 2 * (int64_t)h_cnts[3];
         }
         return FC_OK;
     };
+    bool first_list = true;
     // one scan of the universes in `list` (their covariance slots in lslot, by list position)
     auto scan_list = [&](const int32_t* sl_list, int64_t sl_n, const int32_t* sl_slot) -> fc_status {
-        FC_CUDA(cudaMemsetAsync(cnts + 3, 0, 12, c->stream));  // n_fin, n_fb2, n_tiles
-        FC_CUDA(cudaMemsetAsync(cnts + 1, 0, 4, c->stream));   // n_fb
+        if (!first_list) {  // a later wave: the scan's first list finds the counts cleared
+            FC_CUDA(cudaMemsetAsync(cnts + 3, 0, 12, c->stream));  // n_fin, n_fb2, n_tiles
+            FC_CUDA(cudaMemsetAsync(cnts + 1, 0, 4, c->stream));   // n_fb
+        }
+        first_list = false;
         if (!mixed) {
-            FC_TRY(exact_scan(sl_list, sl_n));
+            FC_TRY(exact_scan(sl_list, sl_n, sl_slot));
         } else {
             int32_t *fb = L->fb, *fb2 = L->fb2, *fslot = L->fbslot;
             float* thr = L->thr;
@@ -1048,17 +1081,17 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 FC_TRY(scratch(c, ("cval" + sfx).c_str(), n_cand, &cval));
                 FC_TRY(scratch(c, ("cidx" + sfx).c_str(), n_cand, &cidx));
                 FC_TRY(scratch(c, "ccount", (size_t)max_tiles * kBM * 2, &ccount));
-                stage_begin(c);
+                FC_TRY(stage_begin(c));
                 launch_group(list, cnt, lslot, (int)n_slots, tcnt, tbase, tfill, cnts + 5, tslot, tuniv, max_tiles,
                              g->tune.slot_rows ? g->tune.slot_rows : kQuadRows, c->stream);
-                int32_t n_tiles = 0;
-                FC_CUDA(cudaMemcpyAsync(&n_tiles, cnts + 5, 4, cudaMemcpyDeviceToHost, c->stream));
-                FC_TRY(sync(c));
+                FC_TRY(read_ctrl(c));
+                c->ctrl_read = false;
+                const int32_t n_tiles = h_cnts[5];
                 launch_yprep(tslot, tuniv, n_tiles, d, g->centre_df, g->nfit, g->K, g->A32, g->rho, cur, g->spec(),
                              g->gnorm, g->Qc, g->Qb, g->G_pad, Yt, alpha, tau0, tj0, c->stream);
                 if (seeded) launch_min_tau(tuniv, n_tiles, thr, tau0, c->stream);
                 FC_TRY(stage_end(c, &S->ms_prep));
-                stage_begin(c);
+                FC_TRY(stage_begin(c));
                 // round 0: a min-only pass to tighten the seeds when most rows are on their first scan (the probe
                 // at the true point is loose there; later scans probe at the previous minimum), then the top-k
                 // pass.  Later rounds are seeded by the best binary64 value (round 1: top-k, round 2: list).
@@ -1084,10 +1117,9 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     S->screen_tiles += n_tiles;
                     S->screen_rows += cnt;
                 }
+                // a screen that gave up (a bounded wait ran out) leaves its candidates incomplete: the
+                // resolution does nothing then, and the next read_ctrl reports it
                 FC_TRY(stage_end(c, &S->ms_screen));
-                // a screen that gave up (a bounded wait ran out) leaves its candidates incomplete:
-                // report it before anything reads them
-                FC_TRY(check_status(c));
                 S->screen_flops += 2.0 * g->nfit * (double)cnt * (double)g->G;
                 ResolveArgs ra{};
                 ra.quad_slot = tslot;
@@ -1130,7 +1162,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 ra.round_bit = round == 0 ? 0 : (round == 1 ? kDecidedTop16 : (round == 2 ? kDecidedList
                                                                                           : kDecidedExactList));
                 ra.n_sm = c->n_sm;
-                stage_begin(c);
+                ra.status = c->status_dev;
+                FC_TRY(stage_begin(c));
                 if (listing)
                 {
                     int32_t* lrows = nullptr;
@@ -1164,8 +1197,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     FC_TRY(scratch(c, "rs_tiles2", (size_t)n_tiles * kQuads, &ra.tile_items2));
                     launch_resolve(ra, n_tiles, cnt, c->stream);
                 }
-                FC_TRY(stage_end(c, &S->ms_rescore));
-                return check_status(c);
+                return stage_end(c, &S->ms_rescore);
             };
             // fourth round for universes whose candidate lists overflowed: the same list screen
             // again with exact-size storage, then binary64 rescoring of every listed point;
@@ -1222,21 +1254,20 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     FC_TRY(screen_round(3, d_u, nb4, fslot, kMaxTopK, d_x, n_x, true, loff, lnum, total));
                     int32_t nx = 0;
                     FC_CUDA(cudaMemcpyAsync(&nx, n_x, 4, cudaMemcpyDeviceToHost, c->stream));
-                    FC_TRY(sync(c));
+                    FC_TRY(read_ctrl(c));
                     S->fallback += nx;
-                    if (nx > 0) FC_TRY(exact_scan(d_x, nx));
+                    if (nx > 0) FC_TRY(exact_scan(d_x, nx, nullptr));
                 }
                 if (!exact_u.empty()) {
                     FC_CUDA(cudaMemcpyAsync(d_u, exact_u.data(), exact_u.size() * 4, cudaMemcpyHostToDevice,
                                             c->stream));
-                    FC_TRY(exact_scan(d_u, (int64_t)exact_u.size()));
+                    FC_TRY(exact_scan(d_u, (int64_t)exact_u.size(), nullptr));
                 }
                 return FC_OK;
             };
             FC_TRY(screen_round(0, sl_list, sl_n, sl_slot, topk, fb, cnts + 1, false));
-            int32_t n_fb = 0;
-            FC_CUDA(cudaMemcpyAsync(&n_fb, cnts + 1, 4, cudaMemcpyDeviceToHost, c->stream));
-            FC_TRY(sync(c));
+            FC_TRY(read_ctrl(c));
+            const int32_t n_fb = h_cnts[1];
             if (n_fb > 0 && skip16) {
                 // straight to the list round, seeded by the binary64 value round 1 found
                 if (o.cov == FC_COV_IDENTITY)
@@ -1244,9 +1275,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 else
                     launch_lookup_slots(fb, n_fb, cur, g->slot_of, fslot, c->stream);
                 FC_TRY(screen_round(2, fb, n_fb, fslot, kMaxTopK, fb2, cnts + 4, true));
-                int32_t n_ov = 0;
-                FC_CUDA(cudaMemcpyAsync(&n_ov, cnts + 4, 4, cudaMemcpyDeviceToHost, c->stream));
-                FC_TRY(sync(c));
+                FC_TRY(read_ctrl(c));
+                const int32_t n_ov = h_cnts[4];
                 if (n_ov > 0) FC_TRY(big_lists(fb2, n_ov, lcount));
             } else if (n_fb > 0) {
                 // second certified round for the universes whose certificate failed
@@ -1255,9 +1285,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 else
                     launch_lookup_slots(fb, n_fb, cur, g->slot_of, fslot, c->stream);
                 FC_TRY(screen_round(1, fb, n_fb, fslot, kMaxTopK, fb2, cnts + 4, true));
-                int32_t n_fb2 = 0;
-                FC_CUDA(cudaMemcpyAsync(&n_fb2, cnts + 4, 4, cudaMemcpyDeviceToHost, c->stream));
-                FC_TRY(sync(c));
+                FC_TRY(read_ctrl(c));
+                const int32_t n_fb2 = h_cnts[4];
                 if (n_fb2 > 0) {
                     // third round: list every point that can still be the minimum
                     if (o.cov == FC_COV_IDENTITY)
@@ -1266,9 +1295,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                         launch_lookup_slots(fb2, n_fb2, cur, g->slot_of, fslot, c->stream);
                     FC_CUDA(cudaMemsetAsync(cnts + 1, 0, 4, c->stream));
                     FC_TRY(screen_round(2, fb2, n_fb2, fslot, kMaxTopK, fb, cnts + 1, true));
-                    int32_t n_fb3 = 0;
-                    FC_CUDA(cudaMemcpyAsync(&n_fb3, cnts + 1, 4, cudaMemcpyDeviceToHost, c->stream));
-                    FC_TRY(sync(c));
+                    FC_TRY(read_ctrl(c));
+                    const int32_t n_fb3 = h_cnts[1];
                     if (n_fb3 > 0) FC_TRY(big_lists(fb, n_fb3, lcount));
                 }
             }
@@ -1277,19 +1305,18 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
     };
     S->chi2_evals += n_active * g->G;
     S->scans += n_active;
-    FC_CUDA(cudaMemsetAsync(cnts + 2, 0, 4, c->stream));  // n_next: continuing universes of the whole scan
     // ---- covariances for this scan, then the scan itself; a scan that needs more
     // distinct covariances than the cache holds runs in waves of cache-sized groups
     if (o.cov == FC_COV_IDENTITY) {
         std::vector<int32_t> qs, slots;
-        stage_begin(c);
+        FC_TRY(stage_begin(c));
         FC_TRY(ensure_slots(c, g, qs, o.cov, mixed, !mixed, &slots));
         launch_fill_i32(uslot, n_active, slots[0], c->stream);
         FC_TRY(stage_end(c, &S->ms_cov));
         FC_TRY(scan_list(active, n_active, uslot));
     } else {
         std::vector<int32_t> qs;
-        stage_begin(c);
+        FC_TRY(stage_begin(c));
         FC_TRY(distinct_cur(c, g, active, n_active, cur, qs));
         FC_TRY(ensure_cache(c, g));
         const int64_t lim =
@@ -1320,7 +1347,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 const std::vector<int32_t> part(qs.begin() + q0,
                                                 qs.begin() + std::min(qs.size(), q0 + (size_t)wave));
                 S->scan_waves += 1;
-                stage_begin(c);
+                FC_TRY(stage_begin(c));
                 // the universes whose covariance index is in this part
                 FC_CUDA(cudaMemsetAsync(flag, 0, (size_t)g->G, c->stream));
                 FC_CUDA(cudaMemsetAsync(wn, 0, 4, c->stream));
@@ -1337,14 +1364,12 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
             }
         }
     }
-    int32_t n_next = 0;
-    FC_CUDA(cudaMemcpyAsync(&n_next, cnts + 2, 4, cudaMemcpyDeviceToHost, c->stream));
+    if (!c->ctrl_read) FC_TRY(read_ctrl(c));
+    const int32_t n_next = h_cnts[2];
     // [0..2] round 1: screened, rescored, handed on; [3..5] round 2 likewise; [6] listed, [7] list
     // overflow; [9] resolved from exact-size lists, [10] their failures (counted with the fallback)
     // [12] residual chi2 evaluated by the certified rounds
-    unsigned long long cn[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    FC_CUDA(cudaMemcpyAsync(cn, c->counters_dev, sizeof(cn), cudaMemcpyDeviceToHost, c->stream));
-    FC_TRY(sync(c));
+    const unsigned long long* cn = c->ctrl_host->counters;
     std::swap(L->active, L->next);
     L->n_active = n_next;
     S->screened += (int64_t)(cn[0] + cn[3]);
@@ -1352,7 +1377,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
     S->rescreened += (int64_t)(cn[2] + cn[5]);
     S->big_listed += (int64_t)(cn[9] + cn[10]);
     S->residuals += (int64_t)cn[12];
-    return check_status(c);
+    return flush_stages(c, true);
 }
 
 // Jobs of the lane whose universes have all finished: results to the
@@ -1360,9 +1385,11 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
 // them (in job-slot order).
 fc_status lane_harvest(fc_ctx* c, Lane* L, std::vector<std::shared_ptr<LaneJob>>* done) {
     if (lane_idle(L)) return FC_OK;
-    std::vector<int32_t> left(kLaneJobs);
-    FC_CUDA(cudaMemcpyAsync(left.data(), L->job_left, kLaneJobs * 4, cudaMemcpyDeviceToHost, c->stream));
-    FC_TRY(sync(c));
+    std::vector<int32_t> left(kLaneJobs, 0);
+    if (L->n_active > 0) {  // with no universe active every job is complete
+        FC_CUDA(cudaMemcpyAsync(left.data(), L->job_left, kLaneJobs * 4, cudaMemcpyDeviceToHost, c->stream));
+        FC_TRY(sync(c));
+    }
     for (int j = 0; j < kLaneJobs; ++j) {
         std::shared_ptr<LaneJob> J = L->jobs[j];
         if (!J || left[j] != 0) continue;
@@ -1511,10 +1538,7 @@ fc_status run_points_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t
     c->stats = fc_stats{};
     c->acc = &c->stats;
     const long long launches0 = g_launches.load();
-    cudaEvent_t e0, e1, e2;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    cudaEventCreate(&e2);
+    cudaEvent_t e0 = c->run_ev[0], e1 = c->run_ev[1], e2 = c->run_ev[2];
     cudaEventRecord(e0, c->stream);
     fc_status st = run_sync(c, g, o, hps, U, seed, nullptr, dchi2, bestfit, nscans, nullptr, e1);
     if (st == FC_OK) {
@@ -1531,9 +1555,6 @@ fc_status run_points_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t
         c->stats.kernel_launches = g_launches.load() - launches0;
         c->stats.cache_slots = g->cap;
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaEventDestroy(e2);
     return st;
 }
 
@@ -1764,11 +1785,14 @@ fc_status fc_create(fc_ctx** out, int device, size_t hbm_budget_bytes, void* cud
         FC_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
         c->own_stream = true;
     }
-    FC_CUDA(cudaEventCreate(&c->ev_a));
-    FC_CUDA(cudaEventCreate(&c->ev_b));
-    FC_TRY(dalloc_t(c.get(), &c->status_dev, 1));
-    FC_TRY(dalloc_t(c.get(), &c->counters_dev, 16));
-    FC_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), c->stream));
+    for (cudaEvent_t& e : c->run_ev) FC_CUDA(cudaEventCreate(&e));
+    FC_TRY(dalloc_t(c.get(), &c->ctrl, 1));
+    c->status_dev = &c->ctrl->status;
+    c->counters_dev = c->ctrl->counters;
+    FC_CUDA(cudaMallocHost((void**)&c->ctrl_host, sizeof(Ctrl)));
+    FC_CUDA(cudaMallocHost((void**)&c->list_host, kListHost * sizeof(int32_t)));
+    memset(c->ctrl_host, 0, sizeof(Ctrl));
+    FC_CUDA(cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
     FC_CUDA(cudaStreamSynchronize(c->stream));
     *out = c.release();
     return FC_OK;
@@ -1787,8 +1811,14 @@ fc_status fc_destroy(fc_ctx* c) {
     for (auto& kv : c->allocs) cudaFree(kv.first);
     c->allocs.clear();
     if (c->own_stream) cudaStreamDestroy(c->stream);
-    if (c->ev_a) cudaEventDestroy(c->ev_a);
-    if (c->ev_b) cudaEventDestroy(c->ev_b);
+    for (cudaEvent_t e : c->run_ev)
+        if (e) cudaEventDestroy(e);
+    for (auto& e : c->stage_ev) {
+        cudaEventDestroy(e.first);
+        if (e.second) cudaEventDestroy(e.second);
+    }
+    cudaFreeHost(c->ctrl_host);
+    cudaFreeHost(c->list_host);
     delete c;
     return FC_OK;
 }
@@ -2118,6 +2148,7 @@ fc_status fc_covariance(fc_ctx* c, int32_t grid_id, int64_t q, double* A, double
     if (A) {
         std::vector<int32_t> qs{(int32_t)q}, slots;
         FC_TRY(ensure_slots(c, g, qs, FC_COV_ITERATE, false, false, &slots));
+        FC_TRY(check_status(c));
         FC_TRY(copy_out(c, A, g->A64 + (size_t)slots[0] * g->nfit * g->nfit, (size_t)g->nfit * g->nfit * 8));
     }
     if (L_sys) {

@@ -287,6 +287,7 @@ struct ResolveArgs {
     int2* tile_items;      // (first item, item count) of each quadrant's items (a quadrant shares one W)
     int2* tile_items2;     // the same for items2
     unsigned long long* n_resid;  // residual chi2 evaluated (all rounds)
+    const int* status;     // the context's status word: after a timeout the resolution does nothing
     int n_sm;
 };
 // Bits of a universe's round record (the FC_DECIDED_* values of fc.h).
@@ -327,9 +328,10 @@ struct UniverseState {
     const int32_t* job_of;
     int32_t* job_left;
 };
+// The first *count (device) of list, at most n, under slot_of[cur[u]], or ident_slot when >= 0.
 // Wdf given: the mixed path's double-float residuals; null: binary64 (plain path)
-void launch_finish(const int32_t* list, int64_t n, const int32_t* uslot_of_list, const int32_t* best,
-                   const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64,
+void launch_finish(const int32_t* list, int64_t n, const int32_t* count, int ident_slot, const int32_t* slot_of,
+                   const int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64,
                    const float* Wdf, double* dchi2, double* chi2min, cudaStream_t st);
 // advance: converged / exhausted universes -> finish list, others stay active
 void launch_advance(const int32_t* active, int64_t n_active, const int32_t* best, const UniverseState& us,

@@ -1704,8 +1704,10 @@ __global__ void __launch_bounds__(kBM) k_resolve_emit(ResolveArgs a) {
     const int64_t row = t * kBM + threadIdx.x;
     const int slot = a.quad_slot[row / kQuadRows];
     const int u = a.tile_univ[row];
+    // an aborted screen's candidates are incomplete (and may be unwritten): nothing is read of them
+    const bool aborted = (*a.status & kDevTimeout) != 0;
     RowDecision D;
-    decide_row(a, row, slot, u, D);
+    decide_row(a, row, slot, aborted ? -1 : u, D);
     int total = 0;
     const int off = block_excl_scan(D.ncodes, s_warp, &total);
     if (threadIdx.x == 0) {
@@ -1803,6 +1805,7 @@ __global__ void __launch_bounds__(32 * kRowsWarps) k_resid_rows(const ResolveArg
 }
 
 __global__ void __launch_bounds__(kBM) k_resolve_conclude(ResolveArgs a) {
+    if (*a.status & kDevTimeout) return;  // an aborted screen decides nothing
     __shared__ int s_nnext, s_nfb, s_n2[kQuads], s_cnt[3];
     __shared__ int s_base_next, s_base_fb, s_base2;
     const int64_t t = blockIdx.x;
@@ -1953,6 +1956,7 @@ __global__ void k_list_plan(ResolveArgs a, const int32_t* __restrict__ cand_coun
                             int64_t n_rows, const int32_t* __restrict__ n_rows_dev, ListPlan lp) {
     const int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (w >= n_rows || w >= *n_rows_dev) return;
+    if (*a.status & kDevTimeout) return;  // an aborted screen's counts are not read: no chunks, nothing handed on
     const int64_t row = rows[w];
     const int u = a.tile_univ[row];
     const int n0 = cand_count[row * 2], n1 = cand_count[row * 2 + 1];
@@ -2098,12 +2102,12 @@ __global__ void k_min_tau(const int32_t* __restrict__ tile_univ, int64_t n_rows,
 
 // ---------------------------------------------------------- finishing -------
 
-// One warp per finishing universe: chi2_p and chi2_min in residual form under
+// One warp per finishing universe (*count of list): chi2_p and chi2_min in residual form under
 // the last scan's covariance (A = W^T W), dchi2 = chi2_p - chi2_min.
 template <bool MODEL>
-__global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list, int64_t n,
-                                                 const int32_t* __restrict__ uslot, const int32_t* __restrict__ best,
-                                                 UniverseState us, const float* __restrict__ d, GridSpec gs,
+__global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list, const int32_t* __restrict__ count,
+                                                 int ident_slot, const int32_t* __restrict__ slot_of,
+                                                 const int32_t* __restrict__ best, UniverseState us, const float* __restrict__ d, GridSpec gs,
                                                  int nfit, const double* __restrict__ W64,
                                                  const float* __restrict__ Wdf, double* __restrict__ dchi2,
                                                  double* __restrict__ chi2min) {
@@ -2111,9 +2115,9 @@ __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list
     __shared__ double rp[4][kMaxBins], rm[4][kMaxBins], tt[4][kMaxBins];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * 4LL + w;
-    if (i >= n) return;
+    if (i >= *count) return;
     const int u = list[i];
-    const int slot = uslot[i];
+    const int slot = ident_slot >= 0 ? ident_slot : slot_of[us.cur[u]];
     const int p = us.pt[u];
     const int g = best[u];
     const float* du = d + (size_t)u * nfit;
@@ -2737,8 +2741,8 @@ void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaS
     k_resolve_tail<<<g3, 256, 0, st>>>(a);
 }
 
-void launch_finish(const int32_t* list, int64_t n, const int32_t* uslot, const int32_t* best, const UniverseState& us,
-                   const float* d, const GridSpec& gs, int nfit, const double* W64, const float* Wdf, double* dchi2,
+void launch_finish(const int32_t* list, int64_t n, const int32_t* count, int ident_slot, const int32_t* slot_of,
+                   const int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64, const float* Wdf, double* dchi2,
                    double* chi2min, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();
@@ -2747,7 +2751,7 @@ void launch_finish(const int32_t* list, int64_t n, const int32_t* uslot, const i
     const size_t smem = Wdf ? rows_smem(nfit) : 0;
     auto kern = gs.Sdf || !Wdf ? k_finish<false> : k_finish<true>;
     allow_smem(kern, smem);
-    kern<<<grid, 128, smem, st>>>(list, n, uslot, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
+    kern<<<grid, 128, smem, st>>>(list, count, ident_slot, slot_of, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
 }
 
 size_t wdf_bytes(int nfit) { return (size_t)df_blocks(nfit) * nfit * 8 * sizeof(float); }
