@@ -8,6 +8,7 @@
 // last scan's A.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <cooperative_groups.h>
 #include <float.h>
 
 #include <algorithm>
@@ -425,10 +426,7 @@ __global__ void k_centred(GridSpec gs, int64_t G, int K, double* __restrict__ Sc
 
 // ------------------------------------------------------------ covariances ---
 
-// The systematic factor is staged in shared memory as a packed lower triangle
-// (element (i, j), j <= i, at i(i+1)/2 + j) up to this N_full: 98 KB at 155,
-// 33 KB at N_full = 90, so six true points share an SM.
-constexpr int kCholPackN = 155;
+__host__ __device__ __forceinline__ int tri(int n) { return n * (n + 1) / 2; }
 
 // e -> (a, b) with 0 <= b <= a and e = a(a+1)/2 + b
 __device__ __forceinline__ void tri_decode(int e, int& a, int& b) {
@@ -438,107 +436,140 @@ __device__ __forceinline__ void tri_decode(int e, int& a, int& b) {
     b = e - a * (a + 1) / 2;
 }
 
-template <bool PACKED>
-__device__ __forceinline__ int lidx(int i, int j, int n) {
-    return PACKED ? i * (i + 1) / 2 + j : i * n + j;
+// Systematic Cholesky factor of a true point, in binary64.  Each element's
+// terms are subtracted in increasing k with a separately rounded multiply and
+// subtract, then divided by the pivot, so the factor is reproducible bit for
+// bit; any blocking that keeps that order gives it.  Bound by the narrow
+// binary64 pipe when points are many (a multiply and a subtract a term), by the
+// chain of roots and divisions when they are few.
+// Panels of kCholPanel columns: the panel is gathered into P, factored there
+// column by column (the thread that makes the next pivot takes its root while
+// the others update), and its terms are then subtracted from the trailing
+// triangle in one visit of each element.  The matrix is a packed lower triangle
+// in shared memory (161 KB at N_full = 200).
+// A cluster of CTAs shares one point when points are few: row i belongs to CTA
+// i mod C, which updates it; every CTA gathers the next panel from the owners'
+// shared memory and factors it for itself, so one cluster barrier a panel is
+// all they exchange.
+// Four points of N_full = 200 (one CTA a point, in global memory): 1680 -> 443 us;
+// one of 90: 212 -> 136 us; 10 000 of 90, where a CTA has a point either way and
+// the pipe decides: 6.4 -> 6.5 ms.
+constexpr int kCholPanel = 8;
+constexpr int kCholThreads = 256;
+constexpr int kCholCluster = 8;        // CTAs a point when points are few
+constexpr int kCholClusterPoints = 19; // 19 x 8 = the SMs
+
+constexpr int kCholLonePanel = 4;      // panel of a lone CTA
+
+inline size_t chol_sys_smem(int nf, int C) {
+    return (size_t)(tri(nf) + (C > 1 ? kCholPanel : kCholLonePanel) * nf) * sizeof(double);
 }
 
-// Cholesky in place on the lower triangle (packed, or row-major n x n with the
-// upper triangle zeroed at the end; shared or global memory); every element's
-// sum runs k = 0..j-1 with separately rounded multiply and subtract, so the
-// factor is reproducible bit for bit.
-template <bool PACKED>
-__device__ bool chol_inplace(double* L, int n) {
-    // Right-looking form: after column k is final, every trailing element
-    // (i >= j > k) subtracts L_ik L_jk.  Each element therefore still sees its
-    // terms in increasing k with a separately rounded multiply and subtract --
-    // the same sequence as the left-looking sum -- while the dependency chain
-    // shrinks to one step per column.
+__global__ void __launch_bounds__(kCholThreads, 6) k_chol_sys(FullSrc src, int nf, const double* __restrict__ F,
+                                                           const int64_t* __restrict__ ps, int gauss,
+                                                           double* __restrict__ L64, float* __restrict__ L32,
+                                                           float* __restrict__ s32, int* __restrict__ status) {
+    extern __shared__ double sT[];
+    __shared__ double s_row[kMaxBins];
     __shared__ double s_d;
     __shared__ int s_bad;
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
-            double acc = L[lidx<PACKED>(k, k, n)];
-            if (!(acc > 0.0)) {
-                s_bad = 1;
-                acc = 1.0;
-            }
-            s_d = __dsqrt_rn(acc);
-            L[lidx<PACKED>(k, k, n)] = s_d;
-        }
-        __syncthreads();
-        const double dk = s_d;
-        for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x)
-            L[lidx<PACKED>(i, k, n)] = __ddiv_rn(L[lidx<PACKED>(i, k, n)], dk);
-        __syncthreads();
-        // trailing update of the lower triangle, rows i > k, columns k < j <= i
-        const int m = n - k - 1;
-        const int cnt = m * (m + 1) / 2;
-        for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-            int a, b;
-            tri_decode(e, a, b);
-            const int i = k + 1 + a, jj = k + 1 + b;
-            L[lidx<PACKED>(i, jj, n)] =
-                __dsub_rn(L[lidx<PACKED>(i, jj, n)], __dmul_rn(L[lidx<PACKED>(i, k, n)], L[lidx<PACKED>(jj, k, n)]));
-        }
-        __syncthreads();
-    }
-    if (!PACKED) {
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            const int i = e / n, c = e % n;
-            if (c > i) L[e] = 0.0;
-        }
-        __syncthreads();
-    }
-    return s_bad == 0;
-}
-
-__global__ void k_chol_sys(FullSrc src, int nf, const double* __restrict__ F, const int64_t* __restrict__ ps,
-                           int gauss, double* __restrict__ L64, float* __restrict__ L32, float* __restrict__ s32,
-                           int* __restrict__ status) {
-    extern __shared__ double sL[];
-    __shared__ double s_row[kMaxBins];
-    const int ip = blockIdx.x;
-    stage_full_row(src, nf, ps[ip], s_row);
-    const double* s = s_row;
+    cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int ip = blockIdx.x / C;
+    const int n = nf, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int kWarps = kCholThreads / 32;
     double* Lg = L64 + (size_t)ip * nf * nf;
     float* Lf = L32 + (size_t)ip * nf * nf;
+    double* T = sT;             // packed; this CTA's rows (i % C == rank) are kept up to date
+    double* P = sT + tri(n);    // [kCholPanel][n]: column c of the panel by row
+    stage_full_row(src, nf, ps[ip], s_row);
+    const double* s = s_row;
+    if (tid == 0) s_bad = 0;
     // element (i, j), j <= i, of diag(s) F diag(s) (+ diag(s) in the Gaussian mode)
-    auto msys = [&](int i, int j) {
-        double v = __dmul_rn(__dmul_rn(s[i], F[i * nf + j]), s[j]);
-        if (gauss && i == j) v = __dadd_rn(v, s[i]);
-        return v;
+    for (int i = rank + C * warp; i < n; i += C * kWarps)
+        for (int j = lane; j <= i; j += 32) {
+            double v = __dmul_rn(__dmul_rn(s[i], F[i * nf + j]), s[j]);
+            if (gauss && i == j) v = __dadd_rn(v, s[i]);
+            T[tri(i) + j] = v;
+        }
+    auto meet = [&]() {
+        if (C > 1)
+            cluster.sync();
+        else
+            __syncthreads();
     };
-    bool ok;
-    if (nf <= kCholPackN) {
-        // packed in shared memory (the dependent sums run at shared-memory latency)
-        const int np = nf * (nf + 1) / 2;
-        for (int e = threadIdx.x; e < np; e += blockDim.x) {
-            int i, j;
-            tri_decode(e, i, j);
-            sL[e] = msys(i, j);
+    meet();
+    auto pivot = [&](double acc) {
+        if (!(acc > 0.0)) {
+            s_bad = 1;
+            acc = 1.0;
+        }
+        s_d = __dsqrt_rn(acc);
+    };
+    const int W = C > 1 ? kCholPanel : kCholLonePanel;
+    for (int p0 = 0; p0 < n; p0 += W) {
+        const int w = min(W, n - p0);
+        for (int e = tid; e < (n - p0) * W; e += kCholThreads) {
+            const int i = p0 + e / W, c = e % W;
+            if (c < w && p0 + c <= i) {
+                const double* own = C > 1 ? cluster.map_shared_rank(T, i % C) : T;
+                const double v = own[tri(i) + p0 + c];
+                P[c * n + i] = v;
+                if (e == 0) pivot(v);
+            }
         }
         __syncthreads();
-        ok = chol_inplace<true>(sL, nf);
-        for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) {
-            const int i = e / nf, j = e % nf;
-            const double v = (j <= i) ? sL[i * (i + 1) / 2 + j] : 0.0;
-            Lg[e] = v;
-            Lf[e] = __double2float_rn(v);
+        for (int c = 0; c < w; ++c) {
+            const int k = p0 + c;
+            const double dk = s_d;
+            double* Pc = P + c * n;
+            for (int i = k + tid; i < n; i += kCholThreads) Pc[i] = i == k ? dk : __ddiv_rn(Pc[i], dk);
+            __syncthreads();
+            // columns c + 1 .. w - 1 of the panel: rows on and below their diagonal
+            const int below = n - k - 1;
+            for (int e = tid; e < (w - c - 1) * below; e += kCholThreads) {
+                const int c2 = c + 1 + e / below, i = k + 1 + e % below;
+                if (p0 + c2 > i) continue;
+                const double v = __dsub_rn(P[c2 * n + i], __dmul_rn(Pc[i], Pc[p0 + c2]));
+                P[c2 * n + i] = v;
+                if (e == 0) pivot(v);  // (k + 1, k + 1)
+            }
+            __syncthreads();
         }
-    } else {
-        for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) {
-            const int i = e / nf, j = e % nf;
-            if (j <= i) Lg[e] = msys(i, j);
+        // the finished columns of this CTA's rows go straight out (T keeps what the others may still gather)
+        for (int e = tid; e < n * W; e += kCholThreads) {
+            const int i = e / W, c = e % W;
+            if (i % C != rank || c >= w) continue;
+            const double v = p0 + c <= i ? P[c * n + i] : 0.0;
+            Lg[i * n + p0 + c] = v;
+            Lf[i * n + p0 + c] = __double2float_rn(v);
         }
-        __syncthreads();
-        ok = chol_inplace<false>(Lg, nf);
-        for (int e = threadIdx.x; e < nf * nf; e += blockDim.x) Lf[e] = __double2float_rn(Lg[e]);
+        // trailing triangle
+        const int q0 = p0 + w;
+        auto update = [&](int i, int j) {
+            double x = T[tri(i) + j];
+#pragma unroll
+            for (int c = 0; c < kCholPanel; ++c)
+                if (c < w) x = __dsub_rn(x, __dmul_rn(P[c * n + i], P[c * n + j]));
+            T[tri(i) + j] = x;
+        };
+        if (C == 1) {
+            for (int e = tid; e < tri(n - q0); e += kCholThreads) {
+                int a, b;
+                tri_decode(e, a, b);
+                update(q0 + a, q0 + b);
+            }
+        } else {
+            // this CTA's rows from q0 on, a row per warp
+            for (int i = q0 + (rank - q0 % C + C) % C + C * warp; i < n; i += C * kWarps)
+                for (int j = q0 + lane; j <= i; j += 32) update(i, j);
+        }
+        meet();
     }
-    if (!ok && threadIdx.x == 0) atomicOr(status, kDevNotSpd);
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) s32[(size_t)ip * nf + i] = __double2float_rn(s[i]);
+    if (rank == 0) {
+        if (s_bad && tid == 0) atomicOr(status, kDevNotSpd);
+        for (int i = tid; i < nf; i += kCholThreads) s32[(size_t)ip * nf + i] = __double2float_rn(s[i]);
+    }
 }
 
 // One CTA per (slot, q): M(q) = C [diag(s) F diag(s) + diag(s)] C^T, L = chol(M),
@@ -558,7 +589,6 @@ __global__ void k_chol_sys(FullSrc src, int nf, const double* __restrict__ F, co
 // squares (in global memory above N_fit = 64): 597 covariances of N = 200 in
 // four launches 18.1 -> 11.3 ms, 10 500 of N = 120 30.1 -> 22.4 ms (their
 // multiply-adds alone take 4.1 and 15.7 ms), 10 000 of N = 45 2.8 -> 1.8 ms.
-__host__ __device__ __forceinline__ int tri(int n) { return n * (n + 1) / 2; }
 inline int build_cov_threads(int nfit) { return nfit > 120 ? 512 : 256; }
 inline size_t build_cov_smem(int nfit) { return (size_t)(tri(nfit) + 2 * nfit) * sizeof(double); }
 
@@ -2469,11 +2499,22 @@ void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t*
                      float* L32, float* s32, double*, int* status, cudaStream_t st) {
     if (P <= 0) return;
     count_launch();
-    const size_t smem = nf <= kCholPackN ? (size_t)nf * (nf + 1) / 2 * sizeof(double) : 0;
-    // the attribute belongs to the current device, so it is set at every launch (a cheap host call)
-    cudaFuncSetAttribute(k_chol_sys, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         kCholPackN * (kCholPackN + 1) / 2 * (int)sizeof(double));
-    k_chol_sys<<<P, 256, smem, st>>>(src, nf, F, ps, gauss, L64, L32, s32, status);
+    const int C = P <= kCholClusterPoints && nf > 2 * kCholPanel ? kCholCluster : 1;
+    const size_t smem = chol_sys_smem(nf, C);
+    allow_smem(k_chol_sys, smem);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)P * C);
+    cfg.blockDim = dim3(kCholThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)C;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_chol_sys, src, nf, F, ps, gauss, L64, L32, s32, status);
 }
 
 void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* coll, const double* F, const int32_t* q_list,

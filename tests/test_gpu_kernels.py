@@ -176,3 +176,23 @@ def test_fake_data_blocks(ctx, nf, collapse, U):
         want = oracle.fake_data(S, F, ps, 17, U, coll, n_fit, fluct)
         assert np.array_equal(got, want)
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- systematic factor: panels of 8 columns, one CTA or a cluster of 8 a point ----------------
+
+@pytest.mark.parametrize("nf", [1, 7, 8, 9, 16, 17, 24, 63, 90, 155, 156, 200])
+def test_systematic_factor(ctx, nf):
+    """Bit for bit the oracle's, for a lone point (a cluster) and through the fake data of many (a CTA each)."""
+    import oracle
+
+    S, F = _grid(40, nf, nf + 3)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    for q in (0, 39):
+        assert np.array_equal(fc.fc_covariance(ctx, gid, q, nf, nf, want_A=False)[1], oracle.chol_sys(S[q], F))
+    ps = np.arange(40, dtype=np.int64)
+    many = fc.fc_fake_data(ctx, gid, ps, 5, 3, nf)
+    for k in (0, 20, 39):
+        assert np.array_equal(fc.fc_fake_data(ctx, gid, ps[k:k + 1], 5, 3, nf)[0], many[k])
+    assert np.array_equal(many, oracle.fake_data(S, F, ps, 5, 3))
+    fc.fc_unload_grid(ctx, gid)
