@@ -169,22 +169,37 @@ __device__ __forceinline__ void rows_products(const ulonglong2* __restrict__ W, 
         const int i = i0 + lane;
         const ulonglong2* Wi = W + 2 * (i < n ? i : n - 1);
         const int nblk = min(nb, (i0 + 31) / 4 + 1);
+        constexpr int kAhead = B > 2 ? 2 : 4;
         df2x s02[B], s13[B];
 #pragma unroll
         for (int k = 0; k < B; ++k) s02[k] = s13[k] = df2x{0ull, 0ull};
-        ulonglong2 w0 = __ldg(Wi), w1 = __ldg(Wi + 1);
-#pragma unroll 2
-        for (int jb = 0; jb < nblk; ++jb) {
-            const ulonglong2 c0 = w0, c1 = w1;
-            if (jb + 1 < nblk) {  // the next block's W is on its way while this one is used
-                w0 = __ldg(Wi + (size_t)(jb + 1) * 2 * n);
-                w1 = __ldg(Wi + (size_t)(jb + 1) * 2 * n + 1);
-            }
+        // kAhead blocks of W are on their way while as many are used (past the last one, the last again):
+        // a warp alone on its scheduler waits for W, not for the pipe (a block ahead only: residuals of the
+        // 25x25 point 28 instead of 17 us a launch, of N = 200 289 instead of 134)
+        ulonglong2 w[2 * kAhead];
+        auto fetch = [&](int jb) {
 #pragma unroll
-            for (int k = 0; k < B; ++k) {
-                const ulonglong2 r0 = sr[(k * nb + jb) * 2], r1 = sr[(k * nb + jb) * 2 + 1];
-                s02[k] = df2_fma(s02[k], c0.x, c0.y, r0.x, r0.y);
-                s13[k] = df2_fma(s13[k], c1.x, c1.y, r1.x, r1.y);
+            for (int h = 0; h < kAhead; ++h) {
+                const ulonglong2* p = Wi + (size_t)min(jb + h, nblk - 1) * 2 * n;
+                w[2 * h] = __ldg(p);
+                w[2 * h + 1] = __ldg(p + 1);
+            }
+        };
+        fetch(0);
+        for (int jb = 0; jb < nblk; jb += kAhead) {
+            ulonglong2 c[2 * kAhead];
+#pragma unroll
+            for (int h = 0; h < 2 * kAhead; ++h) c[h] = w[h];
+            if (jb + kAhead < nblk) fetch(jb + kAhead);
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) {
+                if (jb + h >= nblk) break;
+#pragma unroll
+                for (int k = 0; k < B; ++k) {
+                    const ulonglong2 r0 = sr[(k * nb + jb + h) * 2], r1 = sr[(k * nb + jb + h) * 2 + 1];
+                    s02[k] = df2_fma(s02[k], c[2 * h].x, c[2 * h].y, r0.x, r0.y);
+                    s13[k] = df2_fma(s13[k], c[2 * h + 1].x, c[2 * h + 1].y, r1.x, r1.y);
+                }
             }
         }
         if (i < n) {
@@ -2021,8 +2036,10 @@ __global__ void k_list_plan(ResolveArgs a, const int32_t* __restrict__ cand_coun
 // takes the first minimum (lowest index among equal values) and publishes it.
 // The warp that completes a row's last chunk takes the first minimum over the
 // row's chunks and finishes (dchi2) or advances the row.
+// Four CTAs an SM where rows are stored: the lists of 128 points of 64^3 take
+// 38.4 ms, with the registers of three 40.6.
 template <bool MODEL>
-__global__ void __launch_bounds__(32 * kRowsWarps) k_list_chunks(ResolveArgs a, const int32_t* __restrict__ cand_count,
+__global__ void __launch_bounds__(32 * kRowsWarps, MODEL ? 3 : 4) k_list_chunks(ResolveArgs a, const int32_t* __restrict__ cand_count,
                                                                  const int32_t* __restrict__ rows, ListPlan lp) {
     extern __shared__ float4 s_rows[];
     const int n = a.nfit;

@@ -196,3 +196,32 @@ def test_systematic_factor(ctx, nf):
         assert np.array_equal(fc.fc_fake_data(ctx, gid, ps[k:k + 1], 5, 3, nf)[0], many[k])
     assert np.array_equal(many, oracle.fake_data(S, F, ps, 5, 3))
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- list rounds: long lists ------------------------------------------------------------------
+
+@pytest.mark.parametrize("n", [7, 33, 62, 77, 120, 199])
+def test_crowded_lists(ctx, n):
+    """Thousands of nearly equal spectra along one direction: long lists, the plain path's minimum, and ties
+    (every spectrum twice) to the lowest index."""
+    rng = np.random.default_rng(n)
+    b, f = rng.uniform(50.0, 500.0, n), rng.uniform(5.0, 50.0, n)
+    amp = np.concatenate([np.logspace(-5, 0, 3000), np.linspace(0.0, 1.0, 2001)])
+    S = b + amp[:, None] * np.sin(np.linspace(0.1, 9.0, n))[None, :] ** 2 * f
+    S = np.repeat(S, 2, axis=0)
+    _, F = _grid(4, n, n)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    pts = np.array([0, 5000, 9000], np.int64)
+    d, q = _data(S, pts, 30, 1)
+    chi2 = {}
+    for prec in (fc.FC_PREC_MIXED, fc.FC_PREC_FP64):
+        chi2[prec] = fc.fc_scan(ctx, gid, d, q, prec, 8)
+    best, c = chi2[fc.FC_PREC_MIXED]
+    b64, c64 = chi2[fc.FC_PREC_FP64]
+    np.testing.assert_allclose(c, c64, rtol=1e-9)
+    assert (best % 2 == 0).all()
+    # neighbours closer than the two paths' own rounding may change places
+    differ = best != b64
+    assert np.all(np.abs(best - b64)[differ] <= 4) and differ.mean() < 0.2
+    fc.fc_unload_grid(ctx, gid)
