@@ -159,6 +159,7 @@ struct Ctrl {
     int status;                       // kDev* flags, sticky until reported
 };
 constexpr int32_t kListHost = 4096;   // entries of a device list fetched along with its count
+constexpr size_t kStageHost = 256 * 1024;  // bytes of small host lists on their way to the device
 
 // Served job: a copy of the caller's arguments and its completion state.
 struct JobRec {
@@ -231,6 +232,8 @@ struct fc_ctx {
     Ctrl* ctrl_host = nullptr;       // pinned; the device's values as of the last read_ctrl
     bool ctrl_read = false;          // nothing that changes the counts was launched since then
     int32_t* list_host = nullptr;    // pinned [kListHost]
+    char* stage_host = nullptr;      // pinned [kStageHost]: sources of the copies launched since the last wait
+    size_t stage_used = 0;
     int* status_dev = nullptr;       // &ctrl->status
     unsigned long long* counters_dev = nullptr;  // ctrl->counters
     // stage timers: event pairs around the stages since the last flush_stages, and where each one counts
@@ -351,7 +354,28 @@ fc_status put_out(fc_ctx* c, void* dst, const void* host_src, size_t bytes) {
 
 fc_status sync(fc_ctx* c) {
     FC_CUDA(cudaStreamSynchronize(c->stream));
+    c->stage_used = 0;
     FC_CUDA(cudaGetLastError());
+    return FC_OK;
+}
+
+// Host data of this call to the device, for launches that nothing waits for: a
+// copy from pageable memory may still be reading it when the call returns (it
+// "might" be synchronous), so the bytes go through the context's pinned block
+// and the source may end as soon as this returns.  The block fills up until
+// the next wait; what does not fit is copied and waited for.
+fc_status to_device(fc_ctx* c, void* dst, const void* src, size_t bytes) {
+    if (bytes == 0) return FC_OK;
+    const size_t room = (bytes + 15) & ~(size_t)15;
+    if (room > kStageHost) {
+        FC_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream));
+        return sync(c);
+    }
+    if (c->stage_used + room > kStageHost) FC_TRY(sync(c));
+    char* at = c->stage_host + c->stage_used;
+    memcpy(at, src, bytes);
+    c->stage_used += room;
+    FC_CUDA(cudaMemcpyAsync(dst, at, bytes, cudaMemcpyHostToDevice, c->stream));
     return FC_OK;
 }
 
@@ -659,14 +683,14 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
     if (!evicted_q.empty()) {
         // evicted grid indices lose their slot on the device too
         std::vector<int32_t> minus(evicted_q.size(), -1);
-        FC_CUDA(cudaMemcpyAsync(dq, evicted_q.data(), evicted_q.size() * 4, cudaMemcpyHostToDevice, c->stream));
-        FC_CUDA(cudaMemcpyAsync(ds, minus.data(), minus.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        FC_TRY(to_device(c, dq, evicted_q.data(), evicted_q.size() * 4));
+        FC_TRY(to_device(c, ds, minus.data(), minus.size() * 4));
         launch_set_slots(dq, ds, (int)evicted_q.size(), g->slot_of, c->stream);
         c->acc->evicted += (int64_t)evicted_q.size();
     }
     if (!new_q.empty()) {
-        FC_CUDA(cudaMemcpyAsync(dq, new_q.data(), new_q.size() * 4, cudaMemcpyHostToDevice, c->stream));
-        FC_CUDA(cudaMemcpyAsync(ds, new_s.data(), new_s.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        FC_TRY(to_device(c, dq, new_q.data(), new_q.size() * 4));
+        FC_TRY(to_device(c, ds, new_s.data(), new_s.size() * 4));
         launch_build_cov(g->full(), g->nf, g->nfit, g->identity_collapse ? nullptr : g->collapse, g->F, dq, ds,
                          (int)new_q.size(), cov_mode == FC_COV_IDENTITY ? 2 : 0, g->A64, g->W64, g->A32, g->rho,
                          c->status_dev, c->stream);
@@ -676,7 +700,7 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
     }
     if (!q32_list.empty()) {
         FC_TRY(ensure_q32_storage(c, g));
-        FC_CUDA(cudaMemcpyAsync(ds, q32_list.data(), q32_list.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        FC_TRY(to_device(c, ds, q32_list.data(), q32_list.size() * 4));
         if (use_qvec_tc(g)) {
             if (!g->Wimg) FC_TRY(dalloc_t(c, &g->Wimg, (size_t)g->cap * 2 * g->K * g->K));
             if (!g->wnorm) FC_TRY(dalloc_t(c, &g->wnorm, (size_t)g->cap));
@@ -690,7 +714,7 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
     }
     if (!q64_list.empty()) {
         FC_TRY(ensure_q64_storage(c, g));
-        FC_CUDA(cudaMemcpyAsync(ds, q64_list.data(), q64_list.size() * 4, cudaMemcpyHostToDevice, c->stream));
+        FC_TRY(to_device(c, ds, q64_list.data(), q64_list.size() * 4));
         launch_qvec64(g->spec(), g->G, g->nfit, g->W64, ds, (int)q64_list.size(), g->G, g->Q64, c->stream);
     }
     return FC_OK;
@@ -913,7 +937,7 @@ fc_status lane_admit(fc_ctx* c, Lane* L, const std::shared_ptr<LaneJob>& J, cons
     const int64_t n = J->n;
     int64_t* ps_dev = nullptr;
     FC_TRY(scratch(c, "ps", (size_t)P, &ps_dev));
-    FC_CUDA(cudaMemcpyAsync(ps_dev, ps_host, (size_t)P * 8, cudaMemcpyHostToDevice, c->stream));
+    FC_TRY(to_device(c, ps_dev, ps_host, (size_t)P * 8));
     float* dst = L->d + (size_t)J->base * g->nfit;
     if (d_in) {
         FC_TRY(copy_in(c, dst, d_in, (size_t)n * g->nfit * sizeof(float)));
@@ -1240,10 +1264,9 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     FC_TRY(scratch(c, "big_off", (size_t)nb4, &d_off));
                     FC_TRY(scratch(c, "big_x", (size_t)nb4, &d_x));
                     FC_TRY(scratch(c, "big_nx", 1, &n_x));
-                    FC_CUDA(cudaMemcpyAsync(d_u, big_u.data(), (size_t)nb4 * 4, cudaMemcpyHostToDevice, c->stream));
-                    FC_CUDA(cudaMemcpyAsync(d_off, big_off.data(), (size_t)nb4 * 8, cudaMemcpyHostToDevice,
-                                            c->stream));
-                    FC_CUDA(cudaMemcpyAsync(dn, big_n.data(), (size_t)nb4 * 8, cudaMemcpyHostToDevice, c->stream));
+                    FC_TRY(to_device(c, d_u, big_u.data(), (size_t)nb4 * 4));
+                    FC_TRY(to_device(c, d_off, big_off.data(), (size_t)nb4 * 8));
+                    FC_TRY(to_device(c, dn, big_n.data(), (size_t)nb4 * 8));
                     count_launch();
                     k_scatter_lists<<<nb(nb4), 256, 0, c->stream>>>(d_u, nb4, d_off, dn, loff, lnum);
                     if (o.cov == FC_COV_IDENTITY)
@@ -1259,8 +1282,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     if (nx > 0) FC_TRY(exact_scan(d_x, nx, nullptr));
                 }
                 if (!exact_u.empty()) {
-                    FC_CUDA(cudaMemcpyAsync(d_u, exact_u.data(), exact_u.size() * 4, cudaMemcpyHostToDevice,
-                                            c->stream));
+                    FC_TRY(to_device(c, d_u, exact_u.data(), exact_u.size() * 4));
                     FC_TRY(exact_scan(d_u, (int64_t)exact_u.size(), nullptr));
                 }
                 return FC_OK;
@@ -1351,7 +1373,7 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 // the universes whose covariance index is in this part
                 FC_CUDA(cudaMemsetAsync(flag, 0, (size_t)g->G, c->stream));
                 FC_CUDA(cudaMemsetAsync(wn, 0, 4, c->stream));
-                FC_CUDA(cudaMemcpyAsync(wq, part.data(), part.size() * 4, cudaMemcpyHostToDevice, c->stream));
+                FC_TRY(to_device(c, wq, part.data(), part.size() * 4));
                 count_launch(2);
                 k_flag_list<<<nb((int64_t)part.size()), 256, 0, c->stream>>>(wq, (int)part.size(), flag);
                 k_select_cur<<<nb(n_active), 256, 0, c->stream>>>(active, n_active, cur0, flag, wl, wn);
@@ -1436,7 +1458,7 @@ fc_status lane_drop_cancelled(fc_ctx* c, Lane* L) {
     if (hit.empty() || L->n_active == 0) return FC_OK;
     int32_t* cnt = nullptr;
     FC_TRY(scratch(c, "dropcnt", 1, &cnt));
-    FC_CUDA(cudaMemcpyAsync(L->job_dead, dead.data(), kLaneJobs, cudaMemcpyHostToDevice, c->stream));
+    FC_TRY(to_device(c, L->job_dead, dead.data(), kLaneJobs));
     FC_CUDA(cudaMemsetAsync(cnt, 0, 4, c->stream));
     count_launch();
     k_drop_jobs<<<nb(L->n_active), 256, 0, c->stream>>>(L->active, L->n_active, L->job_of, L->job_dead, L->next, cnt);
@@ -1513,7 +1535,10 @@ fc_status run_sync(fc_ctx* c, Grid* g, const fc_opts& o, const std::vector<int64
     if (st == FC_OK) st = lane_harvest(c, L, &done);
     if (st == FC_OK && (done.size() != 1 || !lane_idle(L)))
         st = fail(FC_ERR_STATE, "internal: synchronous job did not complete");
-    if (st != FC_OK) lane_reset(L);
+    if (st != FC_OK) {
+        cudaStreamSynchronize(c->stream);  // the caller's data may still be on its way
+        lane_reset(L);
+    }
     c->last_base = J->base;
     c->last_n = st == FC_OK ? n : -1;
     return st;
@@ -1574,7 +1599,7 @@ fc_status fake_data_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t 
     double* L64 = nullptr;
     float *L32 = nullptr, *s32 = nullptr, *d = nullptr;
     FC_TRY(scratch(c, "ps", (size_t)P, &ps_dev));
-    FC_CUDA(cudaMemcpyAsync(ps_dev, hps.data(), (size_t)P * 8, cudaMemcpyHostToDevice, c->stream));
+    FC_TRY(to_device(c, ps_dev, hps.data(), (size_t)P * 8));
     FC_TRY(scratch(c, "L64", (size_t)P * g->nf * g->nf, &L64));
     FC_TRY(scratch(c, "L32", (size_t)P * g->nf * g->nf, &L32));
     FC_TRY(scratch(c, "s32", (size_t)P * g->nf, &s32));
@@ -1791,6 +1816,7 @@ fc_status fc_create(fc_ctx** out, int device, size_t hbm_budget_bytes, void* cud
     c->counters_dev = c->ctrl->counters;
     FC_CUDA(cudaMallocHost((void**)&c->ctrl_host, sizeof(Ctrl)));
     FC_CUDA(cudaMallocHost((void**)&c->list_host, kListHost * sizeof(int32_t)));
+    FC_CUDA(cudaMallocHost((void**)&c->stage_host, kStageHost));
     memset(c->ctrl_host, 0, sizeof(Ctrl));
     FC_CUDA(cudaMemsetAsync(c->ctrl, 0, sizeof(Ctrl), c->stream));
     FC_CUDA(cudaStreamSynchronize(c->stream));
@@ -1819,6 +1845,7 @@ fc_status fc_destroy(fc_ctx* c) {
     }
     cudaFreeHost(c->ctrl_host);
     cudaFreeHost(c->list_host);
+    cudaFreeHost(c->stage_host);
     delete c;
     return FC_OK;
 }
@@ -2308,7 +2335,7 @@ fc_status fc_fc_region_adaptive(fc_ctx* c, int32_t grid_id, const int64_t* ps, i
         FC_TRY(scratch(c, "ad_cnt", (size_t)Pr, &dcnt));
         FC_TRY(run_sync(c, g, o, rps, (int32_t)U_r, seed + (uint64_t)round, nullptr, dx, nullptr, nullptr, nullptr,
                         nullptr));
-        FC_CUDA(cudaMemcpyAsync(dthr, rthr.data(), (size_t)Pr * 8, cudaMemcpyHostToDevice, c->stream));
+        FC_TRY(to_device(c, dthr, rthr.data(), (size_t)Pr * 8));
         FC_CUDA(cudaMemsetAsync(dcnt, 0, (size_t)Pr * 8, c->stream));
         launch_count_below(dx, (int)Pr, (int)U_r, dthr, dcnt, c->stream);
         FC_CUDA(cudaMemcpyAsync(rcnt.data(), dcnt, (size_t)Pr * 8, cudaMemcpyDeviceToHost, c->stream));

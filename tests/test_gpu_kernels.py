@@ -225,3 +225,20 @@ def test_crowded_lists(ctx, n):
     differ = best != b64
     assert np.all(np.abs(best - b64)[differ] <= 4) and differ.mean() < 0.2
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- host lists on their way to the device ----------------------------------------------------
+
+def test_long_host_lists(ctx):
+    """A list longer than the staging block, and lists that fill it up between two waits: every point of a grid
+    as a true point, against the same points alone."""
+    S, F = _grid(192 * 192, 2, 8)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    opts = dict(precision=fc.FC_PREC_FP64, cov=fc.FC_COV_FIXED)
+    ps = np.arange(len(S), dtype=np.int64)[::-1].copy()
+    d, b, ns = fc.fc_run_points(ctx, gid, ps, 3, 1, opts=opts)
+    for k in (0, 1, 20000, len(ps) - 1):
+        d1, b1, n1 = fc.fc_run_points(ctx, gid, ps[k:k + 1], 3, 1, opts=opts)
+        assert np.array_equal(d[k], d1[0]) and np.array_equal(b[k], b1[0]) and np.array_equal(ns[k], n1[0])
+    fc.fc_unload_grid(ctx, gid)
