@@ -154,7 +154,8 @@ struct Scratch {
 // pinned mirror, so that a decision costs one small copy and one wait: the
 // counts of a scan, its counters, and the status word the kernels raise.
 struct Ctrl {
-    int32_t cnts[8];                  // [1] failed rows, [2] continuing, [3] finishing, [4] failed again, [5] tiles, [6] rows
+    int32_t cnts[8];                  // [1] failed rows, [2] continuing, [3] finishing, [4] failed again, [5] tiles, [6] rows,
+                                      // [7] universes of a wave
     unsigned long long counters[16];  // see scan_once
     int status;                       // kDev* flags, sticky until reported
 };
@@ -1355,11 +1356,10 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
         } else {
             FC_TRY(stage_end(c, &S->ms_cov));
             uint8_t* flag = nullptr;
-            int32_t *wq = nullptr, *wl = nullptr, *wn = nullptr, *cur0 = nullptr;
+            int32_t *wq = nullptr, *wl = nullptr, *wn = cnts + 7, *cur0 = nullptr;
             FC_TRY(scratch(c, "wave_flag", (size_t)g->G, &flag));
             FC_TRY(scratch(c, "wave_q", (size_t)wave, &wq));
             FC_TRY(scratch(c, "wave_list", (size_t)n_active, &wl));
-            FC_TRY(scratch(c, "wave_n", 1, &wn));
             FC_TRY(scratch(c, "wave_cur0", (size_t)n_active, &cur0));
             // the waves partition the universes by their covariance index before any of them
             // moves on (a universe advanced by one wave must not join a later one)
@@ -1377,9 +1377,11 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 count_launch(2);
                 k_flag_list<<<nb((int64_t)part.size()), 256, 0, c->stream>>>(wq, (int)part.size(), flag);
                 k_select_cur<<<nb(n_active), 256, 0, c->stream>>>(active, n_active, cur0, flag, wl, wn);
-                int32_t n_w = 0;
-                FC_CUDA(cudaMemcpyAsync(&n_w, wn, 4, cudaMemcpyDeviceToHost, c->stream));
                 FC_TRY(ensure_slots(c, g, part, o.cov, mixed, !mixed, nullptr));
+                FC_TRY(read_ctrl(c));
+                c->ctrl_read = false;
+                const int32_t n_w = h_cnts[7];
+                if (n_w <= 0) return fail(FC_ERR_STATE, "internal: a wave of no universes");
                 launch_lookup_slots(wl, n_w, cur, g->slot_of, uslot, c->stream);
                 FC_TRY(stage_end(c, &S->ms_cov));
                 FC_TRY(scan_list(wl, n_w, uslot));

@@ -207,3 +207,20 @@ def test_scan_waves_when_cache_is_small(fc, ctx, prec):
     for a, b in zip(got, ref):
         np.testing.assert_array_equal(a, b)
     fc.fc_unload_grid(ctx, gid)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("slots", [2, 3, 9])
+def test_waves_of_few_covariances(fc, ctx, prec, slots):
+    """Caches of a few slots: a scan is many waves, some of one covariance and one universe."""
+    w = workloads.cfg1()
+    gid = _load(fc, ctx, w)
+    pts = np.array([0, 77, 312, 624], np.int64)
+    ref = _run_all(fc, ctx, gid, pts, 6, 40, precision=prec)
+    fc.fc_set_frac_cov(ctx, gid, w.F)
+    fc.fc_set_tuning(ctx, gid, cache_slots=slots)
+    got = _run_all(fc, ctx, gid, pts, 6, 40, precision=prec)
+    assert fc.fc_get_stats(ctx)["scan_waves"] > 2
+    for a, b in zip(got, ref):
+        np.testing.assert_array_equal(a, b)
+    fc.fc_unload_grid(ctx, gid)
