@@ -158,6 +158,7 @@ struct Ctrl {
                                       // [7] universes of a wave
     unsigned long long counters[16];  // see scan_once
     int status;                       // kDev* flags, sticky until reported
+    int32_t sync_left;                // universes of a synchronous call that have not finished (its lane's job_left)
 };
 constexpr int32_t kListHost = 4096;   // entries of a device list fetched along with its count
 constexpr size_t kStageHost = 256 * 1024;  // bytes of small host lists on their way to the device
@@ -208,7 +209,7 @@ struct Lane {
     float* thr = nullptr;
     int32_t *active = nullptr, *next = nullptr, *fin = nullptr, *uslot = nullptr;
     int32_t *fb = nullptr, *fb2 = nullptr, *fbslot = nullptr;
-    int32_t* job_left = nullptr;  // [kLaneJobs]
+    int32_t* job_left = nullptr;  // [kLaneJobs]; of the synchronous lane, which holds one job: [1], in the control block
     uint8_t* job_dead = nullptr;  // [kLaneJobs]
     int64_t n_active = 0;
     int64_t n_first = 0;          // universes admitted since the last scan
@@ -838,6 +839,7 @@ fc_status distinct_cur(fc_ctx* c, Grid* g, const int32_t* active, int64_t n_acti
 // ------------------------------------------------------------------ lanes ---
 
 void lane_free(fc_ctx* c, Lane* L) {
+    if (c->ctrl && L->job_left == &c->ctrl->sync_left) L->job_left = nullptr;
     for (void* p : {(void*)L->d, (void*)L->cur, (void*)L->pt, (void*)L->best, (void*)L->job_of, (void*)L->nscan,
                     (void*)L->maxit, (void*)L->rmask, (void*)L->dchi2, (void*)L->chi2min, (void*)L->thr, (void*)L->active,
                     (void*)L->next, (void*)L->fin, (void*)L->uslot, (void*)L->fb, (void*)L->fb2, (void*)L->fbslot,
@@ -884,7 +886,10 @@ fc_status lane_alloc(fc_ctx* c, Lane* L, Grid* g, const fc_opts& o, int64_t cap)
     A(&L->fb, cap);
     A(&L->fb2, cap);
     A(&L->fbslot, cap);
-    A(&L->job_left, kLaneJobs);
+    if (L == &c->sync_lane)
+        L->job_left = &c->ctrl->sync_left;
+    else
+        A(&L->job_left, kLaneJobs);
     A(&L->job_dead, kLaneJobs);
     if (st != FC_OK) {
         lane_free(c, L);
@@ -1410,10 +1415,18 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
 fc_status lane_harvest(fc_ctx* c, Lane* L, std::vector<std::shared_ptr<LaneJob>>* done) {
     if (lane_idle(L)) return FC_OK;
     std::vector<int32_t> left(kLaneJobs, 0);
-    if (L->n_active > 0) {  // with no universe active every job is complete
+    if (L == &c->sync_lane) {  // job slot 0; it came with the scan's last read of the control block
+        if (!c->ctrl_read) FC_TRY(read_ctrl(c));
+        left[0] = c->ctrl_host->sync_left;
+    } else {
         FC_CUDA(cudaMemcpyAsync(left.data(), L->job_left, kLaneJobs * 4, cudaMemcpyDeviceToHost, c->stream));
         FC_TRY(sync(c));
     }
+    // the universes' own count against the scan's: a universe that left the active list unfinished is an error,
+    // not a job that never completes
+    for (int j = 0; j < kLaneJobs; ++j)
+        if (L->jobs[j] && left[j] != 0 && L->n_active == 0)
+            return fail(FC_ERR_STATE, "internal: universes left the scan unfinished");
     for (int j = 0; j < kLaneJobs; ++j) {
         std::shared_ptr<LaneJob> J = L->jobs[j];
         if (!J || left[j] != 0) continue;
