@@ -244,7 +244,8 @@ FC_API fc_status fc_covariance(fc_ctx* ctx, int32_t grid_id, int64_t q, double* 
  * d [U][N_fit] float32, q_cov [U] int64.  Outputs [U]: best (int64 first
  * index of the minimum), chi2_min (float64, residual form).  precision selects
  * the plain binary64 scan or the tensor-core screen with certified double-float
- * rescoring.  Errors as above. */
+ * rescoring.  Data for which no chi2 is a number (not finite, or so large that
+ * it overflows) has no minimum: best -1, chi2_min NaN.  Errors as above. */
 FC_API fc_status fc_scan(fc_ctx* ctx, int32_t grid_id, const float* d, const int64_t* q_cov, int32_t U,
                   int32_t precision, int32_t top_k, int64_t* best, double* chi2_min);
 

@@ -1006,6 +1006,8 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
     us.maxit = L->maxit;
     us.job_of = L->job_of;
     us.job_left = L->job_left;
+    us.status = c->status_dev;
+    us.G = g->G;
     // counts ([2], the continuing universes, is the whole scan's) and counters; not the status
     FC_CUDA(cudaMemsetAsync(c->ctrl, 0, offsetof(Ctrl, status), c->stream));
     c->ctrl_read = false;

@@ -320,6 +320,10 @@ void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaS
 // ---- final residual-form chi2 and dchi2 ----
 // Per-universe state of a scan: cur (covariance index), pt (true point),
 // nscan (scans done), maxit (limit), job_of / job_left (completion counting).
+// status: the context's status word; while a kernel has raised it, what the
+// scan read may be unwritten, and no universe advances or finishes.
+// G: grid points; a minimum outside [0, G) is none (no chi2 of the universe
+// compares, its data being too large or not a number).
 struct UniverseState {
     int32_t* cur;
     const int32_t* pt;
@@ -327,11 +331,14 @@ struct UniverseState {
     const int8_t* maxit;
     const int32_t* job_of;
     int32_t* job_left;
+    const int* status;
+    int64_t G;
 };
 // The first *count (device) of list, at most n, under slot_of[cur[u]], or ident_slot when >= 0.
 // Wdf given: the mixed path's double-float residuals; null: binary64 (plain path)
+// A universe without a minimum gets best = -1 and NaN.
 void launch_finish(const int32_t* list, int64_t n, const int32_t* count, int ident_slot, const int32_t* slot_of,
-                   const int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64,
+                   int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64,
                    const float* Wdf, double* dchi2, double* chi2min, cudaStream_t st);
 // advance: converged / exhausted universes -> finish list, others stay active
 void launch_advance(const int32_t* active, int64_t n_active, const int32_t* best, const UniverseState& us,

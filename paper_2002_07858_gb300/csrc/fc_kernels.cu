@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <cooperative_groups.h>
 #include <float.h>
+#include <math_constants.h>
 
 #include <algorithm>
 #include <cstdint>
@@ -1898,8 +1899,8 @@ __global__ void __launch_bounds__(kBM) k_resolve_conclude(ResolveArgs a) {
                 bg = D.g[c];
             }
         }
-        bool ok = !D.full || (D.min_ub < D.tau);
-        if (!ok) ok = (double)D.tau > (bchi - cu) + 1e-9 * (fabs(bchi) + fabs(cu));
+        bool ok = (!D.full || (D.min_ub < D.tau)) && bg != INT32_MAX;
+        if (!ok && bg != INT32_MAX) ok = (double)D.tau > (bchi - cu) + 1e-9 * (fabs(bchi) + fabs(cu));
         if (ok) {
             state = 1;
             g_best = bg;
@@ -2107,11 +2108,15 @@ __global__ void __launch_bounds__(32 * kRowsWarps, MODEL ? 3 : 4) k_list_chunks(
         if (lane == 0 && a.rmask) a.rmask[u] |= a.round_bit;
         if (lane == 0 && a.n_resid) atomicAdd(a.n_resid, (unsigned long long)(n0 + n1));
         const int32_t cur_u = a.cur[u];
-        const bool finishing = (bg == cur_u) || (a.nscan[u] + 1 >= a.maxit[u]);
+        const bool none = bg == INT32_MAX;  // no chi2 of the list compares: best -1, NaN (as k_finish)
+        const bool finishing = none || (bg == cur_u) || (a.nscan[u] + 1 >= a.maxit[u]);
         if (finishing) {
             const int p = a.pt[u];
             double cp = 0.0;
-            if (p != bg) {
+            if (none) {
+                bg = -1;
+                bv = CUDART_NAN;
+            } else if (p != bg) {
                 rows_stage(sm, 0, n, srow<MODEL>(a.gs, nullptr, p), du, lane);
                 cp = rows_chi2(W, n, sm, 1, lane);
                 if (lane == 0 && a.n_resid) atomicAdd(a.n_resid, 1ull);
@@ -2154,7 +2159,7 @@ __global__ void k_min_tau(const int32_t* __restrict__ tile_univ, int64_t n_rows,
 template <bool MODEL>
 __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list, const int32_t* __restrict__ count,
                                                  int ident_slot, const int32_t* __restrict__ slot_of,
-                                                 const int32_t* __restrict__ best, UniverseState us, const float* __restrict__ d, GridSpec gs,
+                                                 int32_t* __restrict__ best, UniverseState us, const float* __restrict__ d, GridSpec gs,
                                                  int nfit, const double* __restrict__ W64,
                                                  const float* __restrict__ Wdf, double* __restrict__ dchi2,
                                                  double* __restrict__ chi2min) {
@@ -2162,8 +2167,17 @@ __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list
     __shared__ double rp[4][kMaxBins], rm[4][kMaxBins], tt[4][kMaxBins];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i = blockIdx.x * 4LL + w;
-    if (i >= *count) return;
+    if (i >= *count || *us.status) return;
     const int u = list[i];
+    if (best[u] < 0 || best[u] >= us.G) {  // no row to read
+        if (lane == 0) {
+            best[u] = -1;
+            dchi2[u] = CUDART_NAN;
+            if (chi2min) chi2min[u] = CUDART_NAN;
+            atomicSub(&us.job_left[us.job_of[u]], 1);
+        }
+        return;
+    }
     const int slot = ident_slot >= 0 ? ident_slot : slot_of[us.cur[u]];
     const int p = us.pt[u];
     const int g = best[u];
@@ -2197,16 +2211,18 @@ __global__ void __launch_bounds__(128) k_finish(const int32_t* __restrict__ list
 }
 
 // exact-path bookkeeping: a universe finishes when its minimum repeats its
-// covariance index or it used its last scan; the others move on
+// covariance index, when it has none, or when it used its last scan; the
+// others move on
 __global__ void k_advance(const int32_t* __restrict__ active, int64_t n, const int32_t* __restrict__ best,
                           UniverseState us, int32_t* __restrict__ next_active, int32_t* __restrict__ n_next,
                           int32_t* __restrict__ fin, int32_t* __restrict__ n_fin) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || *us.status) return;
     const int u = active[i];
     const int done = us.nscan[u] + 1;
     us.nscan[u] = (int8_t)done;
-    if (best[u] == us.cur[u] || done >= us.maxit[u]) {
+    const bool none = best[u] < 0 || best[u] >= us.G;
+    if (none || best[u] == us.cur[u] || done >= us.maxit[u]) {
         fin[atomicAdd(n_fin, 1)] = u;
     } else {
         us.cur[u] = best[u];
@@ -2800,7 +2816,7 @@ void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaS
 }
 
 void launch_finish(const int32_t* list, int64_t n, const int32_t* count, int ident_slot, const int32_t* slot_of,
-                   const int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64, const float* Wdf, double* dchi2,
+                   int32_t* best, const UniverseState& us, const float* d, const GridSpec& gs, int nfit, const double* W64, const float* Wdf, double* dchi2,
                    double* chi2min, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();

@@ -1,0 +1,98 @@
+"""Calls that fail, what they leave behind, and data that has no minimum."""
+import numpy as np
+import pytest
+
+import paper_2002_07858_gb300 as fc
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+PRECISIONS = [fc.FC_PREC_FP64, fc.FC_PREC_MIXED]
+
+
+@pytest.fixture()
+def ctx():
+    fc.load()
+    c = fc.fc_create(0)
+    yield c
+    fc.fc_destroy(c)
+
+
+@pytest.fixture(scope="module")
+def grid():
+    S, F, _ = workloads.osc_2d(20, 20, 40, seed=4)
+    return S, F
+
+
+def _indefinite(F):
+    """Symmetric and finite, but diag(s) F diag(s) (+ diag(s)) has a negative diagonal entry for s > 1."""
+    bad = F.copy()
+    bad[7, 7] = -1.0
+    return bad
+
+
+def _not_spd(call):
+    with pytest.raises(fc.FCError) as e:
+        call()
+    assert e.value.status == fc.FC_ERR_NOT_SPD
+
+
+# ---- covariances that are not positive definite ---------------------------------------------
+
+CALLS = {
+    "scan": lambda c, g, d, prec: fc.fc_scan(c, g, d, np.arange(len(d)), prec, 8),
+    "data": lambda c, g, d, prec: fc.fc_data_dchi2(c, g, d[0], np.array([3, 9]), opts=dict(precision=prec)),
+    "data_fixed": lambda c, g, d, prec: fc.fc_data_dchi2(c, g, d[0], np.array([3]), opts=dict(precision=prec,
+                                                                                           cov=fc.FC_COV_FIXED)),
+    "points": lambda c, g, d, prec: fc.fc_run_points(c, g, np.array([5, 300]), 1, 30, opts=dict(precision=prec)),
+    "points_identity": lambda c, g, d, prec: fc.fc_run_points(c, g, np.array([5, 300]), 1, 30, opts=dict(
+        precision=prec, cov=fc.FC_COV_IDENTITY)),
+    "points_gauss_identity": lambda c, g, d, prec: fc.fc_run_points(c, g, np.array([5]), 1, 30, opts=dict(
+        precision=prec, cov=fc.FC_COV_IDENTITY, fluct=fc.FC_FLUCT_GAUSS)),
+}
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("name", list(CALLS))
+def test_not_spd_is_reported_and_the_context_goes_on(ctx, grid, name, prec):
+    S, F = grid
+    d = np.random.default_rng(0).poisson(S[:24]).astype(np.float32)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    ref = CALLS[name](ctx, gid, d, prec)
+    fc.fc_set_frac_cov(ctx, gid, _indefinite(F))
+    _not_spd(lambda: CALLS[name](ctx, gid, d, prec))
+    fc.fc_set_frac_cov(ctx, gid, F)
+    for a, b in zip(CALLS[name](ctx, gid, d, prec), ref):
+        assert np.array_equal(a, b)
+
+
+def test_not_spd_covariance_and_factor(ctx, grid):
+    S, F = grid
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, _indefinite(F))
+    _not_spd(lambda: fc.fc_covariance(ctx, gid, 5, 40, 40, want_L=False))
+    _not_spd(lambda: fc.fc_covariance(ctx, gid, 5, 40, 40, want_A=False))
+    _not_spd(lambda: fc.fc_fake_data(ctx, gid, np.array([5]), 1, 3, 40))
+
+
+# ---- data without a minimum -----------------------------------------------------------------
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("G", [1, 400, 3 * 256 + 1])
+def test_universe_without_a_minimum(ctx, prec, G):
+    """NaN data: best -1 and chi2 NaN for that universe alone, the others as without it."""
+    S, F, _ = workloads.osc_2d(28, 28, 40, seed=4)
+    S = np.ascontiguousarray(S[:G])
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    d = np.random.default_rng(1).poisson(S[np.arange(70) % G]).astype(np.float32)
+    q = np.arange(70) % G
+    best, chi2 = fc.fc_scan(ctx, gid, d, q, prec, 8)
+    bad = d.copy()
+    bad[[0, 33], [2, 39]] = np.nan
+    b, c = fc.fc_scan(ctx, gid, bad, q, prec, 8)
+    none = np.zeros(70, bool)
+    none[[0, 33]] = True
+    assert np.array_equal(b[~none], best[~none]) and np.array_equal(c[~none], chi2[~none])
+    assert (b[none] == -1).all() and np.isnan(c[none]).all()
