@@ -1851,7 +1851,10 @@ __global__ void __launch_bounds__(32 * kRowsWarps) k_resid_rows(const ResolveArg
 }
 
 __global__ void __launch_bounds__(kBM) k_resolve_conclude(ResolveArgs a) {
-    if (*a.status & kDevTimeout) return;  // an aborted screen decides nothing
+    if (*a.status & kDevTimeout) {  // an aborted screen decides nothing, and leaves no items to k_resid_tiles
+        if (threadIdx.x < kQuads) a.tile_items2[blockIdx.x * (int64_t)kQuads + threadIdx.x] = make_int2(0, 0);
+        return;
+    }
     __shared__ int s_nnext, s_nfb, s_n2[kQuads], s_cnt[3];
     __shared__ int s_base_next, s_base_fb, s_base2;
     const int64_t t = blockIdx.x;

@@ -96,3 +96,26 @@ def test_universe_without_a_minimum(ctx, prec, G):
     none[[0, 33]] = True
     assert np.array_equal(b[~none], best[~none]) and np.array_equal(c[~none], chi2[~none])
     assert (b[none] == -1).all() and np.isnan(c[none]).all()
+
+
+# ---- a screen whose waits run out ------------------------------------------------------------
+
+@pytest.mark.parametrize("stop_after", [0, 1, 3])
+@pytest.mark.parametrize("G,n,P,U", [(400, 40, 1, 24576),      # tiles for every SM: one thread per residual
+                                     (400, 16, 200, 128),      # the same with a covariance per tile
+                                     (256 * 40, 20, 2, 33)])   # few tiles: the grid split over the SMs
+def test_screen_timeout_leaves_no_items(ctx, G, n, P, U, stop_after):
+    """After an aborted screen nothing is rescored from what an earlier launch left behind, and the context goes on."""
+    side = int(np.ceil(np.sqrt(G)))
+    S, F, _ = workloads.osc_2d(side, side, n, seed=6)
+    gid = fc.fc_load_grid(ctx, S[:G])
+    fc.fc_set_frac_cov(ctx, gid, F)
+    ps = np.linspace(0, G - 1, P).astype(np.int64)
+    ref = fc.fc_run_points(ctx, gid, ps, 2, U)
+    fc.fc_set_wait_test(ctx, 150_000_000, stop_after)
+    with pytest.raises(fc.FCError) as e:
+        fc.fc_run_points(ctx, gid, ps, 3, U)
+    assert e.value.status == fc.FC_ERR_TIMEOUT
+    fc.fc_set_wait_test(ctx, 0, -1)
+    for a, b in zip(fc.fc_run_points(ctx, gid, ps, 2, U), ref):
+        assert np.array_equal(a, b)
