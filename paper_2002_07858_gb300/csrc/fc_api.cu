@@ -141,6 +141,7 @@ struct Grid {
     uint16_t* Qb3 = nullptr;         // [cap][G_pad][8] bf16 q-step rows of the screen
     double* Q64 = nullptr;           // [cap][G]   (plain)
     std::vector<uint8_t> q32_ready, q64_ready;
+    bool unread = false;             // covariances or q-vectors launched whose status the host has not read yet
     fc_tuning tune{};                // kernel choices (all zero: built-in)
     int busy = 0;                    // queued jobs referencing the grid
 };
@@ -381,12 +382,20 @@ fc_status to_device(fc_ctx* c, void* dst, const void* src, size_t bytes) {
     return FC_OK;
 }
 
-// The control block as of now (waits for the stream), and the errors the kernels raised.
+void reset_cache(fc_ctx* c, Grid* g);
+
+// The control block as of now (waits for the stream), and the errors the kernels raised.  With an error the
+// grids whose covariances or q-vectors were launched since the last read forget them: one that is not
+// positive definite was never written, and the next call has to build it and fail again, not use it.
 fc_status read_ctrl(fc_ctx* c) {
     FC_CUDA(cudaMemcpyAsync(c->ctrl_host, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
     FC_TRY(sync(c));
     c->ctrl_read = true;
     const int st = c->ctrl_host->status;
+    for (auto& kv : c->grids) {
+        if (st && kv.second->unread) reset_cache(c, kv.second.get());
+        kv.second->unread = false;
+    }
     if (st) {
         FC_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), c->stream));
         if (st & kDevTimeout) return fail(FC_ERR_TIMEOUT, "a device-side wait timed out");
@@ -396,7 +405,13 @@ fc_status read_ctrl(fc_ctx* c) {
     return FC_OK;
 }
 
-fc_status check_status(fc_ctx* c) { return read_ctrl(c); }
+// After a call that failed half-way: waits for what it launched (its sources may end with it) and takes the
+// status it left, which is not the next call's.  The error and its message stay the call's own.
+void settle(fc_ctx* c) {
+    const std::string msg = t_last_error;
+    read_ctrl(c);
+    t_last_error = msg;
+}
 
 // Stage timing: an event pair on the context stream around a stage's kernels.
 // The pairs are read together once the stream has been waited for anyway.
@@ -577,10 +592,10 @@ fc_status ensure_cache(fc_ctx* c, Grid* g) {
 }
 
 fc_status ensure_q32_storage(fc_ctx* c, Grid* g) {
-    if (g->Qc) return FC_OK;
-    FC_TRY(dalloc_t(c, &g->Qc, (size_t)g->cap * g->G_pad));
-    FC_TRY(dalloc_t(c, &g->Qb, (size_t)g->cap * g->G_pad));
-    FC_TRY(dalloc_t(c, &g->Qb3, (size_t)g->cap * g->G_pad * 8));
+    // each by itself: an earlier call may have had room for some of them only
+    if (!g->Qc) FC_TRY(dalloc_t(c, &g->Qc, (size_t)g->cap * g->G_pad));
+    if (!g->Qb) FC_TRY(dalloc_t(c, &g->Qb, (size_t)g->cap * g->G_pad));
+    if (!g->Qb3) FC_TRY(dalloc_t(c, &g->Qb3, (size_t)g->cap * g->G_pad * 8));
     return FC_OK;
 }
 
@@ -603,7 +618,7 @@ bool use_qvec_tc(const Grid* g) {
 // full cache hands out only slots that this call does not need.  The kernels
 // are launched, not waited for: a covariance that is not positive definite
 // raises the status word, which the next read_ctrl reports.
-fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int cov_mode, bool need_q32,
+fc_status fill_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int cov_mode, bool need_q32,
                        bool need_q64, std::vector<int32_t>* slots_out) {
     FC_TRY(ensure_cache(c, g));
     const int64_t ep = ++g->epoch;
@@ -690,6 +705,7 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
         launch_set_slots(dq, ds, (int)evicted_q.size(), g->slot_of, c->stream);
         c->acc->evicted += (int64_t)evicted_q.size();
     }
+    if (!new_q.empty() || !q32_list.empty() || !q64_list.empty()) g->unread = true;
     if (!new_q.empty()) {
         FC_TRY(to_device(c, dq, new_q.data(), new_q.size() * 4));
         FC_TRY(to_device(c, ds, new_s.data(), new_s.size() * 4));
@@ -720,6 +736,14 @@ fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int c
         launch_qvec64(g->spec(), g->G, g->nfit, g->W64, ds, (int)q64_list.size(), g->G, g->Q64, c->stream);
     }
     return FC_OK;
+}
+
+fc_status ensure_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int cov_mode, bool need_q32,
+                       bool need_q64, std::vector<int32_t>* slots_out) {
+    const fc_status st = fill_slots(c, g, qs, cov_mode, need_q32, need_q64, slots_out);
+    // slots are handed out before they are filled: after an error none of them can be told from a filled one
+    if (st != FC_OK) reset_cache(c, g);
+    return st;
 }
 
 fc_status validate_opts(const fc_opts* o, const Grid* g) {
@@ -957,7 +981,7 @@ fc_status lane_admit(fc_ctx* c, Lane* L, const std::shared_ptr<LaneJob>& J, cons
                         c->status_dev, c->stream);
         // a served job's own factor must not fail the jobs it would join; a synchronous call reports it
         // with the first count it reads
-        if (J->jr) FC_TRY(check_status(c));
+        if (J->jr) FC_TRY(read_ctrl(c));
         launch_fake_data(L32, s32, g->nf, g->identity_collapse ? nullptr : g->collapse, g->nfit, ps_dev, P, U, seed,
                          fluct == FC_FLUCT_GAUSS, dst, c->stream);
     }
@@ -1553,7 +1577,7 @@ fc_status run_sync(fc_ctx* c, Grid* g, const fc_opts& o, const std::vector<int64
     if (st == FC_OK && (done.size() != 1 || !lane_idle(L)))
         st = fail(FC_ERR_STATE, "internal: synchronous job did not complete");
     if (st != FC_OK) {
-        cudaStreamSynchronize(c->stream);  // the caller's data may still be on its way
+        settle(c);
         lane_reset(L);
     }
     c->last_base = J->base;
@@ -1622,7 +1646,7 @@ fc_status fake_data_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t 
     FC_TRY(scratch(c, "s32", (size_t)P * g->nf, &s32));
     launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, nullptr,
                     c->status_dev, c->stream);
-    FC_TRY(check_status(c));
+    FC_TRY(read_ctrl(c));
     if (is_device_ptr(out)) {
         d = out;
     } else {
@@ -1772,7 +1796,10 @@ void worker_main(fc_ctx* c) {
             fc_status st = lane_drop_cancelled(c, L);
             if (st == FC_OK) st = scan_once(c, L);
             if (st == FC_OK) st = lane_harvest(c, L, &done);
-            if (st != FC_OK) lane_fail_all(L, st, &done);
+            if (st != FC_OK) {
+                settle(c);
+                lane_fail_all(L, st, &done);
+            }
             for (auto& J : done) {
                 c->reserved -= std::min(c->reserved, J->jr->need);
                 complete(c, J->jr, J->status);
@@ -2192,7 +2219,7 @@ fc_status fc_covariance(fc_ctx* c, int32_t grid_id, int64_t q, double* A, double
     if (A) {
         std::vector<int32_t> qs{(int32_t)q}, slots;
         FC_TRY(ensure_slots(c, g, qs, FC_COV_ITERATE, false, false, &slots));
-        FC_TRY(check_status(c));
+        FC_TRY(read_ctrl(c));
         FC_TRY(copy_out(c, A, g->A64 + (size_t)slots[0] * g->nfit * g->nfit, (size_t)g->nfit * g->nfit * 8));
     }
     if (L_sys) {
@@ -2205,7 +2232,7 @@ fc_status fc_covariance(fc_ctx* c, int32_t grid_id, int64_t q, double* A, double
         FC_TRY(scratch(c, "cov_s32", (size_t)g->nf, &s32));
         FC_CUDA(cudaMemcpyAsync(pd, &q, 8, cudaMemcpyHostToDevice, c->stream));
         launch_chol_sys(g->full(), g->nf, g->F, pd, 1, 0, L64, L32, s32, nullptr, c->status_dev, c->stream);
-        FC_TRY(check_status(c));
+        FC_TRY(read_ctrl(c));
         FC_TRY(copy_out(c, L_sys, L64, (size_t)g->nf * g->nf * 8));
     }
     return sync(c);

@@ -1,4 +1,6 @@
 """Calls that fail, what they leave behind, and data that has no minimum."""
+import time
+
 import numpy as np
 import pytest
 
@@ -119,3 +121,57 @@ def test_screen_timeout_leaves_no_items(ctx, G, n, P, U, stop_after):
     fc.fc_set_wait_test(ctx, 0, -1)
     for a, b in zip(fc.fc_run_points(ctx, gid, ps, 2, U), ref):
         assert np.array_equal(a, b)
+
+
+# ---- a failed covariance is not kept ---------------------------------------------------------
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("slots", [0, 4])
+def test_failed_covariance_fails_again(ctx, grid, prec, slots):
+    """One spectrum with an empty bin: its covariance fails on every call, and the others keep their results."""
+    S, F = grid
+    S = S.copy()
+    S[17, 3] = 0.0
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    fc.fc_set_tuning(ctx, gid, cache_slots=slots)
+    d = np.random.default_rng(2).poisson(S[:12] + 1.0).astype(np.float32)
+    good, bad = np.array([0, 1, 2] * 4), np.array([0, 1, 17] * 4)
+    ref = fc.fc_scan(ctx, gid, d, good, prec, 8)
+    A, _ = fc.fc_covariance(ctx, gid, 2, 40, 40, want_L=False)
+    for _ in range(3):
+        _not_spd(lambda: fc.fc_scan(ctx, gid, d, bad, prec, 8))
+        _not_spd(lambda: fc.fc_covariance(ctx, gid, 17, 40, 40, want_L=False))
+        for a, b in zip(fc.fc_scan(ctx, gid, d, good, prec, 8), ref):
+            assert np.array_equal(a, b)
+        assert np.array_equal(fc.fc_covariance(ctx, gid, 2, 40, 40, want_L=False)[0], A)
+
+
+def test_served_job_fails_alone(ctx, grid):
+    """A job that starts at such a spectrum fails; the jobs around it on another grid give their results."""
+    S, F = grid
+    bad = S.copy()
+    bad[17, 3] = 0.0
+    g1, g2 = fc.fc_load_grid(ctx, S), fc.fc_load_grid(ctx, bad)
+    for g in (g1, g2):
+        fc.fc_set_frac_cov(ctx, g, F)
+    ref = fc.fc_run_points(ctx, g1, np.array([5, 6]), 3, 50)
+    jobs = [fc.fc_submit(ctx, g, np.array([p, 6]), 3, 50, want_bestfit=True, want_nscans=True)
+            for g, p in ((g1, 5), (g2, 17), (g1, 5))]
+    status = {}
+    end = time.time() + 60
+    while len(status) < 3 and time.time() < end:
+        for t, _ in jobs:
+            if t in status:
+                continue
+            try:
+                st, _ = fc.fc_poll(ctx, t)
+            except fc.FCError as e:
+                st = e.status
+            if st != fc.FC_PENDING:
+                status[t] = st
+        time.sleep(0.001)
+    assert [status[t] for t, _ in jobs] == [fc.FC_OK, fc.FC_ERR_NOT_SPD, fc.FC_OK]
+    for k in (0, 2):
+        for a, b in zip(jobs[k][1], ref):
+            assert np.array_equal(np.asarray(a).ravel(), np.asarray(b).ravel())
