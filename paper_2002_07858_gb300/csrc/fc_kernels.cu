@@ -2316,6 +2316,7 @@ __device__ void quantiles_by_sort(unsigned long long* key, int n, int npow2, con
 // were copied first).
 constexpr int kQuantSelect = 8;   // quantiles of a call that selects
 constexpr int kQuantList = 128;   // values of a quantile's list
+constexpr int kQuantMaxRow = 16384;  // values of a row (the entry points refuse longer ones)
 
 template <int BINS>
 __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, const double* __restrict__ probs,
@@ -2505,11 +2506,14 @@ bool measure_fma_peaks(int n_sm, double* fp64_tflops, double* fp32_tflops, cudaS
 // ------------------------------------------------------------- launchers ----
 
 namespace {
-// shared memory beyond the 48 KB default, which also holds a kernel's static arrays (an attribute of the
-// current device, so set per launch)
+// Shared memory of `bytes`, beyond the 48 KB default, which also holds a kernel's static arrays.  The limit
+// belongs to the kernel on the current device, which every thread and context shares: it is set to what the
+// kernel's largest size takes, the same value at every launch, so that no thread lowers it between another's
+// setting and launch.
 template <class K>
-void allow_smem(K kern, size_t bytes) {
-    if (bytes > 24 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+void allow_smem(K kern, size_t bytes, size_t largest) {
+    if (bytes > 24 * 1024)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)largest);
 }
 }  // namespace
 
@@ -2537,7 +2541,7 @@ void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t*
     count_launch();
     const int C = P <= kCholClusterPoints && nf > 2 * kCholPanel ? kCholCluster : 1;
     const size_t smem = chol_sys_smem(nf, C);
-    allow_smem(k_chol_sys, smem);
+    allow_smem(k_chol_sys, smem, chol_sys_smem(kMaxBins, kCholCluster));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)P * C);
     cfg.blockDim = dim3(kCholThreads);
@@ -2559,7 +2563,7 @@ void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* coll,
     if (n <= 0) return;
     count_launch();
     const size_t smem = build_cov_smem(nfit);
-    allow_smem(k_build_cov, smem);
+    allow_smem(k_build_cov, smem, build_cov_smem(kMaxBins));
     k_build_cov<<<n, build_cov_threads(nfit), smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64,
                                                           A32, rho, status);
 }
@@ -2612,7 +2616,7 @@ void launch_fake_data(const float* L32, const float* s32, int nf, const int32_t*
         const int np = P - p0 < kMaxGridY ? P - p0 : kMaxGridY;
         dim3 grid((U + kFakeU - 1) / kFakeU, np);
         const size_t smem = fake_smem(nf);
-        allow_smem(k_fake_data, smem);
+        allow_smem(k_fake_data, smem, fake_smem(kMaxBins));
         count_launch();
         k_fake_data<<<grid, kFakeThreads, smem, st>>>(L32 + (size_t)p0 * nf * nf, s32 + (size_t)p0 * nf, nf, coll, nfit, ps + p0,
                                            U, (uint32_t)seed, (uint32_t)(seed >> 32), gauss,
@@ -2672,7 +2676,7 @@ void launch_scan64(const int32_t* list, int64_t n, const int32_t* uslot, const f
                    double* y, double* part_v, int32_t* part_g, cudaStream_t st) {
     if (n <= 0) return;
     const size_t smem = (size_t)nfit * (kS64U + kS64LdS) * sizeof(double);
-    cudaFuncSetAttribute(k_scan64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_scan64, smem, (size_t)kMaxBins * (kS64U + kS64LdS) * sizeof(double));
     const bool split = nsp > 1;
     if (split) {
         count_launch();
@@ -2696,7 +2700,7 @@ void launch_scan_resid(const int32_t* list, int64_t n, const int32_t* uslot, con
     count_launch(2);
     const dim3 grid((unsigned)n, (unsigned)nsp);
     auto kern = gs.Sdf ? k_scan_resid<false> : k_scan_resid<true>;
-    allow_smem(kern, smem);
+    allow_smem(kern, smem, rows_smem(kMaxBins));
     kern<<<grid, 32 * kRowsWarps, smem, st>>>(list, uslot, d, gs, G, nfit, Wdf, part_v, part_g);
     k_scan_resid_reduce<<<blocks_for(n), kThreads, 0, st>>>(list, n, nsp, part_v, part_g, best);
 }
@@ -2727,7 +2731,7 @@ void launch_yprep(const int32_t* quad_slot, const int32_t* tile_univ, int64_t n_
                   uint16_t* Yt, float4* alpha, float* tau0, int32_t* tile_j0, cudaStream_t st) {
     if (n_tiles <= 0) return;
     const size_t smem = yprep_smem(nfit, K);
-    allow_smem(k_yprep, smem);
+    allow_smem(k_yprep, smem, yprep_smem(kMaxBins, kMaxScreenK));  // grows with N_fit
     count_launch();
     k_yprep<<<(unsigned)(n_tiles * kQuads), 32 * yprep_warps(K), smem, st>>>(quad_slot, tile_univ, d, centre, nfit, K,
                                                                             A32, rho, cur, gs, gnorm, Qc, Qb, G_pad,
@@ -2775,7 +2779,7 @@ void launch_resolve_list(const ResolveArgs& a, const int32_t* cand_count, int64_
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min(want, cap));
     const size_t smem = rows_smem(a.nfit);
     auto kern = a.gs.Sdf ? k_list_chunks<false> : k_list_chunks<true>;
-    allow_smem(kern, smem);
+    allow_smem(kern, smem, rows_smem(kMaxBins));
     kern<<<grid, 32 * kRowsWarps, smem, st>>>(a, cand_count, rows, lp);
 }
 
@@ -2795,7 +2799,7 @@ void launch_resolve(const ResolveArgs& a, int64_t n_tiles, int64_t n_rows, cudaS
             const unsigned grid = (unsigned)std::max<int64_t>(1, std::min(want, cap));
             const size_t smem = rows_smem(a.nfit);
             auto kern = a.gs.Sdf ? k_resid_rows<false> : k_resid_rows<true>;
-            allow_smem(kern, smem);
+            allow_smem(kern, smem, rows_smem(kMaxBins));
             kern<<<grid, 32 * kRowsWarps, smem, st>>>(a, items, count, res);
             return;
         }
@@ -2827,7 +2831,7 @@ void launch_finish(const int32_t* list, int64_t n, const int32_t* count, int ide
     static_assert(kRowsWarps == 4, "a warp of k_finish has one warp's row storage");
     const size_t smem = Wdf ? rows_smem(nfit) : 0;
     auto kern = gs.Sdf || !Wdf ? k_finish<false> : k_finish<true>;
-    allow_smem(kern, smem);
+    allow_smem(kern, smem, rows_smem(kMaxBins));
     kern<<<grid, 128, smem, st>>>(list, count, ident_slot, slot_of, best, us, d, gs, nfit, W64, Wdf, dchi2, chi2min);
 }
 
@@ -2875,13 +2879,16 @@ void launch_osc_spectra(const SpecModel& m, int64_t G, double* S, int* bad, cuda
 void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, cudaStream_t st) {
     int p2 = 1;
     while (p2 < n) p2 <<= 1;
-    const size_t smem = ((size_t)p2 + (nq <= kQuantSelect ? nq * kQuantList : 0)) * sizeof(unsigned long long);
+    const auto smem_of = [](size_t keys, int lists) {
+        return (keys + (size_t)lists * kQuantList) * sizeof(unsigned long long);
+    };
+    const size_t smem = smem_of(p2, nq <= kQuantSelect ? nq : 0);
     count_launch();
     // short rows: small CTAs, many rows in flight; long rows (and a sort of many quantiles) a wide CTA,
     // with as many buckets as keep a bucket of a smooth distribution below the list's length
     const bool small = n <= 2048 && nq <= kQuantSelect;
     auto kern = small ? k_quantiles<1024> : k_quantiles<4096>;
-    allow_smem(kern, smem);
+    allow_smem(kern, smem, smem_of(small ? 2048 : kQuantMaxRow, kQuantSelect));
     kern<<<rows, small ? 128 : 512, smem, st>>>(x, n, p2, probs, nq, out);
 }
 

@@ -515,7 +515,8 @@ bool launch_qvec_tc(const uint16_t* Bt, const uint16_t* Wimg, const float4* wnor
     if (!qvec_tc_supported(K)) return false;
     QvecLayout lay{};
     if (!qvec_pick_layout(K, n, &lay)) return false;
-    cudaFuncSetAttribute(k_qvec_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes);
+    // the largest layout's, not this launch's: the limit is shared by every thread that launches the kernel
+    cudaFuncSetAttribute(k_qvec_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQSmemMax);
     const int64_t groups = (n + lay.m - 1) / lay.m;
     const int64_t items = groups * (G_pad / kQM);
     const int grid = (int)(items < n_sm ? items : n_sm);

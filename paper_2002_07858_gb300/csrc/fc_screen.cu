@@ -843,7 +843,8 @@ void run_screen(const ScreenLayout& lay, const uint16_t* Yt, const uint16_t* Bt,
                 int64_t G_pad, float* cv, int32_t* ci, int32_t* cc, int* status, const ProbeArgs& pa,
                 const ListArgs& la, const WaitTest& wt, const ScreenSplit& ss, int n_sm, cudaStream_t st) {
     auto kern = k_screen<TOPK, MODE, KCHUNK>;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes);
+    // the largest layout's, not this launch's: the limit is shared by every thread that launches the kernel
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
     const int n_gt = (int)(G_pad / kBN);
     const bool split = ss.parts > 1;
     const int64_t rows = n_tiles * kBM;

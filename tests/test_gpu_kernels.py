@@ -242,3 +242,43 @@ def test_long_host_lists(ctx):
         d1, b1, n1 = fc.fc_run_points(ctx, gid, ps[k:k + 1], 3, 1, opts=opts)
         assert np.array_equal(d[k], d1[0]) and np.array_equal(b[k], b1[0]) and np.array_equal(ns[k], n1[0])
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- several threads on one device ------------------------------------------------------------
+
+def test_threads_of_different_sizes():
+    """Contexts of two threads whose launches need different shared memory: neither's limit cuts the other's."""
+    import threading
+
+    S1, F1 = _grid(30, 200, 1)
+    S2, F2 = _grid(30, 90, 2)
+    errors, out = [], {}
+
+    def work(key, S, F, reps):
+        try:
+            n = S.shape[1]
+            c = fc.fc_create(0)
+            gid = fc.fc_load_grid(c, S)
+            fc.fc_set_frac_cov(c, gid, F)
+            ps = np.arange(20, dtype=np.int64)  # a CTA a point
+            x = np.random.default_rng(n).random((4, 16384 if n == 200 else 5000))
+            got = []
+            for _ in range(reps):
+                A, L = fc.fc_covariance(c, gid, 3, n, n)
+                fc.fc_set_frac_cov(c, gid, F)  # the next covariance is built again
+                got.append((A, L, fc.fc_fake_data(c, gid, ps, 5, 3, n), *fc.fc_run_points(c, gid, ps[:2], 5, 9),
+                            fc.fc_quantiles(c, x, np.array([0.1, 0.9]))))
+            out[key] = got
+            fc.fc_destroy(c)
+        except Exception as e:  # the launch that finds the limit too low is an error of the call
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=a) for a in ((200, S1, F1, 150), (90, S2, F2, 300))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors[0]
+    for got in out.values():
+        for g in got[1:]:
+            assert all(np.array_equal(a, b) for a, b in zip(g, got[0]))
