@@ -149,6 +149,7 @@ struct Grid {
 struct Scratch {
     void* p = nullptr;
     size_t bytes = 0;
+    bool spare = false;  // only makes a call faster: given up where something it needs finds no room
 };
 
 // What the host reads between launches, in one block on the device and one
@@ -265,14 +266,36 @@ struct fc_ctx {
 
 namespace {
 
-fc_status dalloc(fc_ctx* c, void** p, size_t bytes) {
+void dfree(fc_ctx* c, void* p);
+
+// Gives up the spare scratch (its users are launched by the time anything else is allocated, and freeing waits
+// for them); false: there was none.
+bool drop_spare(fc_ctx* c) {
+    bool any = false;
+    for (auto& kv : c->scratch) {
+        Scratch& s = kv.second;
+        if (!s.spare || !s.p) continue;
+        dfree(c, s.p);
+        s.p = nullptr;
+        s.bytes = 0;
+        any = true;
+    }
+    return any;
+}
+
+fc_status dalloc(fc_ctx* c, void** p, size_t bytes, bool spare = false) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     bytes = (bytes + 255) & ~(size_t)255;
+    if (!spare && c->budget && c->used + bytes > c->budget) drop_spare(c);
     if (c->budget && c->used + bytes > c->budget)
         return fail(FC_ERR_BUDGET, "device-memory budget exceeded (" + std::to_string(c->used + bytes) + " > " +
                                        std::to_string(c->budget) + " bytes)");
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && !spare && drop_spare(c)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -303,8 +326,9 @@ void dfree(fc_ctx* c, void* p) {
 
 // grow-only named scratch buffer
 template <class T>
-fc_status scratch(fc_ctx* c, const char* name, size_t count, T** out) {
+fc_status scratch(fc_ctx* c, const char* name, size_t count, T** out, bool spare = false) {
     Scratch& s = c->scratch[name];
+    s.spare = spare;
     const size_t bytes = std::max<size_t>(count * sizeof(T), 16);
     if (s.bytes < bytes) {
         dfree(c, s.p);
@@ -312,12 +336,25 @@ fc_status scratch(fc_ctx* c, const char* name, size_t count, T** out) {
         s.bytes = 0;
         const size_t want = bytes + bytes / 4;
         void* p = nullptr;
-        FC_TRY(dalloc(c, &p, want));
+        FC_TRY(dalloc(c, &p, want, spare));
         s.p = p;
         s.bytes = want;
     }
     *out = (T*)s.p;
     return FC_OK;
+}
+
+void drop_scratch(fc_ctx* c, const char* name) {
+    Scratch& s = c->scratch[name];
+    dfree(c, s.p);
+    s.p = nullptr;
+    s.bytes = 0;
+}
+
+size_t spare_bytes(const fc_ctx* c) {
+    size_t n = 0;
+    for (const auto& kv : c->scratch) n += kv.second.spare ? kv.second.bytes : 0;
+    return n;
 }
 
 // The caller's array where a kernel can read it in place: memory of this context's device, aligned for
@@ -533,12 +570,13 @@ size_t cache_reserve(fc_ctx* c) {
 }
 
 // Bytes a cache may still take: what the budget (or the device) has left
-// above the reserve.
+// above the reserve, with the spare scratch, which gives way.
 size_t cache_headroom(fc_ctx* c) {
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    size_t room = free_b;
-    if (c->budget) room = std::min(room, c->budget > c->used ? c->budget - c->used : 0);
+    const size_t spare = spare_bytes(c);
+    size_t room = free_b + spare;
+    if (c->budget) room = std::min(room, c->budget + spare > c->used ? c->budget + spare - c->used : 0);
     const size_t res = cache_reserve(c);
     return room > res ? room - res : 0;
 }
@@ -1065,9 +1103,9 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
             int nsp = scan64_splits(cnt, g->G, c->n_sm);
             double *pv = nullptr, *py = nullptr;
             int32_t* pg = nullptr;
-            if (nsp > 1 && (scratch(c, "fb_y", (size_t)cnt * g->nfit, &py) != FC_OK ||
-                            scratch(c, "fb_pv", (size_t)cnt * nsp, &pv) != FC_OK ||
-                            scratch(c, "fb_pg", (size_t)cnt * nsp, &pg) != FC_OK))
+            if (nsp > 1 && (scratch(c, "s64_y", (size_t)cnt * g->nfit, &py, true) != FC_OK ||
+                            scratch(c, "s64_pv", (size_t)cnt * nsp, &pv, true) != FC_OK ||
+                            scratch(c, "s64_pg", (size_t)cnt * nsp, &pg, true) != FC_OK))
                 nsp = 1;  // no room for the partial minima
             FC_TRY(stage_begin(c));
             launch_scan64(list, cnt, lslot, d, g->spec(), g->G, g->nfit, g->A64, g->Q64, g->G, L->best, nsp, py, pv,
@@ -1157,9 +1195,9 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                 if (ss.parts > 1) {
                     // a split that has no room for its storage runs unsplit
                     const size_t rows = (size_t)n_tiles * kBM, cand = listing ? 0 : rows * ss.parts * rtopk;
-                    if ((min_pass && scratch(c, "split_key", rows, &ss.key) != FC_OK) ||
-                        (cand && (scratch(c, "split_val", cand, &ss.val) != FC_OK ||
-                                  scratch(c, "split_idx", cand, &ss.idx) != FC_OK)))
+                    if ((min_pass && scratch(c, "split_key", rows, &ss.key, true) != FC_OK) ||
+                        (cand && (scratch(c, "split_val", cand, &ss.val, true) != FC_OK ||
+                                  scratch(c, "split_idx", cand, &ss.idx, true) != FC_OK)))
                         ss.parts = 1;
                 }
                 for (int pass = min_pass ? 0 : 1; pass < 2; ++pass) {
@@ -1225,17 +1263,27 @@ fc_status scan_once(fc_ctx* c, Lane* L) {
                     int32_t* lrows = nullptr;
                     FC_TRY(scratch(c, "lrows", (size_t)n_tiles * kBM, &lrows));
                     // chunks: a complete list holds at most 2 kListCap points (round 2) or its exact
-                    // size (round 3, list_total over the rows), and a row adds at most one partial chunk
+                    // size (round 3, list_total over the rows), and a row adds at most one partial chunk.
+                    // Wide chunks take a quarter of the plan's storage: where it has no room for the others,
+                    // or its 32-bit positions would not reach
                     ListPlan lp{};
-                    lp.max_chunks = loff ? list_total / kListChunk + cnt
-                                         : cnt * ((2 * kListCap + kListChunk - 1) / kListChunk);
-                    FC_TRY(scratch(c, "lp_chunk", (size_t)lp.max_chunks, &lp.chunk));
-                    FC_TRY(scratch(c, "lp_pv", (size_t)lp.max_chunks, &lp.pv));
-                    FC_TRY(scratch(c, "lp_pg", (size_t)lp.max_chunks, &lp.pg));
                     FC_TRY(scratch(c, "lp_base", (size_t)cnt, &lp.row_base));
                     FC_TRY(scratch(c, "lp_nc", (size_t)cnt, &lp.row_nc));
                     FC_TRY(scratch(c, "lp_done", (size_t)cnt, &lp.row_done));
                     FC_TRY(scratch(c, "lp_n", 1, &lp.n_chunk));
+                    auto plan = [&](int pts) -> fc_status {
+                        lp.pts = pts;
+                        lp.max_chunks = loff ? list_total / pts + cnt : cnt * ((2 * kListCap + pts - 1) / pts);
+                        const bool spare = pts < kListChunkWide;
+                        FC_TRY(scratch(c, "lp_chunk", (size_t)lp.max_chunks, &lp.chunk, spare));
+                        FC_TRY(scratch(c, "lp_pv", (size_t)lp.max_chunks, &lp.pv, spare));
+                        return scratch(c, "lp_pg", (size_t)lp.max_chunks, &lp.pg, spare);
+                    };
+                    const bool reach = (loff ? list_total : cnt * 2 * kListCap) / kListChunk + cnt < INT32_MAX;
+                    if (!reach || plan(kListChunk) != FC_OK) {
+                        for (const char* name : {"lp_chunk", "lp_pv", "lp_pg"}) drop_scratch(c, name);
+                        FC_TRY(plan(kListChunkWide));
+                    }
                     launch_resolve_list(ra, ccount, n_tiles, cnt, lrows, cnts + 6, lp, c->stream);
                 }
                 else {

@@ -300,9 +300,12 @@ void launch_min_tau(const int32_t* tile_univ, int64_t n_tiles, const float* thr,
 // Third round: binary64 residual chi2 of every listed candidate of each row
 // (complete lists certify the minimum); overflowing rows go to `fb`.
 // list rounds: n_rows = universes in the round's tiles; rows [n_tiles * BM] and n_rows_dev are scratch
-// Work split of a list round: chunks of kListChunk listed points of one row.
+// Work split of a list round: chunks of pts listed points of one row, kListChunk of them or, where the plan
+// has no room for that many chunks, kListChunkWide.
 constexpr int kListChunk = 8;
+constexpr int kListChunkWide = 32;
 struct ListPlan {
+    int pts;
     int2* chunk;        // [max_chunks] (listed-row index w, chunk k of that row); w < 0: no work
     int32_t* n_chunk;   // device count of chunks
     int32_t* row_base;  // [n_rows] first chunk of row w

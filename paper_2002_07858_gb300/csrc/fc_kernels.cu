@@ -1996,8 +1996,8 @@ __global__ void k_resolve_tail(ResolveArgs a) {
 // List rounds: every grid point whose screen lower bound is at or below the
 // row's seed (an upper bound of the minimum) is listed, so the residual-form
 // minimum over a complete list is the minimum of the scan.  A row's list is
-// cut into chunks of kListChunk points, one per lane of a warp, so a long list
-// spreads over many warps.  k_list_plan checks each listed row (rows[] holds
+// cut into chunks of lp.pts points, a warp each, so a long list spreads over
+// many warps.  k_list_plan checks each listed row (rows[] holds
 // the round's occupied tile rows) and reserves its chunks; rows whose list
 // overflowed go to the exact scan (their counts size the next, exact-size list
 // round).
@@ -2018,7 +2018,7 @@ __global__ void k_list_plan(ResolveArgs a, const int32_t* __restrict__ cand_coun
     }
     lp.row_nc[w] = 0;
     if (complete && n0 + n1 > 0) {
-        const int nc = (n0 + n1 + kListChunk - 1) / kListChunk;
+        const int nc = (n0 + n1 + lp.pts - 1) / lp.pts;
         const int base = atomicAdd(lp.n_chunk, nc);
         if ((int64_t)base + nc <= lp.max_chunks) {
             lp.row_base[w] = base;
@@ -2070,8 +2070,8 @@ __global__ void __launch_bounds__(32 * kRowsWarps, MODEL ? 3 : 4) k_list_chunks(
         const float* du = a.d + (size_t)u * n;
         double bv = DBL_MAX;
         int32_t bg = INT32_MAX;
-        const int k_end = min((ck.y + 1) * kListChunk, n0 + n1);
-        for (int k0 = ck.y * kListChunk; k0 < k_end; k0 += kRowsB) {
+        const int k_end = min((ck.y + 1) * lp.pts, n0 + n1);
+        for (int k0 = ck.y * lp.pts; k0 < k_end; k0 += kRowsB) {
             const int m = min(kRowsB, k_end - k0);
             int32_t mine = INT32_MAX;  // lane k: the group's point k
             for (int k = 0; k < m; ++k) {

@@ -175,3 +175,31 @@ def test_served_job_fails_alone(ctx, grid):
     for k in (0, 2):
         for a, b in zip(jobs[k][1], ref):
             assert np.array_equal(np.asarray(a).ravel(), np.asarray(b).ravel())
+
+
+# ---- tight budgets ---------------------------------------------------------------------------
+
+@pytest.mark.parametrize("side,n,P,U,prec,budget", [
+    (100, 20, 2, 64, fc.FC_PREC_MIXED, 18_800_000),      # no room for the split screen's lists
+    (100, 20, 2, 20000, fc.FC_PREC_MIXED, 45_500_000),   # nor for the small chunks of a list round
+    (60, 45, 40, 500, fc.FC_PREC_MIXED, 46_600_000),
+    (60, 45, 40, 500, fc.FC_PREC_FP64, 17_800_000),
+    (30, 100, 10, 2000, fc.FC_PREC_MIXED, 51_200_000),
+])
+def test_storage_that_only_saves_time_gives_way(side, n, P, U, prec, budget):
+    """Budgets that these fits, the first of a context, have always fitted in: what they take beyond the least is
+    given up, with the same results."""
+    fc.load()
+    S, F, _ = workloads.osc_2d(side, side, n, seed=1)
+    ps = np.linspace(0, len(S) - 1, P).astype(np.int64)
+    out = []
+    for b in (0, budget):
+        c = fc.fc_create(0, b)
+        try:
+            gid = fc.fc_load_grid(c, S)
+            fc.fc_set_frac_cov(c, gid, F)
+            out.append(fc.fc_run_points(c, gid, ps, 4, U, opts=dict(precision=prec)))
+            assert not b or fc.fc_get_stats(c)["device_bytes"] <= b
+        finally:
+            fc.fc_destroy(c)
+    assert all(np.array_equal(x, y) for x, y in zip(*out))
