@@ -2254,7 +2254,8 @@ __global__ void k_count_below(const double* __restrict__ x, int n, const double*
 
 
 // Order of binary64 values as unsigned integers (comparing integers keeps the
-// narrow binary64 pipe out of a sort); NaN sorts by its bits, -0 before +0.
+// narrow binary64 pipe out of a sort); -0 before +0, NaN by its bits (rows that
+// hold any are sorted, where every NaN comes last).
 // It takes the bits, loaded as an integer: of a value that was a binary64
 // before, the compiler may set the sign by negating it, which a NaN ignores.
 __device__ __forceinline__ unsigned long long f64_key(unsigned long long b) {
@@ -2278,6 +2279,10 @@ __device__ __forceinline__ void quantile_ranks(int n, double prob, int& lo, int&
 __device__ void quantiles_by_sort(unsigned long long* key, int n, int npow2, const double* __restrict__ probs, int nq,
                                   double* __restrict__ out) {
     for (int i = n + threadIdx.x; i < npow2; i += blockDim.x) key[i] = ~0ull;
+    // keys below -infinity's are the NaN with the sign set: last, like the others (thread i wrote key i)
+    const unsigned long long first = f64_key(0xfff0000000000000ull);
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (key[i] < first) key[i] = ~0ull;
     __syncthreads();
     for (int k = 2; k <= npow2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {

@@ -282,3 +282,22 @@ def test_threads_of_different_sizes():
     for got in out.values():
         for g in got[1:]:
             assert all(np.array_equal(a, b) for a, b in zip(g, got[0]))
+
+
+@pytest.mark.parametrize("n", [5, 100, 3000])
+@pytest.mark.parametrize("nq", [3, 9])
+def test_quantiles_sort_every_nan_last(ctx, n, nq):
+    """NaN of both signs behind the row's numbers and infinities, as numpy sorts them."""
+    x = np.random.default_rng(n).standard_normal((4, n))
+    x[1, 0], x[2, n - 1], x[3, 0], x[3, 3] = -np.nan, np.nan, -np.nan, np.nan
+    assert np.signbit(x[1, 0]) and not np.signbit(x[2, n - 1])
+    x[3, 1], x[3, 2] = -np.inf, np.inf
+    probs = np.linspace(0.0, 1.0, nq)
+    s, h = np.sort(x, axis=1), (n - 1) * probs
+    lo = np.floor(h).astype(int)
+    with np.errstate(invalid="ignore"):
+        a, b = s[:, lo], s[:, np.minimum(lo + 1, n - 1)]
+        want = a + (h - lo) * (b - a)
+    # two orders of the blend's three roundings differ by at most 10 half-ulps of the row's largest number
+    np.testing.assert_allclose(fc.fc_quantiles(ctx, x, probs), want, rtol=0,
+                               atol=1.2e-15 * np.max(np.abs(x), where=np.isfinite(x), initial=0.0))
