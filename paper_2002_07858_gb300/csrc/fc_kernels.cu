@@ -1517,7 +1517,9 @@ __global__ void k_yprep(const int32_t* __restrict__ quad_slot, const int32_t* __
     }
     copy_async_wait();
     // d - v by the thread that copied the value; v as double-float keeps the difference off the narrow
-    // binary64 pipe (its error, 2^-24 (1 + 2^-20) |d - v|, is inside alpha's)
+    // binary64 pipe.  Its error is at most 1.5 2^-24 |d - v|: one half unit from rounding the result, and what
+    // v loses as hi + lo, at most 2^-24 |lo|, where |lo| is below |d - v| unless d = hi (then the result is -lo
+    // itself), and where it comes near |d - v| hi - d + lo loses at most the bit that makes up the sum.
     for (int k = warp; k < kQuadRows; k += nw) {
         const bool used = __shfl_sync(0xffffffffu, u, k) >= 0;
         for (int j = lane; j < nfit; j += 32)
@@ -1612,9 +1614,9 @@ __global__ void k_yprep(const int32_t* __restrict__ quad_slot, const int32_t* __
     // -2 y.s~_g - (hi*hi + lo*hi + hi*lo products)  =  -2 (y - y^).s~ + Y_lo.S_lo + (Y_hi + Y_lo).r_S + r_Y.s~
     // and the binary32 accumulation of the 3K products (each add bounded as truncated, Sum|products| <= 1.02 |Y||s~|):
     //   |error| <= [2 |y - y^| + |r_Y| + (3K+2) 1.02 2^-23 |Y|] |s~| + |Y_lo| |S_lo| + |Y_hi+Y_lo| |r_S|
-    // with |y - y^| <= (nfit+2) 2^-24 rho |d~| (A and d~ rounded to binary32, binary32 dot products).
+    // with |y - y^| <= (nfit+2.5) 2^-24 rho |d~| (A rounded to binary32, d~ as above, binary32 dot products).
     const float dn = sqrtf(dn2) * 1.0001f, yn = sqrtf(yn2) * 1.0001f;
-    const float a_acc = 1.02f * (2.0f * (float)(nfit + 2) * 5.9604645e-08f * rho[slot] * dn +
+    const float a_acc = 1.02f * (2.0f * ((float)nfit + 2.5f) * 5.9604645e-08f * rho[slot] * dn +
                                  (float)(3 * K + 2) * 1.1920929e-07f * 1.02f * yn + sqrtf(ry2));
     const float4 al = make_float4(a_acc, 1.0001f * sqrtf(yl2), 1.0001f * sqrtf(yhl2), 0.0f);
     alpha[t * kBM + r] = al;
