@@ -1015,7 +1015,7 @@ fc_status lane_admit(fc_ctx* c, Lane* L, const std::shared_ptr<LaneJob>& J, cons
         FC_TRY(scratch(c, "L64", (size_t)P * g->nf * g->nf, &L64));
         FC_TRY(scratch(c, "L32", (size_t)P * g->nf * g->nf, &L32));
         FC_TRY(scratch(c, "s32", (size_t)P * g->nf, &s32));
-        launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, nullptr,
+        launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, c->n_sm,
                         c->status_dev, c->stream);
         // a served job's own factor must not fail the jobs it would join; a synchronous call reports it
         // with the first count it reads
@@ -1692,7 +1692,7 @@ fc_status fake_data_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t 
     FC_TRY(scratch(c, "L64", (size_t)P * g->nf * g->nf, &L64));
     FC_TRY(scratch(c, "L32", (size_t)P * g->nf * g->nf, &L32));
     FC_TRY(scratch(c, "s32", (size_t)P * g->nf, &s32));
-    launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, nullptr,
+    launch_chol_sys(g->full(), g->nf, g->F, ps_dev, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, c->n_sm,
                     c->status_dev, c->stream);
     FC_TRY(read_ctrl(c));
     if (is_device_ptr(out)) {
@@ -2279,7 +2279,7 @@ fc_status fc_covariance(fc_ctx* c, int32_t grid_id, int64_t q, double* A, double
         FC_TRY(scratch(c, "cov_L32", (size_t)g->nf * g->nf, &L32));
         FC_TRY(scratch(c, "cov_s32", (size_t)g->nf, &s32));
         FC_CUDA(cudaMemcpyAsync(pd, &q, 8, cudaMemcpyHostToDevice, c->stream));
-        launch_chol_sys(g->full(), g->nf, g->F, pd, 1, 0, L64, L32, s32, nullptr, c->status_dev, c->stream);
+        launch_chol_sys(g->full(), g->nf, g->F, pd, 1, 0, L64, L32, s32, c->n_sm, c->status_dev, c->stream);
         FC_TRY(read_ctrl(c));
         FC_TRY(copy_out(c, L_sys, L64, (size_t)g->nf * g->nf * 8));
     }

@@ -131,7 +131,7 @@ void launch_centred(const GridSpec& gs, int64_t G, int64_t G_pad, int K, double*
 // ---- covariances (a2) ----
 // L_p (binary64 and binary32 copies) for every true point; gauss adds diag(s).
 void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t* ps, int P, int gauss,
-                     double* L64, float* L32, float* s32, double* work, int* status, cudaStream_t st);
+                     double* L64, float* L32, float* s32, int n_sm, int* status, cudaStream_t st);
 // A(q) = M(q)^-1 for a list of (slot, q): A64, W64 (A = W^T W), A32, rho (max abs row sum of A).
 void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* collapse, const double* F,
                       const int32_t* q_list, const int32_t* slot_list, int n, int cov_mode, double* A64,

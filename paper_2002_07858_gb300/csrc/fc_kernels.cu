@@ -455,9 +455,9 @@ __device__ __forceinline__ void tri_decode(int e, int& a, int& b) {
 // Systematic Cholesky factor of a true point, in binary64.  Each element's
 // terms are subtracted in increasing k with a separately rounded multiply and
 // subtract, then divided by the pivot, so the factor is reproducible bit for
-// bit; any blocking that keeps that order gives it.  Bound by the narrow
-// binary64 pipe when points are many (a multiply and a subtract a term), by the
-// chain of roots and divisions when they are few.
+// bit; any blocking that keeps that order gives it.  Bound by the chain of roots
+// and divisions when points are few, by the narrow binary64 pipe (a multiply
+// and a subtract a term) when they are many.
 // Panels of kCholPanel columns: the panel is gathered into P, factored there
 // column by column (the thread that makes the next pivot takes its root while
 // the others update), and its terms are then subtracted from the trailing
@@ -467,15 +467,29 @@ __device__ __forceinline__ void tri_decode(int e, int& a, int& b) {
 // i mod C, which updates it; every CTA gathers the next panel from the owners'
 // shared memory and factors it for itself, so one cluster barrier a panel is
 // all they exchange.
-// Four points of N_full = 200 (one CTA a point, in global memory): 1680 -> 443 us;
-// one of 90: 212 -> 136 us; 10 000 of 90, where a CTA has a point either way and
-// the pipe decides: 6.4 -> 6.5 ms.
+// Three forms, by what bounds the launch (us measured at points x N_full, the
+// form above the line against the one below):
+//  cluster   N_full >= 40 and at most 1.5 CTAs an SM: the chain decides, and
+//            eight CTAs shorten it (against a CTA a point: 30 x 90 155 / 188, 30
+//            x 200 858 / 1062; 38 x 130, where CTAs wait for one another, 477 /
+//            390; 4 x 20 28.0 / 24.5 with the columns below)
+//  panels    N_full >= 64 and a point an SM at most: the chain again (152 x 90
+//            188 / 212, 152 x 200 1064 / 1705; 152 x 40 58.6 / 55.7)
+//  columns   else (k_chol_columns): enough points keep the pipe busy, and the
+//            panel's gathering is work on top (500 x 90 429 / 413, 9000 x 40 980
+//            / 899, 2000 x 200 14853 / 12903; 500 x 120, just above one round of
+//            CTAs, is the exception: 985 / 1035)
 constexpr int kCholPanel = 8;
 constexpr int kCholThreads = 256;
 constexpr int kCholCluster = 8;        // CTAs a point when points are few
-constexpr int kCholClusterPoints = 19; // 19 x 8 = the SMs
 
 constexpr int kCholLonePanel = 4;      // panel of a lone CTA
+
+enum { kCholColumnsForm, kCholPanelForm, kCholClusterForm };
+inline int chol_form(int P, int nf, int n_sm) {
+    if (nf >= 40 && 2 * (int64_t)P * kCholCluster <= 3 * (int64_t)n_sm) return kCholClusterForm;
+    return nf >= 64 && P <= n_sm ? kCholPanelForm : kCholColumnsForm;
+}
 
 inline size_t chol_sys_smem(int nf, int C) {
     return (size_t)(tri(nf) + (C > 1 ? kCholPanel : kCholLonePanel) * nf) * sizeof(double);
@@ -586,6 +600,71 @@ __global__ void __launch_bounds__(kCholThreads, 6) k_chol_sys(FullSrc src, int n
         if (s_bad && tid == 0) atomicOr(status, kDevNotSpd);
         for (int i = tid; i < nf; i += kCholThreads) s32[(size_t)ip * nf + i] = __double2float_rn(s[i]);
     }
+}
+
+// The same factor for many points, one CTA a point and a column at a time: after
+// column k is final, every trailing element (i >= j > k) subtracts L_ik L_jk.
+// Bound by the binary64 pipe.  The triangle is packed in shared memory up to
+// kCholPackN (98 KB; 33 KB at N_full = 90, so six points share an SM), beyond it
+// lies in the output, row-major, where the several points of an SM hide one
+// another's latency better than the one that 161 KB leave room for.
+constexpr int kCholPackN = 155;
+
+template <bool PACKED>
+__global__ void __launch_bounds__(kCholThreads) k_chol_columns(FullSrc src, int nf, const double* __restrict__ F,
+                                                              const int64_t* __restrict__ ps, int gauss,
+                                                              double* __restrict__ L64, float* __restrict__ L32,
+                                                              float* __restrict__ s32, int* __restrict__ status) {
+    extern __shared__ double sT[];
+    __shared__ double s_row[kMaxBins];
+    __shared__ double s_d;
+    __shared__ int s_bad;
+    const int ip = blockIdx.x, n = nf, tid = threadIdx.x;
+    double* Lg = L64 + (size_t)ip * n * n;
+    float* Lf = L32 + (size_t)ip * n * n;
+    double* L = PACKED ? sT : Lg;
+    auto at = [n](int i, int j) { return PACKED ? tri(i) + j : i * n + j; };
+    stage_full_row(src, n, ps[ip], s_row);
+    const double* s = s_row;
+    if (tid == 0) s_bad = 0;
+    for (int e = tid; e < tri(n); e += kCholThreads) {
+        int i, j;
+        tri_decode(e, i, j);
+        double v = __dmul_rn(__dmul_rn(s[i], F[i * n + j]), s[j]);
+        if (gauss && i == j) v = __dadd_rn(v, s[i]);
+        L[at(i, j)] = v;
+    }
+    __syncthreads();
+    for (int k = 0; k < n; ++k) {
+        if (tid == 0) {
+            double acc = L[at(k, k)];
+            if (!(acc > 0.0)) {
+                s_bad = 1;
+                acc = 1.0;
+            }
+            s_d = __dsqrt_rn(acc);
+            L[at(k, k)] = s_d;
+        }
+        __syncthreads();
+        const double dk = s_d;
+        for (int i = k + 1 + tid; i < n; i += kCholThreads) L[at(i, k)] = __ddiv_rn(L[at(i, k)], dk);
+        __syncthreads();
+        for (int e = tid; e < tri(n - k - 1); e += kCholThreads) {
+            int a, b;
+            tri_decode(e, a, b);
+            const int i = k + 1 + a, j = k + 1 + b;
+            L[at(i, j)] = __dsub_rn(L[at(i, j)], __dmul_rn(L[at(i, k)], L[at(j, k)]));
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < n * n; e += kCholThreads) {
+        const int i = e / n, j = e % n;
+        const double v = j <= i ? L[at(i, j)] : 0.0;
+        Lg[e] = v;
+        Lf[e] = __double2float_rn(v);
+    }
+    if (s_bad && tid == 0) atomicOr(status, kDevNotSpd);
+    for (int i = tid; i < n; i += kCholThreads) s32[(size_t)ip * n + i] = __double2float_rn(s[i]);
 }
 
 // One CTA per (slot, q): M(q) = C [diag(s) F diag(s) + diag(s)] C^T, L = chol(M),
@@ -2543,10 +2622,19 @@ void launch_centred(const GridSpec& gs, int64_t G, int64_t G_pad, int K, double*
 }
 
 void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t* ps, int P, int gauss, double* L64,
-                     float* L32, float* s32, double*, int* status, cudaStream_t st) {
+                     float* L32, float* s32, int n_sm, int* status, cudaStream_t st) {
     if (P <= 0) return;
     count_launch();
-    const int C = P <= kCholClusterPoints && nf > 2 * kCholPanel ? kCholCluster : 1;
+    const int form = chol_form(P, nf, n_sm);
+    if (form == kCholColumnsForm) {
+        const bool packed = nf <= kCholPackN;
+        const size_t smem = packed ? (size_t)tri(nf) * sizeof(double) : 0;
+        auto kern = packed ? k_chol_columns<true> : k_chol_columns<false>;
+        allow_smem(kern, smem, (size_t)tri(kCholPackN) * sizeof(double));
+        kern<<<P, kCholThreads, smem, st>>>(src, nf, F, ps, gauss, L64, L32, s32, status);
+        return;
+    }
+    const int C = form == kCholClusterForm ? kCholCluster : 1;
     const size_t smem = chol_sys_smem(nf, C);
     allow_smem(k_chol_sys, smem, chol_sys_smem(kMaxBins, kCholCluster));
     cudaLaunchConfig_t cfg{};

@@ -203,3 +203,12 @@ def test_storage_that_only_saves_time_gives_way(side, n, P, U, prec, budget):
         finally:
             fc.fc_destroy(c)
     assert all(np.array_equal(x, y) for x, y in zip(*out))
+
+
+@pytest.mark.parametrize("n", [40, 170])
+@pytest.mark.parametrize("P", [1, 100, 400])
+def test_not_spd_factor_in_every_form(ctx, n, P):
+    S, F, _ = workloads.osc_2d(20, 20, n, seed=4)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, _indefinite(F))
+    _not_spd(lambda: fc.fc_fake_data(ctx, gid, np.arange(P), 1, 2, n))

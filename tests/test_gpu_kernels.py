@@ -301,3 +301,21 @@ def test_quantiles_sort_every_nan_last(ctx, n, nq):
     # two orders of the blend's three roundings differ by at most 10 half-ulps of the row's largest number
     np.testing.assert_allclose(fc.fc_quantiles(ctx, x, probs), want, rtol=0,
                                atol=1.2e-15 * np.max(np.abs(x), where=np.isfinite(x), initial=0.0))
+
+
+# ---- systematic factor: the form for many points, and the lines between the three -------------
+
+@pytest.mark.parametrize("nf", [1, 20, 39, 40, 63, 64, 90, 155, 156, 200])
+@pytest.mark.parametrize("P", [28, 29, 152, 153, 330])
+def test_systematic_factor_forms(ctx, nf, P):
+    """Bit for bit the oracle's fake data on both sides of every line, in both fluctuation modes."""
+    import oracle
+
+    S, F = _grid(330, nf, nf + 1)
+    gid = fc.fc_load_grid(ctx, S)
+    fc.fc_set_frac_cov(ctx, gid, F)
+    ps = np.arange(P, dtype=np.int64)[::-1].copy()
+    for fluct in (fc.FC_FLUCT_POISSON_SYS, fc.FC_FLUCT_GAUSS):
+        got = fc.fc_fake_data(ctx, gid, ps, 5, 2, nf, fluct)
+        assert np.array_equal(got, oracle.fake_data(S, F, ps, 5, 2, None, nf, fluct))
+    fc.fc_unload_grid(ctx, gid)
