@@ -749,7 +749,7 @@ fc_status fill_slots(fc_ctx* c, Grid* g, const std::vector<int32_t>& qs, int cov
         FC_TRY(to_device(c, ds, new_s.data(), new_s.size() * 4));
         launch_build_cov(g->full(), g->nf, g->nfit, g->identity_collapse ? nullptr : g->collapse, g->F, dq, ds,
                          (int)new_q.size(), cov_mode == FC_COV_IDENTITY ? 2 : 0, g->A64, g->W64, g->A32, g->rho,
-                         c->status_dev, c->stream);
+                         c->n_sm, c->status_dev, c->stream);
         launch_wdf(g->W64, ds, (int)new_q.size(), g->nfit, g->Wdf, c->stream);
         if (cov_mode != FC_COV_IDENTITY) launch_set_slots(dq, ds, (int)new_q.size(), g->slot_of, c->stream);
         c->acc->distinct_cov += (int64_t)new_q.size();

@@ -135,7 +135,7 @@ void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t*
 // A(q) = M(q)^-1 for a list of (slot, q): A64, W64 (A = W^T W), A32, rho (max abs row sum of A).
 void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* collapse, const double* F,
                       const int32_t* q_list, const int32_t* slot_list, int n, int cov_mode, double* A64,
-                      double* W64, float* A32, float* rho, int* status, cudaStream_t st);
+                      double* W64, float* A32, float* rho, int n_sm, int* status, cudaStream_t st);
 // q_g = s~_g^T A s~_g for slots: binary64 |W s~_g|^2 (plain) or binary32 central + lower bound (mixed).
 void launch_qvec64(const GridSpec& gs, int64_t G, int nfit, const double* W64, const int32_t* slots, int n,
                    int64_t ldq, double* Q64, cudaStream_t st);

@@ -684,8 +684,15 @@ __global__ void __launch_bounds__(kCholThreads) k_chol_columns(FullSrc src, int 
 // squares (in global memory above N_fit = 64): 597 covariances of N = 200 in
 // four launches 18.1 -> 11.3 ms, 10 500 of N = 120 30.1 -> 22.4 ms (their
 // multiply-adds alone take 4.1 and 15.7 ms), 10 000 of N = 45 2.8 -> 1.8 ms.
-inline int build_cov_threads(int nfit) { return nfit > 120 ? 512 : 256; }
 inline size_t build_cov_smem(int nfit) { return (size_t)(tri(nfit) + 2 * nfit) * sizeof(double); }
+// 512 threads while an SM holds three CTAs at most, for want of matrices or of shared memory (above N = 112):
+// with four, 256 keep more of the pipe for the phases that need few threads.  Measured, us with 256 / 512
+// threads: 152 matrices of N = 90 314 / 231, 400 431 / 413, 500 516 / 618; 400 of N = 40 84 / 77, 500 97 / 137;
+// 2000 of N = 112 3242 / 3298, of N = 114 3673 / 3440.
+inline int build_cov_threads(int nfit, int n, int n_sm) {
+    constexpr size_t kStatic = 5 * 1024, kSmSmem = 228 * 1024;  // static arrays and what the system keeps, a CTA
+    return n <= 3 * (int64_t)n_sm || 4 * (build_cov_smem(nfit) + kStatic) > kSmSmem ? 512 : 256;
+}
 
 __global__ void k_build_cov(FullSrc src, int nf, int nfit, const int32_t* __restrict__ coll,
                             const double* __restrict__ F, const int32_t* __restrict__ q_list,
@@ -2654,12 +2661,12 @@ void launch_chol_sys(const FullSrc& src, int nf, const double* F, const int64_t*
 
 void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* coll, const double* F, const int32_t* q_list,
                       const int32_t* slot_list, int n, int cov_mode, double* A64, double* W64, float* A32,
-                      float* rho, int* status, cudaStream_t st) {
+                      float* rho, int n_sm, int* status, cudaStream_t st) {
     if (n <= 0) return;
     count_launch();
     const size_t smem = build_cov_smem(nfit);
     allow_smem(k_build_cov, smem, build_cov_smem(kMaxBins));
-    k_build_cov<<<n, build_cov_threads(nfit), smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64,
+    k_build_cov<<<n, build_cov_threads(nfit, n, n_sm), smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64,
                                                           A32, rho, status);
 }
 

@@ -319,3 +319,28 @@ def test_systematic_factor_forms(ctx, nf, P):
         got = fc.fc_fake_data(ctx, gid, ps, 5, 2, nf, fluct)
         assert np.array_equal(got, oracle.fake_data(S, F, ps, 5, 2, None, nf, fluct))
     fc.fc_unload_grid(ctx, gid)
+
+
+# ---- covariances: 256 and 512 threads ---------------------------------------------------------
+
+@pytest.mark.parametrize("n", [1, 2, 40, 112, 113])
+def test_covariance_thread_counts(ctx, n):
+    """A covariance has the same bits alone (512 threads) and among many (256 up to N = 112)."""
+    S, F = _grid(1000, n, n)
+    gid = fc.fc_load_grid(ctx, S)
+    ps = np.arange(len(S), dtype=np.int64)
+    many, alone = [], []
+    fc.fc_set_frac_cov(ctx, gid, F)
+    fc.fc_run_points(ctx, gid, ps, 1, 1, opts=dict(cov=fc.FC_COV_FIXED))
+    for q in (0, 500, 999):
+        many.append(fc.fc_covariance(ctx, gid, q, n, n, want_L=False)[0])
+    fc.fc_set_frac_cov(ctx, gid, F)
+    for q in (0, 500, 999):
+        alone.append(fc.fc_covariance(ctx, gid, q, n, n, want_L=False)[0])
+    for q, a, b in zip((0, 500, 999), many, alone):
+        assert np.array_equal(a, b)
+        M = S[q][:, None] * F * S[q][None, :] + np.diag(S[q])
+        # n multiply-adds a factor, inverse and product element, scaled by the condition number
+        tol = 3 * n * 2.0 ** -52 * np.linalg.cond(M) * np.abs(np.linalg.inv(M)).max()
+        np.testing.assert_allclose(a, np.linalg.inv(M), rtol=0, atol=tol)
+    fc.fc_unload_grid(ctx, gid)
