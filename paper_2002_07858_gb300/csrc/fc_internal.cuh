@@ -158,7 +158,6 @@ void launch_fake_data(const float* L32, const float* s32, int nf, const int32_t*
 
 // ---- scan bookkeeping ----
 void launch_fill_i32(int32_t* p, int64_t n, int32_t v, cudaStream_t st);
-void launch_iota_i32(int32_t* p, int64_t n, cudaStream_t st);
 void launch_mark_used(const int32_t* active, int64_t n_active, const int32_t* cur, uint8_t* flag, cudaStream_t st);
 void launch_compact_flags(uint8_t* flag, int64_t G, int32_t* list, int32_t* count, cudaStream_t st);
 void launch_lookup_slots(const int32_t* active, int64_t n_active, const int32_t* cur, const int32_t* slot_of,

@@ -1145,11 +1145,6 @@ __global__ void k_fill_i32(int32_t* p, int64_t n, int32_t v) {
         p[i] = v;
 }
 
-__global__ void k_iota_i32(int32_t* p, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = (int32_t)i;
-}
-
 __global__ void k_mark_used(const int32_t* __restrict__ active, int64_t n, const int32_t* __restrict__ cur,
                             uint8_t* __restrict__ flag) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -2666,8 +2661,9 @@ void launch_build_cov(const FullSrc& src, int nf, int nfit, const int32_t* coll,
     count_launch();
     const size_t smem = build_cov_smem(nfit);
     allow_smem(k_build_cov, smem, build_cov_smem(kMaxBins));
-    k_build_cov<<<n, build_cov_threads(nfit, n, n_sm), smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64,
-                                                          A32, rho, status);
+    const int threads = build_cov_threads(nfit, n, n_sm);
+    k_build_cov<<<n, threads, smem, st>>>(src, nf, nfit, coll, F, q_list, slot_list, cov_mode, A64, W64, A32, rho,
+                                          status);
 }
 
 void launch_qvec64(const GridSpec& gs, int64_t G, int nfit, const double* W64, const int32_t* slots, int n,
@@ -2732,14 +2728,6 @@ void launch_fill_i32(int32_t* p, int64_t n, int32_t v, cudaStream_t st) {
     if (b > 4096) b = 4096;
     count_launch();
     k_fill_i32<<<b, kThreads, 0, st>>>(p, n, v);
-}
-
-void launch_iota_i32(int32_t* p, int64_t n, cudaStream_t st) {
-    if (n <= 0) return;
-    unsigned b = blocks_for(n);
-    if (b > 4096) b = 4096;
-    count_launch();
-    k_iota_i32<<<b, kThreads, 0, st>>>(p, n);
 }
 
 void launch_mark_used(const int32_t* active, int64_t n, const int32_t* cur, uint8_t* flag, cudaStream_t st) {
