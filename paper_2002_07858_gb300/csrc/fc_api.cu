@@ -2358,7 +2358,7 @@ fc_status fc_fc_region(fc_ctx* c, const double* dchi2_univ, int32_t P, int32_t U
     FC_TRY(scratch(c, "qout", (size_t)P, &dout));
     FC_TRY(quantile_input(c, dchi2_univ, (size_t)P * U, &dx));
     FC_CUDA(cudaMemcpyAsync(dp, &cl, 8, cudaMemcpyHostToDevice, c->stream));
-    launch_quantiles(dx, P, U, dp, 1, dout, c->stream);
+    launch_quantiles(dx, P, U, dp, 1, dout, c->n_sm, c->stream);
     std::vector<double> hc(P), hd(P);
     FC_CUDA(cudaMemcpyAsync(hc.data(), dout, (size_t)P * 8, cudaMemcpyDeviceToHost, c->stream));
     FC_TRY(sync(c));
@@ -2479,7 +2479,7 @@ fc_status fc_quantiles(fc_ctx* c, const double* x, int32_t rows, int32_t n, cons
     FC_TRY(scratch(c, "qout", (size_t)rows * nq, &dout));
     FC_TRY(quantile_input(c, x, (size_t)rows * n, &dx));
     FC_CUDA(cudaMemcpyAsync(dp, hp.data(), (size_t)nq * 8, cudaMemcpyHostToDevice, c->stream));
-    launch_quantiles(dx, rows, n, dp, nq, dout, c->stream);
+    launch_quantiles(dx, rows, n, dp, nq, dout, c->n_sm, c->stream);
     FC_TRY(copy_out(c, out, dout, (size_t)rows * nq * 8));
     return sync(c);
 }

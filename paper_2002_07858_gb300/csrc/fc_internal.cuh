@@ -350,7 +350,8 @@ void launch_advance(const int32_t* active, int64_t n_active, const int32_t* best
 bool measure_fma_peaks(int n_sm, double* fp64_tflops, double* fp32_tflops, cudaStream_t st);
 
 // ---- quantiles ----
-void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, cudaStream_t st);
+void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, int n_sm,
+                      cudaStream_t st);
 // The shape model's sine table (m.sinT, rows rows of m.nf), from the bins' L and E.
 void launch_osc_sin(const SpecModel& m, int rows, const double* L, const double* E, double* sinT, cudaStream_t st);
 // Full-bin spectra of the model into S [G][nf] (S null: only checked); bad counts

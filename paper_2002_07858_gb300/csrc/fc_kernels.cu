@@ -2398,7 +2398,10 @@ __device__ void quantiles_by_sort(unsigned long long* key, int n, int npow2, con
 // count finds the buckets that hold each quantile's two ranks, the values of
 // those buckets go to a short list, and their ranks in it are counted.  Rows
 // that this does not suit (a crowded bucket, infinities, NaN) and calls with
-// many quantiles sort the row.  Bound by shared memory (three passes over the
+// many quantiles sort the row; so do rows whose lists are long enough that
+// counting ranks, a list's square, takes longer than the sort's steps (a call of
+// 10000 rows of 100 values, 63 of them in one bucket: lists 82, 96 and 160 us
+// for 1, 3 and 8 quantiles, a sort 98; 99 in one: 99, 172 and 375).  Bound by shared memory (three passes over the
 // row and its counting atomics).  10000 rows of 1000 values, three quantiles:
 // 1.04 -> 0.13 ms a call (the sort compared on the binary64 pipe and its rows
 // were copied first).
@@ -2413,7 +2416,7 @@ __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, cons
     __shared__ int s_bin[BINS];
     __shared__ int s_warp[16];
     __shared__ float s_lo[16], s_hi[16];
-    __shared__ int s_b0[kQuantSelect], s_b1[kQuantSelect], s_before[kQuantSelect], s_n[kQuantSelect];
+    __shared__ int s_b0[kQuantSelect], s_b1[kQuantSelect], s_before[kQuantSelect], s_len[kQuantSelect], s_n[kQuantSelect];
     __shared__ double s_v[kQuantSelect][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const unsigned long long* xr = reinterpret_cast<const unsigned long long*>(x) + (size_t)blockIdx.x * n;
@@ -2492,8 +2495,18 @@ __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, cons
         s_b0[threadIdx.x] = b0;
         s_b1[threadIdx.x] = b1;
         s_before[threadIdx.x] = b0 ? s_bin[b0 - 1] : 0;
+        s_len[threadIdx.x] = s_bin[b1] - s_before[threadIdx.x];
     }
     __syncthreads();
+    int most = 0;  // the longest list
+    for (int q = 0; q < nq; ++q) most = max(most, s_len[q]);
+    // trips of a warp in all: of the rank loop, and of the sort's steps, each worth three of those
+    const int lg = 31 - __clz(npow2), sort_work = 3 * lg * (lg + 1) / 2 * ((npow2 + 31) / 32);
+    const int rank_work = nq * most * ((most + 31) / 32);
+    if (most > kQuantList || rank_work > sort_work) {  // the same for every thread
+        quantiles_by_sort(s_key, n, npow2, probs, nq, o);
+        return;
+    }
     // the values of those buckets (the buckets between them are empty)
     unsigned long long* list = s_key + npow2;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
@@ -2506,19 +2519,13 @@ __global__ void k_quantiles(const double* __restrict__ x, int n, int npow2, cons
             }
     }
     __syncthreads();
-    bool crowded = false;
-    for (int q = 0; q < nq; ++q) crowded = crowded || s_n[q] > kQuantList;
-    if (crowded) {  // the same for every thread
-        quantiles_by_sort(s_key, n, npow2, probs, nq, o);
-        return;
-    }
     for (int q = warp; q < nq; q += nw) {
         int r0, r1;
         double f;
         quantile_ranks(n, probs[q], r0, r1, f);
         r0 -= s_before[q];
         r1 -= s_before[q];
-        const int m = s_n[q];
+        const int m = s_len[q];
         const unsigned long long* l = list + q * kQuantList;
         for (int e = lane; e < m; e += 32) {
             const unsigned long long k = l[e];
@@ -2966,7 +2973,8 @@ void launch_osc_spectra(const SpecModel& m, int64_t G, double* S, int* bad, cuda
     k_osc_spectra<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(m, G, S, bad);
 }
 
-void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, cudaStream_t st) {
+void launch_quantiles(const double* x, int rows, int n, const double* probs, int nq, double* out, int n_sm,
+                      cudaStream_t st) {
     int p2 = 1;
     while (p2 < n) p2 <<= 1;
     const auto smem_of = [](size_t keys, int lists) {
@@ -2975,8 +2983,10 @@ void launch_quantiles(const double* x, int rows, int n, const double* probs, int
     const size_t smem = smem_of(p2, nq <= kQuantSelect ? nq : 0);
     count_launch();
     // short rows: small CTAs, many rows in flight; long rows (and a sort of many quantiles) a wide CTA,
-    // with as many buckets as keep a bucket of a smooth distribution below the list's length
-    const bool small = n <= 2048 && nq <= kQuantSelect;
+    // with as many buckets as keep a bucket of a smooth distribution below the list's length.  A row an SM
+    // at most gets the wide one too: 10 rows of 1000 values that have to be sorted 61 us a call with 128
+    // threads, 46 with 512 (rows that select 34 either way)
+    const bool small = n <= 2048 && nq <= kQuantSelect && rows > n_sm;
     auto kern = small ? k_quantiles<1024> : k_quantiles<4096>;
     allow_smem(kern, smem, smem_of(small ? 2048 : kQuantMaxRow, kQuantSelect));
     kern<<<rows, small ? 128 : 512, smem, st>>>(x, n, p2, probs, nq, out);

@@ -344,3 +344,21 @@ def test_covariance_thread_counts(ctx, n):
         tol = 3 * n * 2.0 ** -52 * np.linalg.cond(M) * np.abs(np.linalg.inv(M)).max()
         np.testing.assert_allclose(a, np.linalg.inv(M), rtol=0, atol=tol)
     fc.fc_unload_grid(ctx, gid)
+
+
+@pytest.mark.parametrize("kind", ["chi2", "ties", "equal", "outlier", "inf"])
+@pytest.mark.parametrize("n", [1, 2, 33, 100, 129, 1000, 2048])
+@pytest.mark.parametrize("nq", [1, 8])
+def test_quantiles_of_many_rows(ctx, kind, n, nq):
+    """More rows than SMs (the small CTA): every row as alone (the wide one)."""
+    x = _quantile_rows(kind, 200, n, np.random.default_rng(n + nq))
+    probs = np.linspace(0.03, 1.0, nq)
+    got = fc.fc_quantiles(ctx, x, probs)
+    for r in (0, 1, 77, 199):
+        assert np.array_equal(got[r:r + 1], fc.fc_quantiles(ctx, x[r:r + 1], probs), equal_nan=True)
+    with np.errstate(invalid="ignore"):
+        s, h = np.sort(x, axis=1), (n - 1) * probs
+        lo = np.floor(h).astype(int)
+        a, b = s[:, lo], s[:, np.minimum(lo + 1, n - 1)]
+        want = a + (h - lo) * (b - a)
+    np.testing.assert_allclose(got, want, rtol=0, atol=1.2e-15 * np.max(np.abs(x), where=np.isfinite(x), initial=0.0))
