@@ -1021,7 +1021,7 @@ fc_status lane_admit(fc_ctx* c, Lane* L, const std::shared_ptr<LaneJob>& J, cons
         // with the first count it reads
         if (J->jr) FC_TRY(read_ctrl(c));
         launch_fake_data(L32, s32, g->nf, g->identity_collapse ? nullptr : g->collapse, g->nfit, ps_dev, P, U, seed,
-                         fluct == FC_FLUCT_GAUSS, dst, c->stream);
+                         fluct == FC_FLUCT_GAUSS, dst, c->n_sm, c->stream);
     }
     count_launch();
     k_lane_admit<<<nb(n), 256, 0, c->stream>>>(ps_dev, n, U, J->base, (int8_t)max_iter, J->slot, L->cur, L->pt,
@@ -1701,7 +1701,7 @@ fc_status fake_data_impl(fc_ctx* c, int32_t grid_id, const int64_t* ps, int32_t 
         FC_TRY(scratch(c, "d", (size_t)n * g->nfit, &d));
     }
     launch_fake_data(L32, s32, g->nf, g->identity_collapse ? nullptr : g->collapse, g->nfit, ps_dev, P, U, seed,
-                     fluct == FC_FLUCT_GAUSS, d, c->stream);
+                     fluct == FC_FLUCT_GAUSS, d, c->n_sm, c->stream);
     if (d != out) FC_TRY(copy_out(c, out, d, (size_t)n * g->nfit * sizeof(float)));
     return sync(c);
 }

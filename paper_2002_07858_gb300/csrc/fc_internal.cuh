@@ -154,7 +154,7 @@ bool launch_qvec_tc(const uint16_t* Bt, const uint16_t* Wimg, const float4* wnor
 
 // ---- fake data (a3) ----
 void launch_fake_data(const float* L32, const float* s32, int nf, const int32_t* collapse, int nfit,
-                      const int64_t* ps, int P, int U, uint64_t seed, int gauss, float* d, cudaStream_t st);
+                      const int64_t* ps, int P, int U, uint64_t seed, int gauss, float* d, int n_sm, cudaStream_t st);
 
 // ---- scan bookkeeping ----
 void launch_fill_i32(int32_t* p, int64_t n, int32_t v, cudaStream_t st);

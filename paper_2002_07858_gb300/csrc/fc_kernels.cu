@@ -958,23 +958,37 @@ __global__ void k_qvec32_generic(GridSpec gs, const float4* __restrict__ gnorm, 
 //  - normals: one thread per (block of four, universe);
 //  - lam: a warp per eight rows of L, two universes per lane, so each L_ij (one
 //    broadcast) and z_j feed 16 multiply-adds;
-//  - counts: one thread per (bin, universe), first only the quick acceptance of
-//    the rejection sampler's first trial (about seven draws of ten); the others
-//    are queued and tested by full warps, trial by trial, instead of by the few
-//    lanes of every warp that need the logarithms;
-//  - fit bins: four threads per universe, each a quarter of the fit bins.
+//  - counts: one thread per (bin, universe): lam below ten by inversion, else
+//    only the quick acceptance of the rejection sampler's first trial (about
+//    seven draws of ten); the others are queued and tested by full warps, trial
+//    by trial, instead of by the few lanes of every warp that need the
+//    logarithms;
+//  - fit bins: two or four threads per universe, each its part of the fit bins.
 // One thread per universe did all of it with 16 of 32 lanes active: 500 points
-// x 1000 universes of 90 bins 1.50 -> 1.00 ms, the full 100x100 job's draw
-// 26.7 -> 19.4 ms, one point x 1000 universes of 40 bins 100 -> 20 us.
+// x 1000 universes of 90 bins 1.56 -> 0.95 ms, of 16 bins 236 -> 168 us, one
+// point x 1000 universes of 40 bins 100 -> 25 us.
 constexpr int kFakeU = 64;        // universes of a CTA
-constexpr int kFakeThreads = 256;
 constexpr int kFakeLd = kFakeU + 2;
 constexpr int kFakeRows = 8;      // rows of L per warp
 constexpr int kFakePasses = 3;    // trials tested by full warps
+constexpr int kFakeFewBins = 8;   // bins a thread can hold by itself
 
+// A thread per universe (k_fake_few) from there on: with few bins a CTA's phases are shorter than its barriers.
+// Measured, us, a thread / a CTA of 64 universes: 500 points x 1000 universes of 1 bin 25 / 46, of 5 bins 79 / 78
+// (85 / 102 with counts below ten), of 8 bins 115 / 101 (110 / 123); 1216 points x 64 of 5 bins 20.8 / 15.8, of
+// 1 bin 9.1 / 11.1.  From nine bins on the CTA is the faster but for counts below ten in 1500 CTAs and more
+// (9 bins 130 / 134, 12 bins 154 / 152).
+inline bool fake_few(int nf, int64_t ctas, int n_sm) {
+    return nf <= 2 || (nf <= kFakeFewBins && ctas > 8 * (int64_t)n_sm);
+}
+// 128 threads a CTA, eight an SM, when there are more CTAs than four an SM (256 threads) take at once and
+// eight fit in shared memory (N_full = 52): 500 x 1000 of 16 bins 218 -> 185 us, of 48 bins 502 -> 468; 310 x 64
+// of 24 bins, one round either way, 22.6 with 256 and 28.0 with 128.
+inline int fake_threads(int nf, int64_t ctas, int n_sm) { return nf <= 52 && ctas > 4 * (int64_t)n_sm ? 128 : 256; }
 inline size_t fake_smem(int nf) { return (size_t)(2 * nf + 3) * kFakeLd * sizeof(float); }
 
-__global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __restrict__ L32,
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_fake_data(const float* __restrict__ L32,
                                                                const float* __restrict__ s32, int nf,
                                                                const int32_t* __restrict__ coll, int nfit,
                                                                const int64_t* __restrict__ ps, int U, uint32_t k0,
@@ -992,7 +1006,7 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
     const float* L = L32 + (size_t)ip * nf * nf;
     const float* s = s32 + (size_t)ip * nf;
     if (tid < kFakePasses) s_queued[tid] = 0;
-    for (int e = tid; e < (nf + 3) / 4 * kFakeU; e += kFakeThreads) {
+    for (int e = tid; e < (nf + 3) / 4 * kFakeU; e += THREADS) {
         const int j = e / kFakeU, u = e % kFakeU;
         float zz[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         if (u < nu) normal_block((uint32_t)j, (uint32_t)(u0 + u), p, k0, k1, zz);
@@ -1002,7 +1016,7 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
     __syncthreads();
     // the row blocks, longest first, dealt to the warps back and forth
     const int nb = (nf + kFakeRows - 1) / kFakeRows;
-    constexpr int kWarps = kFakeThreads / 32;
+    constexpr int kWarps = THREADS / 32;
     for (int pass = 0; pass * kWarps < nb; ++pass) {
         const int b = nb - 1 - (pass * kWarps + ((pass & 1) ? kWarps - 1 - warp : warp));
         if (b < 0) continue;
@@ -1051,21 +1065,26 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
             if (mine) to[at + __popc(m & ((1u << lane) - 1u))] = (uint16_t)e;
         };
         // kFakeU is a multiple of the warp: a warp's lanes share the bin and are in the loop together
-        for (int e = tid; e < nf * kFakeU; e += kFakeThreads) {
+        for (int e = tid; e < nf * kFakeU; e += THREADS) {
             const int i = e / kFakeU, u = e % kFakeU;
             const float l = lam[i * kFakeLd + u];
             bool wait = u < nu && l > 0.0f;  // lam = 0: the count is 0
-            if (wait && l >= 10.0f) {
+            if (wait) {
                 BinUniforms un;
                 un.init(k0, k1, (uint32_t)(u0 + u), p, (uint32_t)i);
-                Ptrs t;
-                t.init(l);
                 float ua, ub;
                 un.pair(0, ua, ub);
-                if (t.propose(ua, ub)) {
-                    lam[i * kFakeLd + u] = (float)(int32_t)t.kf;
+                int32_t k = 0;
+                if (l < 10.0f) {  // a bin of few counts has few in most universes: the warp is full as it is
+                    k = poisson_inversion(l, ua);
                     wait = false;
+                } else {
+                    Ptrs t;
+                    t.init(l);
+                    wait = !t.propose(ua, ub);
+                    k = (int32_t)t.kf;
                 }
+                if (!wait) lam[i * kFakeLd + u] = (float)k;
             }
             push(queue, &s_queued[0], wait, e);
         }
@@ -1075,9 +1094,10 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
         uint16_t* from = queue;
         for (int t = 0; t < kFakePasses; ++t) {
             const int n = s_queued[t];
+            if (n == 0) break;  // the same for every thread
             uint16_t* to = (t & 1) ? queue : queue + nf * kFakeU;
             const bool last = t + 1 == kFakePasses;
-            for (int q0 = 0; q0 < n; q0 += kFakeThreads) {  // the same trip count for every thread
+            for (int q0 = 0; q0 < n; q0 += THREADS) {  // the same trip count for every thread
                 const bool have = q0 + tid < n;
                 bool again = false;
                 int e = 0;
@@ -1089,31 +1109,25 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
                     un.init(k0, k1, (uint32_t)(u0 + u), p, (uint32_t)i);
                     float ua, ub;
                     un.pair(t, ua, ub);
-                    int32_t k = 0;
-                    if (l < 10.0f) {
-                        k = poisson_inversion(l, ua);
-                    } else {
-                        Ptrs tr;
-                        tr.init(l);
-                        tr.propose(ua, ub);
-                        const float loglam = ln32(l);
-                        again = !tr.accept(loglam);
-                        if (again) {
-                            un.pair(t + 1, ua, ub);
-                            again = !tr.propose(ua, ub);
-                        }
-                        if (again && last) {
-                            int it = t + 1;
-                            while (!tr.accept(loglam) && ++it < kPtrsTrials) {
-                                un.pair(it, ua, ub);
-                                if (tr.propose(ua, ub)) break;
-                            }
-                            if (it >= kPtrsTrials) tr.kf = floorf(l);
-                            again = false;
-                        }
-                        k = (int32_t)tr.kf;
+                    Ptrs tr;
+                    tr.init(l);
+                    tr.propose(ua, ub);
+                    const float loglam = ln32(l);
+                    again = !tr.accept(loglam);
+                    if (again) {
+                        un.pair(t + 1, ua, ub);
+                        again = !tr.propose(ua, ub);
                     }
-                    if (!again) lam[i * kFakeLd + u] = (float)k;
+                    if (again && last) {
+                        int it = t + 1;
+                        while (!tr.accept(loglam) && ++it < kPtrsTrials) {
+                            un.pair(it, ua, ub);
+                            if (tr.propose(ua, ub)) break;
+                        }
+                        if (it >= kPtrsTrials) tr.kf = floorf(l);
+                        again = false;
+                    }
+                    if (!again) lam[i * kFakeLd + u] = (float)(int32_t)tr.kf;
                 }
                 if (!last) push(to, &s_queued[t + 1], again, e);
             }
@@ -1124,18 +1138,80 @@ __global__ void __launch_bounds__(kFakeThreads, 4) k_fake_data(const float* __re
     const float* out = lam;
     if (coll) {
         out = z;
-        for (int e = tid; e < nfit * kFakeLd; e += kFakeThreads) z[e] = 0.0f;
+        for (int e = tid; e < nfit * kFakeLd; e += THREADS) z[e] = 0.0f;
         __syncthreads();
-        const int u = tid % kFakeU, part = tid / kFakeU;  // fit bins part, part + 4, ... of universe u
+        constexpr int kParts = THREADS / kFakeU;
+        const int u = tid % kFakeU, part = tid / kFakeU;  // fit bins part, part + kParts, ... of universe u
         for (int i = 0; i < nf; ++i) {
             const int jf = __ldg(coll + i);
-            if ((jf & 3) == part) z[jf * kFakeLd + u] = __fadd_rn(z[jf * kFakeLd + u], lam[i * kFakeLd + u]);
+            if (jf % kParts == part) z[jf * kFakeLd + u] = __fadd_rn(z[jf * kFakeLd + u], lam[i * kFakeLd + u]);
         }
         __syncthreads();
     }
     float* o = d + ((size_t)ip * U + u0) * nfit;
-    for (int u = warp; u < nu; u += kWarps)
-        for (int j = lane; j < nfit; j += 32) o[(size_t)u * nfit + j] = out[j * kFakeLd + u];
+    if (nfit < 32) {  // several universes a warp
+        for (int e = tid; e < nu * nfit; e += THREADS) o[e] = out[e % nfit * kFakeLd + e / nfit];
+    } else {
+        for (int u = warp; u < nu; u += kWarps)
+            for (int j = lane; j < nfit; j += 32) o[(size_t)u * nfit + j] = out[j * kFakeLd + u];
+    }
+}
+
+// The same for at most kFakeFewBins bins: one thread per universe, everything
+// in registers.
+__global__ void __launch_bounds__(128) k_fake_few(const float* __restrict__ L32, const float* __restrict__ s32, int nf,
+                                                  const int32_t* __restrict__ coll, int nfit,
+                                                  const int64_t* __restrict__ ps, int U, uint32_t k0, uint32_t k1,
+                                                  int gauss, float* __restrict__ d) {
+    const int ip = blockIdx.y;
+    const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    if (u >= U) return;
+    const uint32_t p = (uint32_t)ps[ip];
+    const float* L = L32 + (size_t)ip * nf * nf;
+    const float* s = s32 + (size_t)ip * nf;
+    float z[kFakeFewBins], v[kFakeFewBins];
+#pragma unroll
+    for (int j = 0; j < kFakeFewBins; j += 4) {
+        float zz[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (j < nf) normal_block((uint32_t)(j / 4), (uint32_t)u, p, k0, k1, zz);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) z[j + h] = zz[h];
+    }
+#pragma unroll
+    for (int r = 0; r < kFakeFewBins; ++r) {
+        v[r] = 0.0f;
+        if (r >= nf) continue;
+        float acc = 0.0f;
+#pragma unroll
+        for (int j = 0; j <= r; ++j) acc = __fmaf_rn(__ldg(L + r * nf + j), z[j], acc);
+        v[r] = __fadd_rn(__ldg(s + r), acc);
+    }
+    if (!gauss) {
+        // not unrolled: the draw's code once, with the bins shifted through v
+#pragma unroll 1
+        for (int r = 0; r < nf; ++r) {
+            BinUniforms un;
+            un.init(k0, k1, (uint32_t)u, p, (uint32_t)r);
+            const float n = (float)poisson(v[0], un);
+#pragma unroll
+            for (int k = 0; k + 1 < kFakeFewBins; ++k) v[k] = v[k + 1];
+            v[kFakeFewBins - 1] = n;
+        }
+        // bin r is at kFakeFewBins - nf + r now
+#pragma unroll 1
+        for (int r = nf; r < kFakeFewBins; ++r) {
+#pragma unroll
+            for (int k = 0; k + 1 < kFakeFewBins; ++k) v[k] = v[k + 1];
+        }
+    }
+    float* o = d + ((size_t)ip * U + u) * nfit;
+    for (int j = 0; j < nfit; ++j) {
+        float sum = 0.0f;
+#pragma unroll
+        for (int r = 0; r < kFakeFewBins; ++r)
+            if (r < nf && (coll ? __ldg(coll + r) : r) == j) sum = coll ? __fadd_rn(sum, v[r]) : v[r];
+        o[j] = sum;
+    }
 }
 
 // ------------------------------------------------------- bookkeeping -------
@@ -2713,19 +2789,23 @@ void launch_qvec32(const GridSpec& gs, const float4* gnorm, int64_t G, int64_t G
 }
 
 void launch_fake_data(const float* L32, const float* s32, int nf, const int32_t* coll, int nfit, const int64_t* ps,
-                      int P, int U, uint64_t seed, int gauss, float* d, cudaStream_t st) {
+                      int P, int U, uint64_t seed, int gauss, float* d, int n_sm, cudaStream_t st) {
     if (P <= 0 || U <= 0) return;
     // blockIdx.y is the point within a launch; more points than gridDim.y allows take several launches
     constexpr int kMaxGridY = 65535;
+    const int64_t ctas = (int64_t)P * ((U + kFakeU - 1) / kFakeU);
+    const bool few = fake_few(nf, ctas, n_sm);
+    const int threads = few ? std::min(128, (U + 31) / 32 * 32) : fake_threads(nf, ctas, n_sm);
+    const int per = few ? threads : kFakeU;
+    const size_t smem = few ? 0 : fake_smem(nf);
+    auto kern = few ? k_fake_few : threads == 128 ? k_fake_data<128> : k_fake_data<256>;
+    allow_smem(kern, smem, fake_smem(kMaxBins));
     for (int p0 = 0; p0 < P; p0 += kMaxGridY) {
         const int np = P - p0 < kMaxGridY ? P - p0 : kMaxGridY;
-        dim3 grid((U + kFakeU - 1) / kFakeU, np);
-        const size_t smem = fake_smem(nf);
-        allow_smem(k_fake_data, smem, fake_smem(kMaxBins));
+        const dim3 grid((U + per - 1) / per, np);
         count_launch();
-        k_fake_data<<<grid, kFakeThreads, smem, st>>>(L32 + (size_t)p0 * nf * nf, s32 + (size_t)p0 * nf, nf, coll, nfit, ps + p0,
-                                           U, (uint32_t)seed, (uint32_t)(seed >> 32), gauss,
-                                           d + (size_t)p0 * U * nfit);
+        kern<<<grid, threads, smem, st>>>(L32 + (size_t)p0 * nf * nf, s32 + (size_t)p0 * nf, nf, coll, nfit, ps + p0, U,
+                                          (uint32_t)seed, (uint32_t)(seed >> 32), gauss, d + (size_t)p0 * U * nfit);
     }
 }
 

@@ -136,7 +136,8 @@ fc_status fc_fake_data_noalloc(const double* S, int64_t G, int32_t N_full, const
     fcdev::launch_chol_sys(fcdev::FullSrc{S, {}}, N_full, F, ps, P, fluct == FC_FLUCT_GAUSS, L64, L32, s32, n_sm,
                            status, st);
     if (!launched()) return FC_ERR_CUDA;
-    fcdev::launch_fake_data(L32, s32, N_full, collapse, N_fit, ps, P, U, seed, fluct == FC_FLUCT_GAUSS, d, st);
+    fcdev::launch_fake_data(L32, s32, N_full, collapse, N_fit, ps, P, U, seed, fluct == FC_FLUCT_GAUSS, d,
+                             n_sm, st);
     if (!launched()) return FC_ERR_CUDA;
     if (!read_status(&h)) return noalloc_fail(FC_ERR_CUDA, cudaGetErrorString(cudaGetLastError()));
     if (h & fcdev::kDevNotSpd) return noalloc_fail(FC_ERR_NOT_SPD, "systematic covariance not positive definite");

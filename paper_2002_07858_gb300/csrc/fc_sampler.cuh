@@ -249,4 +249,24 @@ struct Ptrs {
     }
 };
 
+// Poisson(lam) by one thread
+__device__ __forceinline__ int32_t poisson(float lam, BinUniforms& un) {
+    if (!(lam > 0.0f)) return 0;
+    float ua, ub;
+    un.pair(0, ua, ub);
+    if (lam < 10.0f) return poisson_inversion(lam, ua);
+    Ptrs t;
+    t.init(lam);
+    if (!t.propose(ua, ub)) {
+        const float loglam = ln32(lam);
+        int it = 0;
+        while (!t.accept(loglam)) {
+            if (++it == kPtrsTrials) return (int32_t)floorf(lam);
+            un.pair(it, ua, ub);
+            if (t.propose(ua, ub)) break;
+        }
+    }
+    return (int32_t)t.kf;
+}
+
 }  // namespace fcdev

@@ -362,3 +362,27 @@ def test_quantiles_of_many_rows(ctx, kind, n, nq):
         a, b = s[:, lo], s[:, np.minimum(lo + 1, n - 1)]
         want = a + (h - lo) * (b - a)
     np.testing.assert_allclose(got, want, rtol=0, atol=1.2e-15 * np.max(np.abs(x), where=np.isfinite(x), initial=0.0))
+
+
+# ---- fake data: a thread, or a CTA of 128 or 256 threads, per 64 universes --------------------
+
+@pytest.mark.parametrize("nf", [1, 2, 3, 4, 7, 8, 9, 16, 31, 52, 53])
+@pytest.mark.parametrize("P,U", [(3, 1), (3, 33), (700, 2), (1300, 1), (1300, 65), (20, 4000)])
+def test_fake_data_forms(ctx, nf, P, U):
+    """Both sides of every line, with and without a collapse, in both modes: the oracle's bits for some of the
+    points, and the same bits for a point alone."""
+    import oracle
+
+    S, F = _grid(1300, nf, nf + 2)
+    S = S * np.logspace(-2.5, 0.5, nf)[None, ::-1]
+    coll = workloads.pair_collapse(nf)
+    ps = np.arange(P, dtype=np.int64)
+    some = [0, P // 2, P - 1]
+    for c, n_fit in ((None, nf), (coll, (nf + 1) // 2)):
+        gid = fc.fc_load_grid(ctx, S, c, n_fit)
+        fc.fc_set_frac_cov(ctx, gid, F)
+        for fluct in (fc.FC_FLUCT_POISSON_SYS, fc.FC_FLUCT_GAUSS):
+            got = fc.fc_fake_data(ctx, gid, ps, 23, U, n_fit, fluct)
+            assert np.array_equal(got[some], oracle.fake_data(S, F, ps[some], 23, U, c, n_fit, fluct))
+            assert np.array_equal(got[P - 1:], fc.fc_fake_data(ctx, gid, ps[P - 1:], 23, U, n_fit, fluct))
+        fc.fc_unload_grid(ctx, gid)
