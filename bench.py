@@ -37,8 +37,8 @@ UNIT = "chi2 evals/s"
 
 # DRAM bytes (read + write) per screened universe row of the tensor-core screen on the
 # 100x100 grid with N 90->45 (K = 48): an ncu capture of one top-8 launch over 10^6
-# universes (the current kernel, parallel top-k insertion) read 367.0 MB and wrote
-# 56.3 MB.  The traffic is the rows' A images, the q-step rows of their covariance
+# universes (three copy producers, parallel top-k insertion) read 367.6 MB and wrote
+# 55.7 MB.  The traffic is the rows' A images, the q-step rows of their covariance
 # slots and the candidate lists, so a launch's traffic is taken as proportional to the
 # rows it screens.
 SCREEN_DRAM_BYTES_PER_ROW_CFG2 = 423.3

@@ -140,8 +140,8 @@ __device__ __forceinline__ double resid_df_reg(const ulonglong2* __restrict__ W,
 // residual k's t_i^2.  This is the form for few residuals, for covariances
 // with few residuals each and for N_fit > 64: a residual is spread over the
 // warp, W is read coalesced and once per group, and nothing lives in local
-// memory.  Bound by the binary32 pipe when there are enough groups, else by
-// the latency of one group.  Against one thread per residual everywhere: a
+// memory.  Bound by the binary32 pipe (63 % active at N = 120) when there are
+// enough groups, else by the latency of one group.  Against one thread per residual everywhere: a
 // scan of 4096 data sets on 141x141 1.15 -> 0.76 ms, one point of 25x25 x 1000
 // universes 2.59 -> 1.88 ms, 4 points of 27^3 with N = 200 61.3 -> 49.6 ms.
 constexpr int kRowsB = 4;       // residuals of a group
@@ -1140,11 +1140,11 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_fake_data(const flo
         out = z;
         for (int e = tid; e < nfit * kFakeLd; e += THREADS) z[e] = 0.0f;
         __syncthreads();
-        constexpr int kParts = THREADS / kFakeU;
+        constexpr int kParts = THREADS / kFakeU;  // a power of two
         const int u = tid % kFakeU, part = tid / kFakeU;  // fit bins part, part + kParts, ... of universe u
         for (int i = 0; i < nf; ++i) {
             const int jf = __ldg(coll + i);
-            if (jf % kParts == part) z[jf * kFakeLd + u] = __fadd_rn(z[jf * kFakeLd + u], lam[i * kFakeLd + u]);
+            if ((jf & (kParts - 1)) == part) z[jf * kFakeLd + u] = __fadd_rn(z[jf * kFakeLd + u], lam[i * kFakeLd + u]);
         }
         __syncthreads();
     }
@@ -1252,7 +1252,7 @@ __global__ void k_set_slots(const int32_t* __restrict__ q, const int32_t* __rest
 // ------------------------------------------------------ plain fp64 scan -----
 
 // Plain binary64 scan: chi2_g - c = q_g - 2 y.s~_g with y = A (d - v) for every
-// g, the first minimum in index order.  The y.s~ products of 32 universes x 64
+// g, the first minimum in index order.  The y.s~ products of 16 universes x 64
 // grid points are a small dense contraction on the FP64 pipe: y and a tile of
 // s~ (transposed to [j][g]) sit in shared memory and every thread keeps a 4 x 2
 // block of dot products in registers (the binary64 pipe is narrow, so operand
@@ -1805,8 +1805,9 @@ constexpr int kItemCodes = kMaxTopK + 3;
 // waited at barriers for the rows with many).
 //  k_resolve_emit     per row: the screen certificate (decide_row); the
 //                     residual items the row needs, appended in tile order;
-//  k_resid_tiles/rows every item's double-float residual chi2 (W of the row's
-//                     covariance slot; the residual vector in registers);
+//  k_resid_tiles/rows every item's double-float residual chi2 under the row's
+//                     covariance slot: a thread per item in well-filled tiles,
+//                     a warp per group of items else (launch_resolve);
 //  k_resolve_conclude per row: the same decision again, then the rescored
 //                     minimum and its certificate; finish (dchi2) / advance /
 //                     hand on, exactly as one kernel did before; rescored rows
@@ -1942,9 +1943,11 @@ __global__ void __launch_bounds__(kBM) k_resolve_emit(ResolveArgs a) {
 // (every lane reads the same element at once), and the lanes stride over the
 // run's items with no barrier but the staging's.  A tile whose quadrants share
 // one slot stages once.  Small CTAs (two warps) keep the last, partly filled
-// round of a run cheap.  Bound by issue: the packed multiply-add takes 14
-// instructions for two (24 unpacked) and one 16-byte broadcast of W instead of
-// two 8-byte ones; the full 100x100 job went from 178.1 to 171.1 ms with it.
+// round of a run cheap.  Bound by the binary32 pipe (52 % active at N = 45) and
+// the latency of ten warps an SM, all that 140 registers leave: the packed
+// multiply-add takes 14 instructions for two (24 unpacked) and one 16-byte
+// broadcast of W instead of two 8-byte ones; scan 1 of 1000 points x 1000
+// universes of N = 45 1.12 -> 0.88 ms, the full 100x100 job 178.1 -> 171.1.
 constexpr int kResidThreads = 64;
 
 template <int NR>
@@ -2477,10 +2480,11 @@ __device__ void quantiles_by_sort(unsigned long long* key, int n, int npow2, con
 // many quantiles sort the row; so do rows whose lists are long enough that
 // counting ranks, a list's square, takes longer than the sort's steps (a call of
 // 10000 rows of 100 values, 63 of them in one bucket: lists 82, 96 and 160 us
-// for 1, 3 and 8 quantiles, a sort 98; 99 in one: 99, 172 and 375).  Bound by shared memory (three passes over the
-// row and its counting atomics).  10000 rows of 1000 values, three quantiles:
-// 1.04 -> 0.13 ms a call (the sort compared on the binary64 pipe and its rows
-// were copied first).
+// for 1, 3 and 8 quantiles, a sort 98; 99 in one: 99, 172 and 375).  Bound by the
+// binary64 pipe (72 % active: three conversions of each value to binary32), then
+// by shared memory (61 %: three passes over the row and its counting atomics).
+// 10000 rows of 1000 values, three quantiles: 1.04 -> 0.12 ms a call (the sort
+// compared on the binary64 pipe and its rows were copied first).
 constexpr int kQuantSelect = 8;   // quantiles of a call that selects
 constexpr int kQuantList = 128;   // values of a quantile's list
 constexpr int kQuantMaxRow = 16384;  // values of a row (the entry points refuse longer ones)
